@@ -11,6 +11,7 @@
 // totals.  128-bit sums are kept as (lo, hi) words with explicit carries.
 // The doubles of Table 1 are derived on the host from these integers.
 #include <math.h>
+#include <string.h>
 
 #include <algorithm>
 
@@ -22,29 +23,37 @@ namespace {
 typedef unsigned long long u64;
 typedef unsigned __int128 u128;
 
-// Device accumulators; every field starts at 0.  Minima are kept as the
-// maximum of the bitwise complement so that 0 is the identity.
+// The pass's result: integer aggregates (min, max, sums; minima are kept as
+// the maximum of the bitwise complement so that 0 is the identity), in the
+// order of RowAgg's words.  Written by the last block straight into
+// page-locked host memory.  The 128-bit sums are carried as three digits of
+// 32, 32 and 64 bits, whose sums over blocks need no carries.
+constexpr int kFT = 256;        // threads per block of both kernels
+constexpr int kFeatBlocks = 3;  // their resident blocks per SM (80 registers)
+constexpr int64_t kLongRow = 1024;
+constexpr int64_t kPiece = 2048;
+constexpr int kFields = 18;
 struct FeatAcc {
     u64 nnz_min_c, nnz_max, nnz_sum, nnz_sumsq;
-    u64 bw_min_c, bw_max, bw_sum, bw_sq_lo, bw_sq_hi;
-    u64 disp_sum, disp_sq_lo, disp_sq_hi, clust_sum;
+    u64 bw_min_c, bw_max, bw_sum, disp_sum, clust_sum;
     u64 ngroups_sum, misses_sum;
     u64 err;
-    u64 n_long;  // rows of kShortCap < nnz <= kChunk (front of the list)
-    u64 n_huge;  // rows of nnz > kChunk (back of the list, chunked)
+    u64 bw_sq[3], disp_sq[3];
+};
+static_assert(sizeof(FeatAcc) == 8 * kFields, "one word per field");
+
+// Device counters and accumulators of one pass, all 0 between calls (the
+// last block resets them): long rows listed, their pieces listed, blocks of
+// either kernel finished, and kSlots sets of accumulators that the blocks
+// add to in turn, so that no address takes an atomic from every block.
+constexpr int kSlots = 32;
+struct FeatCtl {
+    unsigned n_long, n_pieces, done_pass, done_long;
+    u64 slot[kSlots][kFields];
 };
 
 __device__ __forceinline__ u64 shfl_u64(u64 v, int o) {
     return __shfl_xor_sync(FULL_MASK, v, o);
-}
-
-__device__ __forceinline__ void atomic_add_u128(u64* lo, u64* hi, u128 v) {
-    const u64 vlo = (u64)v, vhi = (u64)(v >> 64);
-    if (vlo) {
-        const u64 old = atomicAdd(lo, vlo);
-        if (old + vlo < old) atomicAdd(hi, 1ull);  // carry out of the low word
-    }
-    if (vhi) atomicAdd(hi, vhi);
 }
 
 __device__ __forceinline__ u128 warp_sum_u128(u128 v) {
@@ -62,87 +71,109 @@ __device__ __forceinline__ u64 warp_sum_u64(u64 v) {
     for (int o = 16; o > 0; o >>= 1) v += shfl_u64(v, o);
     return v;
 }
-__device__ __forceinline__ u64 warp_max_u64(u64 v) {
-    for (int o = 16; o > 0; o >>= 1) { u64 t = shfl_u64(v, o); v = t > v ? t : v; }
-    return v;
-}
 
-constexpr int kFields = 16;  // FeatAcc words reduced per block (err excluded)
-
-// floor(a 2^32 / b) for 0 <= a <= b < 2^31, exactly, without a 64-bit
-// integer division and without 64-bit conversions (which run on the FP64
-// pipe): an FP32 estimate of the quotient (a / b < 1, so it fits 32 bits),
-// then the integer remainder a 2^32 - q b, converted to FP32 from two 32-bit
-// halves, gives a correction, and the remainder is brought into [0, b).  The
-// first estimate is within about 2^9 of the quotient, so |remainder| < 2^41
-// and the second within one; the final steps run at most once (capped at
-// four).  Arguments outside that range come only from rows the pass flags as
-// invalid (columns not strictly increasing or out of range), whose results
-// are discarded: they give 0.
-__device__ __forceinline__ u64 fixq32(u64 a, u64 b)
+// floor(a 2^32 / b) for 0 < a < b < 2^31, exactly, without a 64-bit integer
+// division and without 64-bit conversions (which run on the FP64 pipe): an
+// FP32 estimate of the quotient (a / b < 1, so it fits 32 bits), then the
+// integer remainder a 2^32 - q b, converted to FP32 from two 32-bit halves,
+// gives a correction, and the remainder is brought into [0, b).  The
+// reciprocal and the three products are each off by at most 2 ulp, so the
+// first estimate is within 2^10 of the quotient, |remainder| < 2^42 and the
+// second within one; the final steps run at most once (capped at four).
+// Arguments outside that range come only from rows the pass flags as invalid
+// (columns not strictly increasing or out of range), whose results are
+// discarded: they give 0.
+__device__ __forceinline__ unsigned fixq32(unsigned a, unsigned b)
 {
-    if (a == 0 || b == 0 || b >= (1ull << 31) || a > b) return 0;
-    if (a == b) return 1ull << 32;
-    const unsigned a32 = (unsigned)a, b32 = (unsigned)b;
-    const float rb = __frcp_rn(__uint2float_rn(b32));
-    int64_t q = (int64_t)__float2uint_rz(__fmul_rn(__fmul_rn(__uint2float_rn(a32), rb), 4294967296.0f));
-    int64_t rem = (int64_t)(((u64)a32 << 32) - (u64)q * b32);
+    if (a == 0 || a >= b || b >= (1u << 31)) return 0;
+    const float rb = __fdividef(1.0f, __uint2float_rn(b));
+    unsigned q = __float2uint_rz(__fmul_rn(__fmul_rn(__uint2float_rn(a), rb), 4294967296.0f));
+    int64_t rem = (int64_t)(((u64)a << 32) - (u64)q * b);
     const float rf = __fmaf_rn(__int2float_rn((int)(rem >> 20)), 1048576.0f,
                                __uint2float_rn((unsigned)(rem & 0xFFFFF)));
     const int c = __float2int_rd(__fmul_rn(rf, rb));
-    q += c;
-    rem -= (int64_t)c * b32;
-    for (int i = 0; i < 4 && rem < 0; ++i) { --q; rem += b32; }
-    for (int i = 0; i < 4 && rem >= (int64_t)b32; ++i) { ++q; rem -= b32; }
-    return (u64)q;
+    q += (unsigned)c;
+    rem -= (int64_t)c * b;
+    for (int i = 0; i < 4 && rem < 0; ++i) { --q; rem += b; }
+    for (int i = 0; i < 4 && rem >= (int64_t)b; ++i) { ++q; rem -= b; }
+    return q;
 }
 
-// Per-thread partial aggregates of the rows a thread finalizes.
+// Per-thread partial aggregates of the rows a thread finalizes.  A ratio of
+// exactly 1 (2^32 in fixed point, one bit too wide) is counted apart, so that
+// every per-row quantity fits 32 bits and its square 64.
 struct RowAgg {
-    u64 nnz_min_c = 0, nnz_max = 0, nnz_sum = 0, nnz_sq = 0;
-    u64 bw_min_c = 0, bw_max = 0, bw_sum = 0, disp_sum = 0, clust_sum = 0, ng_sum = 0, ms_sum = 0;
+    unsigned nnz_min = 0xffffffffu, nnz_max = 0, bw_min = 0xffffffffu, bw_max = 0, disp_ones = 0, clust_ones = 0;
+    u64 nnz_sum = 0, nnz_sq = 0, bw_sum = 0, disp_sum = 0, clust_sum = 0, ng_sum = 0, ms_sum = 0;
     u128 bw_sq = 0, disp_sq = 0;
 
     // one row: nz nonzeros, columns first..last, ng / ms counted over its
     // elements after the first (the first element adds one to each)
-    __device__ __forceinline__ void add(u64 nz, int64_t first, int64_t last, u64 ng, u64 ms) {
-        u64 bw = 0, dq = 0, cq = 0;
+    __device__ __forceinline__ void add(unsigned nz, int first, int last, unsigned ng, unsigned ms) {
+        unsigned bw = 0, dq = 0, cq = 0;
         if (nz > 0) {
-            bw = (u64)(last - first);
+            bw = (unsigned)last - (unsigned)first;
             ng += 1;
             ms += 1;
             dq = fixq32(nz, bw + 1);
             cq = fixq32(ng, nz);
+            disp_ones += nz == bw + 1;
+            clust_ones += ng == nz;
         }
-        nnz_min_c = max(nnz_min_c, ~nz);
+        nnz_min = min(nnz_min, nz);
         nnz_max = max(nnz_max, nz);
         nnz_sum += nz;
-        nnz_sq += nz * nz;
-        bw_min_c = max(bw_min_c, ~bw);
+        nnz_sq += (u64)nz * nz;
+        bw_min = min(bw_min, bw);
         bw_max = max(bw_max, bw);
         bw_sum += bw;
-        bw_sq += (u128)bw * bw;
+        bw_sq += (u64)bw * bw;
         disp_sum += dq;
-        disp_sq += (u128)dq * dq;
+        disp_sq += (u64)dq * dq;
         clust_sum += cq;
         ng_sum += ng;
         ms_sum += ms;
     }
+
+    // minima as complements and the ratios of 1 folded in
+    __device__ __forceinline__ void words(u64* t, unsigned err) {
+        const u64 m32 = 0xffffffffull;
+        t[0] = nnz_min == 0xffffffffu ? 0 : ~(u64)nnz_min;
+        t[1] = nnz_max; t[2] = nnz_sum; t[3] = nnz_sq;
+        t[4] = bw_min == 0xffffffffu ? 0 : ~(u64)bw_min;
+        t[5] = bw_max; t[6] = bw_sum;
+        t[7] = disp_sum + ((u64)disp_ones << 32);
+        t[8] = clust_sum + ((u64)clust_ones << 32);
+        t[9] = ng_sum; t[10] = ms_sum; t[11] = err;
+        t[12] = (u64)bw_sq & m32; t[13] = (u64)bw_sq >> 32; t[14] = (u64)(bw_sq >> 64);
+        t[15] = (u64)disp_sq & m32; t[16] = (u64)disp_sq >> 32; t[17] = (u64)(disp_sq >> 64) + disp_ones;
+    }
 };
 
-// Warp reduction, then block reduction, then one set of atomics per block.
-template <bool FEATURES>
-__device__ void flush_block(RowAgg& r, u64 err, u64 (*s_red)[kFields], u64* s_err, FeatAcc* acc)
+// word f of two partials combined: 0, 1, 4 and 5 are maxima, 11 error bits
+__device__ __forceinline__ u64 merge_word(int f, u64 a, u64 b)
 {
-    for (int o = 16; o > 0; o >>= 1) err |= shfl_u64(err, o);
+    if (f == 0 || f == 1 || f == 4 || f == 5) return max(a, b);
+    return f == 11 ? (a | b) : a + b;
+}
+
+// Warp reductions, then the block's words added to one of the kSlots sets.
+// Validation alone adds the error bits.  (One set, 15 atomics from every
+// block to the same line, took longer than the pass over short matrices.)
+template <bool FEATURES>
+__device__ void flush_block(RowAgg& r, unsigned err, u64 (*s_red)[kFields], FeatCtl* ctl)
+{
+    err = __reduce_or_sync(FULL_MASK, err);
     const int w = threadIdx.x >> 5;
     if (FEATURES) {
-        r.nnz_min_c = warp_max_u64(r.nnz_min_c);
-        r.nnz_max = warp_max_u64(r.nnz_max);
+        r.nnz_min = __reduce_min_sync(FULL_MASK, r.nnz_min);
+        r.nnz_max = __reduce_max_sync(FULL_MASK, r.nnz_max);
+        r.bw_min = __reduce_min_sync(FULL_MASK, r.bw_min);
+        r.bw_max = __reduce_max_sync(FULL_MASK, r.bw_max);
+        r.disp_ones = __reduce_add_sync(FULL_MASK, r.disp_ones);
+        r.clust_ones = __reduce_add_sync(FULL_MASK, r.clust_ones);
         r.nnz_sum = warp_sum_u64(r.nnz_sum);
         r.nnz_sq = warp_sum_u64(r.nnz_sq);
-        r.bw_min_c = warp_max_u64(r.bw_min_c);
-        r.bw_max = warp_max_u64(r.bw_max);
         r.bw_sum = warp_sum_u64(r.bw_sum);
         r.bw_sq = warp_sum_u128(r.bw_sq);
         r.disp_sum = warp_sum_u64(r.disp_sum);
@@ -151,303 +182,358 @@ __device__ void flush_block(RowAgg& r, u64 err, u64 (*s_red)[kFields], u64* s_er
         r.ng_sum = warp_sum_u64(r.ng_sum);
         r.ms_sum = warp_sum_u64(r.ms_sum);
     }
+    if ((threadIdx.x & 31) == 0) r.words(s_red[w], err);
     __syncthreads();
-    if ((threadIdx.x & 31) == 0) {
-        if (err) atomicOr(s_err, err);
-        u64* t = s_red[w];
-        t[0] = r.nnz_min_c; t[1] = r.nnz_max; t[2] = r.nnz_sum; t[3] = r.nnz_sq;
-        t[4] = r.bw_min_c; t[5] = r.bw_max; t[6] = r.bw_sum;
-        t[7] = (u64)r.bw_sq; t[8] = (u64)(r.bw_sq >> 64);
-        t[9] = r.disp_sum; t[10] = (u64)r.disp_sq; t[11] = (u64)(r.disp_sq >> 64);
-        t[12] = r.clust_sum; t[13] = r.ng_sum; t[14] = r.ms_sum; t[15] = 0;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const int nw = blockDim.x >> 5;
-        if (*s_err) atomicOr(&acc->err, *s_err);
-        if (FEATURES) {
-            u64 t[kFields] = {0};
-            u128 bsq = 0, dsq = 0;
-            for (int k = 0; k < nw; ++k) {
-                const u64* q = s_red[k];
-                t[0] = max(t[0], q[0]); t[1] = max(t[1], q[1]); t[2] += q[2]; t[3] += q[3];
-                t[4] = max(t[4], q[4]); t[5] = max(t[5], q[5]); t[6] += q[6];
-                bsq += ((u128)q[8] << 64) | q[7];
-                t[9] += q[9];
-                dsq += ((u128)q[11] << 64) | q[10];
-                t[12] += q[12]; t[13] += q[13]; t[14] += q[14];
-            }
-            if (t[0]) atomicMax(&acc->nnz_min_c, t[0]);
-            if (t[1]) atomicMax(&acc->nnz_max, t[1]);
-            if (t[2]) atomicAdd(&acc->nnz_sum, t[2]);
-            if (t[3]) atomicAdd(&acc->nnz_sumsq, t[3]);
-            if (t[4]) atomicMax(&acc->bw_min_c, t[4]);
-            if (t[5]) atomicMax(&acc->bw_max, t[5]);
-            if (t[6]) atomicAdd(&acc->bw_sum, t[6]);
-            atomic_add_u128(&acc->bw_sq_lo, &acc->bw_sq_hi, bsq);
-            if (t[9]) atomicAdd(&acc->disp_sum, t[9]);
-            atomic_add_u128(&acc->disp_sq_lo, &acc->disp_sq_hi, dsq);
-            if (t[12]) atomicAdd(&acc->clust_sum, t[12]);
-            if (t[13]) atomicAdd(&acc->ngroups_sum, t[13]);
-            if (t[14]) atomicAdd(&acc->misses_sum, t[14]);
-        }
+    const int f = threadIdx.x;
+    if (f < kFields && (FEATURES || f == 11)) {
+        u64 t = s_red[0][f];
+        for (int k = 1; k < kFT / 32; ++k) t = merge_word(f, t, s_red[k][f]);
+        u64* to = &ctl->slot[blockIdx.x % kSlots][f];
+        if (t == 0) return;
+        if (f == 0 || f == 1 || f == 4 || f == 5) atomicMax(to, t);
+        else if (f == 11) atomicOr(to, t);
+        else atomicAdd(to, t);
     }
 }
 
-// The per-element tests in 32-bit integers.  Columns of a valid matrix lie
-// in [0, n_cols) with n_cols < 2^31, so the unsigned compare (unsigned)c >=
-// n_cols is c < 0 || c >= n_cols, and the difference of two columns, taken
-// modulo 2^32, is exact; a row with an invalid column or order sets an error
-// bit and the call returns an error, so its counts are never used.  A gap d
-// moves more than a line of line_bytes when 8 d > line_bytes, that is when
-// d > floor(line_bytes / 8) (d an integer).
+// Called by every thread of a block that has flushed: true in the block that
+// comes last of n_blocks (nothing waits), which then sees every flush.
+__device__ __forceinline__ bool last_to_flush(unsigned* done, unsigned n_blocks)
+{
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(done, 1u) == n_blocks - 1;
+    __syncthreads();
+    if (s_last) __threadfence();
+    return s_last;
+}
+
+// The last block: the sets' words combined, written to the host's buffer, and
+// the counters reset for the next call.
+__device__ __forceinline__ void publish(FeatCtl* ctl, FeatAcc* host)
+{
+    const int f = threadIdx.x;
+    if (f < kFields) {
+        u64 t = 0;
+#pragma unroll 16
+        for (int i = 0; i < kSlots; ++i) t = merge_word(f, t, __ldcg(&ctl->slot[i][f]));
+        reinterpret_cast<u64*>(host)[f] = t;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kSlots * kFields; i += kFT) (&ctl->slot[0][0])[i] = 0;
+    if (threadIdx.x == 0) ctl->n_long = ctl->n_pieces = ctl->done_pass = ctl->done_long = 0;
+}
+
+// The warp-wide scan of the columns.  A lane takes eight consecutive elements
+// per step (two 16-byte loads), a warp 256, a batch is four steps, whose
+// loads are in flight together.  Per element and test one subtraction
+// and one funnel shift collect a sign bit:
+//   g    1 + prev - c < 0        the column does not follow its predecessor by
+//                                one (for increasing columns)
+//   m    lb8 + prev - c < 0      it lies more than a line after it: 8 d >
+//                                line_bytes, that is d > lb8 =
+//                                floor(line_bytes / 8) for an integer d
+//   bad  c - prev - 1 < 0        it does not lie after it
+// and a running maximum of the columns as unsigned values finds any outside
+// [0, n_cols).  Columns in range make every difference exact; with one out of
+// range the call returns an error and the counts are not used.  The predecessor
+// of a lane's first element is its neighbour lane's last one, below lane 0
+// lane 31's of the step before.
+// Bound by instruction issue and the waits between a tile's loads
+// (ncu: 2.3 instructions a clock, DRAM 34 %).  Measured on a 100^3 27-point
+// stencil / 1M Zipf rows: 40 / 39 us; one element per lane with a ballot per
+// test (18 instructions where this takes 8) 57 / 66 us; a lane walking its own
+// row 56 / 60 us (rows of at most 64; the longer ones then took 93 us).
+//
+// The bits go to shared memory as bytes, element i of the batch to bit i % 8
+// of byte i / 8, so that 32 consecutive elements form a word.
 struct ColTest {
+    const int* ci;
+    int64_t nnz;
     unsigned n_cols;
-    int lb8;  // floor(line_bytes / 8)
+    int lb8;    // floor(line_bytes / 8)
+    int shift;  // elements ci lies past a 16-byte boundary
+};
+constexpr int kStep = 256, kBatch = 1024;
+struct BatchBits {
+    unsigned g[kBatch / 32], m[kBatch / 32], bad[kBatch / 32];
 };
 
-// Elements [j0, e) of a row starting at b, every `step`-th one, U at a time:
-// ng counts columns that do not follow their predecessor by one, ms those
-// more than a line away from it; bad collects CSR violations.
-template <int U>
-__device__ __forceinline__ void count_elements(int64_t b, int64_t j0, int64_t e, int step,
-                                               const int* __restrict__ ci, ColTest t, u64& ng, u64& ms,
-                                               u64& bad)
+// eight columns from element j on (ci + j on a 16-byte boundary); elements
+// outside [0, nnz) read as 0
+__device__ __forceinline__ void load8(const ColTest& t, int64_t j, int (&c)[8])
 {
-    unsigned g = 0, m = 0;  // at most kChunk / 32 elements a lane per call
-    for (; j0 < e; j0 += (int64_t)U * step) {
-        int c[U], cp[U];
+    if (j >= 0 && j + 8 <= t.nnz) {
+        const int4 a = __ldg(reinterpret_cast<const int4*>(t.ci + j)), b = __ldg(reinterpret_cast<const int4*>(t.ci + j) + 1);
+        c[0] = a.x; c[1] = a.y; c[2] = a.z; c[3] = a.w;
+        c[4] = b.x; c[5] = b.y; c[6] = b.z; c[7] = b.w;
+    } else {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int64_t j = j0 + u * step;
-            c[u] = j < e ? ci[j] : 0;
-            cp[u] = (j < e && j > b) ? ci[j - 1] : 0;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int64_t j = j0 + u * step;
-            if (j < e) {
-                if ((unsigned)c[u] >= t.n_cols) bad |= 8;
-                if (j > b) {
-                    const int d = (int)((unsigned)c[u] - (unsigned)cp[u]);
-                    if (d <= 0) bad |= 16;
-                    g += (d != 1);
-                    m += (d > t.lb8);
-                }
-            }
-        }
+        for (int u = 0; u < 8; ++u) c[u] = j + u >= 0 && j + u < t.nnz ? __ldg(t.ci + j + u) : 0;
     }
-    ng += g;
-    ms += m;
 }
 
-// Rows of at most kShortCap nonzeros: a lane per row, warps taking tiles of
-// 32 consecutive rows.  Each lane walks its row in order, four loads in
-// flight, keeping the previous column in a register, so every element is
-// loaded once and the per-row arithmetic (two 64-bit divisions, 128-bit
-// squares) runs on all 32 lanes.  Longer rows are listed for the chunked
-// kernels below.  Held to 64 registers (4 blocks of 256 per SM; a few bytes
-// of the per-row aggregates spill): 0.126 ms on the 27-point stencil
-// against 0.148 ms at 80 registers and 3 blocks.
-constexpr int64_t kShortCap = 64;
-constexpr int64_t kChunk = 4096;
+// the batch that covers element k: its first element (may be negative)
+__device__ __forceinline__ int64_t batch_start(const ColTest& t, int64_t k) { return ((k + t.shift) & ~(int64_t)7) - t.shift; }
+
+// one step: the lane's eight columns to its bits of the three tests (of bad
+// alone for validation)
+template <bool FEATURES>
+__device__ __forceinline__ void step_bits(const ColTest& t, const int (&c)[8], int lane, int& carry, unsigned& g, unsigned& m,
+                                          unsigned& bad, unsigned& top)
+{
+    const int turned = __shfl_sync(FULL_MASK, c[7], (lane + 31) & 31);
+    const int before = lane == 0 ? carry : turned;
+    carry = turned;
+    g = m = bad = 0;
+#pragma unroll
+    for (int u = 7; u >= 0; --u) {
+        const unsigned cu = (unsigned)c[u], pu = (unsigned)(u > 0 ? c[u - 1] : before);
+        if (FEATURES) {
+            g = __funnelshift_l(1u + pu - cu, g, 1);
+            m = __funnelshift_l((unsigned)t.lb8 + pu - cu, m, 1);
+        }
+        bad = __funnelshift_l(cu - pu - 1u, bad, 1);
+        top = max(top, cu);
+    }
+}
+
+// the lane's columns of the batch's four steps, all loads in flight together
+__device__ __forceinline__ void load_batch(const ColTest& t, int64_t k0, int len, int lane, int (&c)[4][8], int& carry)
+{
+    carry = k0 > 0 ? __ldg(t.ci + k0 - 1) : 0;  // the element before, meaningful in lane 0
+#pragma unroll
+    for (int h = 0; h < kBatch / kStep; ++h) {
+        const int i = h * kStep + lane * 8;
+        if (i < len) {
+            load8(t, k0 + i, c[h]);
+        } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) c[h][u] = 0;
+        }
+    }
+}
+
+// scans len <= kBatch elements from k0 = batch_start(...) on (rounded up to a
+// step's lanes) and leaves their bits in B
+template <bool FEATURES>
+__device__ __forceinline__ void scan_batch(const ColTest& t, int64_t k0, int len, int lane, BatchBits& B, unsigned& top)
+{
+    int c[kBatch / kStep][8], carry;
+    load_batch(t, k0, len, lane, c, carry);
+    uint8_t* bytes = reinterpret_cast<uint8_t*>(&B) + lane;
+#pragma unroll
+    for (int h = 0; h < kBatch / kStep; ++h) {
+        if (h * kStep >= len) break;  // whole warps
+        unsigned g, m, bad;
+        step_bits<FEATURES>(t, c[h], lane, carry, g, m, bad, top);
+        if (FEATURES) {
+            bytes[h * 32] = (uint8_t)g;
+            bytes[kBatch / 8 + h * 32] = (uint8_t)m;
+        }
+        bytes[2 * (kBatch / 8) + h * 32] = (uint8_t)bad;
+    }
+}
+
+// adds the bits of elements [p, es) of the batch
+template <bool FEATURES>
+__device__ __forceinline__ void count_bits(const BatchBits& B, int p, int es, unsigned& ng, unsigned& ms, unsigned& any_bad)
+{
+    while (p < es) {
+        const int i = p >> 5, next = (p | 31) + 1;
+        unsigned mask = 0xffffffffu << (p & 31);
+        if (es < next) mask &= (1u << (es & 31)) - 1u;
+        if (FEATURES) {
+            ng += __popc(B.g[i] & mask);
+            ms += __popc(B.m[i] & mask);
+        }
+        any_bad |= B.bad[i] & mask;
+        p = next;
+    }
+}
+
+// Rows of at most kLongRow nonzeros: warps take tiles of 32 consecutive
+// rows, a lane per row.  A lane walking its own row would read 32 places of
+// colind per instruction and run its tile as long as the tile's longest row;
+// instead the warp streams the tile's nonzeros, which are contiguous, in
+// batches (scan_batch, coalesced), and each lane then counts the bits of its
+// row in the batch's words.  The first element of a row has no predecessor:
+// its bit is left out.  The per-row arithmetic (two ratios, 128-bit sums)
+// runs on all 32 lanes.  Longer rows are listed in pieces of kPiece nonzeros
+// for k_feature_long, which their streaming skips: a tile costs at most 32
+// kLongRow elements.  One resident grid strides over the tiles.
+
+struct LongScratch {
+    FeatCtl* ctl;
+    int4* piece;      // [max_pieces] long row's list index, first element, row begin, row end
+    int2* row;        // [max_long] ng and ms of a long row's finished pieces
+    unsigned* done;   // [max_long] pieces finished
+    unsigned max_long, max_pieces;
+};
 
 template <bool FEATURES>
-__global__ void __launch_bounds__(256, 4)
+__global__ void __launch_bounds__(kFT, kFeatBlocks)
 k_feature_pass(int64_t n_rows, int64_t n_cols, int64_t nnz, const int* __restrict__ rp,
-               const int* __restrict__ ci, int64_t line_bytes, int* __restrict__ long_rows,
-               int64_t max_long, FeatAcc* __restrict__ acc)
+               const int* __restrict__ ci, int64_t line_bytes, LongScratch w, FeatAcc* __restrict__ host)
 {
-    constexpr int U = 4;
-    __shared__ u64 s_red[8][kFields];
-    __shared__ u64 s_err;
+    __shared__ u64 s_red[kFT / 32][kFields];
+    __shared__ BatchBits s_bits[kFT / 32];
     const int lane = threadIdx.x & 31;
+    BatchBits& bits = s_bits[threadIdx.x >> 5];
     RowAgg r;
-    u64 err = 0;
-    if (threadIdx.x == 0) s_err = 0;
+    unsigned err = 0, top = 0;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (rp[0] != 0) err |= 1;
         if ((int64_t)rp[n_rows] != nnz) err |= 2;
     }
     const int64_t n_tiles = (n_rows + 31) / 32;
-    const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x / 32);
-    const ColTest t{(unsigned)n_cols, (int)(line_bytes >> 3)};
-    for (int64_t tile = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; tile < n_tiles;
-         tile += n_warps) {
+    const int64_t n_warps = (int64_t)gridDim.x * (kFT / 32);
+    const ColTest t{ci, nnz, (unsigned)n_cols, (int)(line_bytes >> 3), (int)((uintptr_t)ci >> 2 & 3)};
+    int64_t tile = ((int64_t)blockIdx.x * kFT + threadIdx.x) / 32;
+    // the row pointers of the next tile are loaded one tile ahead
+    int nb = 0, ne = 0;
+    auto fetch = [&](int64_t tl) {
+        const int64_t row = tl * 32 + lane;
+        if (row < n_rows) { nb = rp[row]; ne = rp[row + 1]; }
+    };
+    fetch(tile);
+    for (; tile < n_tiles; tile += n_warps) {
         const int64_t row = tile * 32 + lane;
-        int64_t b = 0, nz = 0;
-        bool is_long = false, row_ok = false;
+        // [b, e): the row when it is valid and not long, else empty
+        int b = nb, e = ne;
+        if (tile + n_warps < n_tiles) fetch(tile + n_warps);
+        bool row_ok = false, is_long = false;
         if (row < n_rows) {
-            b = rp[row];
-            const int64_t e = rp[row + 1];
-            if (b < 0 || e < b || e > nnz) { err |= 4; b = 0; }
-            else if (e - b > kShortCap) is_long = true;
-            else { nz = e - b; row_ok = true; }
+            if (b < 0 || e < b || e > nnz) err |= 4;
+            else if (e - b > kLongRow) is_long = true;
+            else row_ok = true;
         }
+        // long rows: a list entry each and one per piece (pieces start on the
+        // scan's boundaries); overlapping rows (a rowptr that is not
+        // monotone) can list more than the buffers hold, and the error flag
+        // is set for them
+        for (unsigned todo = __ballot_sync(FULL_MASK, is_long); todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1;
+            const int lb = __shfl_sync(FULL_MASK, b, src), le = __shfl_sync(FULL_MASK, e, src);
+            const int64_t l0 = batch_start(t, lb);
+            const unsigned np = (unsigned)((le - l0 + kPiece - 1) / kPiece);
+            unsigned q = 0, p0 = 0;
+            if (lane == src) {
+                q = atomicAdd(&w.ctl->n_long, 1u);
+                if (q < w.max_long) {
+                    p0 = atomicAdd(&w.ctl->n_pieces, np);
+                    w.row[q] = make_int2(0, 0);
+                    w.done[q] = 0;
+                }
+            }
+            q = __shfl_sync(FULL_MASK, q, src);
+            p0 = __shfl_sync(FULL_MASK, p0, src);
+            if (q >= w.max_long) { err |= 4; continue; }
+            // every entry below n_pieces that the buffer holds is written
+            const unsigned room = p0 < w.max_pieces ? w.max_pieces - p0 : 0u;
+            if (np > room) err |= 4;
+            for (unsigned p = lane; p < min(np, room); p += 32)
+                w.piece[p0 + p] = make_int4((int)q, (int)(l0 + p * kPiece), lb, le);
+        }
+        if (!row_ok) b = e = 0;
         unsigned ng = 0, ms = 0;
-        int first = 0, prev = 0;
-        const int nzi = (int)nz;  // at most kShortCap
-        if (nzi > 0) {
-            first = prev = ci[b];
-            if ((unsigned)first >= t.n_cols) err |= 8;
+        int first = 0, last = 0;
+        if (FEATURES && e > b) {
+            first = ci[b];
+            last = ci[e - 1];
         }
-        for (int k = 1; k < nzi; k += U) {
-            int c[U];
+        const int hi = __reduce_max_sync(FULL_MASK, e);
+        for (int cur = 0;;) {
+            // the next element any row still needs (skips the long rows' parts)
+            const unsigned k = __reduce_min_sync(FULL_MASK, e > cur && e > b ? (unsigned)max(b, cur) : 0xffffffffu);
+            if (k == 0xffffffffu) break;
+            const int64_t k0 = batch_start(t, k);
+            const int len = (int)min((int64_t)kBatch, hi - k0);
+            scan_batch<FEATURES>(t, k0, len, lane, bits, top);
+            __syncwarp();
+            // this row's elements in the batch, without the row's first
+            const int64_t k1 = k0 + len;
+            unsigned any_bad = 0;
+            if (e > b) count_bits<FEATURES>(bits, (int)(max((int64_t)max(b + 1, cur), k0) - k0), (int)(min((int64_t)e, k1) - k0), ng, ms, any_bad);
+            if (any_bad) err |= 16;
+            __syncwarp();
+            cur = (int)k1;
+        }
+        if (FEATURES && row_ok) r.add((unsigned)(e - b), first, last, ng, ms);
+    }
+    if (top > 0 && top >= t.n_cols) err |= 8;
+    flush_block<FEATURES>(r, err, s_red, w.ctl);
+    // without long rows the result is complete here
+    if (last_to_flush(&w.ctl->done_pass, gridDim.x) && __ldcg(&w.ctl->n_pieces) == 0) publish(w.ctl, host);
+}
+
+// The long rows' pieces, a warp each.  A piece's counts, taken from the
+// lanes' bits without a detour through shared memory, are added to its row's;
+// the warp that completes a row's last piece (a ticket per row) adds the row
+// to its aggregates.  Integer sums: the result does not depend on the order.
+// The block that finishes last publishes the totals.
+template <bool FEATURES>
+__global__ void __launch_bounds__(kFT, kFeatBlocks)
+k_feature_long(int64_t n_cols, int64_t nnz, const int* __restrict__ ci, int64_t line_bytes, LongScratch w,
+               FeatAcc* __restrict__ host)
+{
+    __shared__ u64 s_red[kFT / 32][kFields];
+    const unsigned total = min(__ldcg(&w.ctl->n_pieces), w.max_pieces);
+    if (total == 0) return;  // published by the pass
+    const int lane = threadIdx.x & 31;
+    RowAgg r;
+    unsigned err = 0, top = 0;
+    const ColTest t{ci, nnz, (unsigned)n_cols, (int)(line_bytes >> 3), (int)((uintptr_t)ci >> 2 & 3)};
+    const unsigned n_warps = gridDim.x * (kFT / 32);
+    unsigned it = (blockIdx.x * kFT + threadIdx.x) / 32;
+    int4 next = it < total ? w.piece[it] : make_int4(0, 0, 0, 0);
+    for (; it < total; it += n_warps) {
+        const int4 pc = next;
+        if (it + n_warps < total) next = w.piece[it + n_warps];
+        const int b = pc.z, e = pc.w;
+        const int64_t p0 = pc.y;  // may be negative
+        const int plen = (int)min((int64_t)e - p0, kPiece);
+        unsigned ng = 0, ms = 0, any_bad = 0;
+        for (int at = 0; at < plen; at += kBatch) {
+            const int64_t k0 = p0 + at;
+            const int len = min(kBatch, plen - at);
+            int c[kBatch / kStep][8], carry;
+            load_batch(t, k0, len, lane, c, carry);
+            // elements of the batch that count: after the row's first, before its end
+            const int from = (int)max((int64_t)0, (int64_t)b + 1 - k0);
 #pragma unroll
-            for (int u = 0; u < U; ++u) c[u] = k + u < nzi ? ci[b + k + u] : 0;
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (k + u < nzi) {
-                    if ((unsigned)c[u] >= t.n_cols) err |= 8;
-                    const int d = (int)((unsigned)c[u] - (unsigned)prev);
-                    if (d <= 0) err |= 16;
-                    ng += (d != 1);
-                    ms += (d > t.lb8);
-                    prev = c[u];
+            for (int h = 0; h < kBatch / kStep; ++h) {
+                unsigned g, m, bad;
+                step_bits<FEATURES>(t, c[h], lane, carry, g, m, bad, top);
+                const int i = h * kStep + lane * 8;  // the lane's first element of the step
+                const unsigned keep = (0xffu << min(max(from - i, 0), 8)) & ((1u << min(max(len - i, 0), 8)) - 1u);
+                ng += __popc(g & keep);
+                ms += __popc(m & keep);
+                any_bad |= bad & keep;
+            }
+        }
+        if (any_bad) err |= 16;
+        if (FEATURES) {
+            ng = __reduce_add_sync(FULL_MASK, ng);
+            ms = __reduce_add_sync(FULL_MASK, ms);
+            if (lane == 0) {
+                int2* tot = w.row + pc.x;
+                atomicAdd(&tot->x, (int)ng);
+                atomicAdd(&tot->y, (int)ms);
+                __threadfence();
+                const unsigned np = (unsigned)((e - batch_start(t, b) + kPiece - 1) / kPiece);
+                if (atomicAdd(&w.done[pc.x], 1u) == np - 1) {
+                    __threadfence();
+                    const int2 all = __ldcg(tot);
+                    r.add((unsigned)(e - b), ci[b], ci[e - 1], (unsigned)all.x, (unsigned)all.y);
                 }
             }
         }
-        if (FEATURES && row_ok) r.add((u64)nz, first, prev, ng, ms);
-        // long rows: up to kChunk nonzeros to the front of the list (a warp
-        // each), longer ones to the back (chunked)
-        const bool huge = is_long && rp[row + 1] - rp[row] > kChunk;
-        const unsigned mm = __ballot_sync(FULL_MASK, is_long && !huge);
-        const unsigned mh = __ballot_sync(FULL_MASK, huge);
-        if (mm | mh) {
-            u64 bm = 0, bh = 0;
-            if (lane == 0) {
-                if (mm) bm = atomicAdd(&acc->n_long, (u64)__popc(mm));
-                if (mh) bh = atomicAdd(&acc->n_huge, (u64)__popc(mh));
-            }
-            bm = __shfl_sync(FULL_MASK, bm, 0);
-            bh = __shfl_sync(FULL_MASK, bh, 0);
-            const unsigned lt = (1u << lane) - 1u;
-            // overlapping rows (a rowptr that is not monotone) can list more
-            // rows than the buffer holds; the error flag is set for them
-            if (is_long && !huge) {
-                const u64 pos = bm + __popc(mm & lt);
-                if (pos < (u64)max_long) long_rows[pos] = (int)row;
-                else err |= 4;
-            }
-            if (huge) {
-                const u64 pos = bh + __popc(mh & lt);
-                if (pos < (u64)max_long) long_rows[max_long - 1 - pos] = (int)row;
-                else err |= 4;
-            }
-        }
     }
-    flush_block<FEATURES>(r, err, s_red, &s_err, acc);
-}
-
-// Exclusive scan of the huge rows' chunk counts (one block, a contiguous
-// segment per thread): chunk_off[q] is the first chunk of huge row q (list
-// entry max_long - 1 - q), chunk_off[n_huge] their total.  Also zeroes the
-// per-row totals, the tickets and the work counter of the chunk kernel.
-__global__ void __launch_bounds__(1024)
-k_chunk_offsets(const int* __restrict__ long_rows, int64_t max_long, const int* __restrict__ rp,
-                int* __restrict__ chunk_off, u64* __restrict__ ng, u64* __restrict__ ms,
-                unsigned* __restrict__ done, unsigned* __restrict__ next,
-                const FeatAcc* __restrict__ acc)
-{
-    __shared__ int part[1024];
-    const int64_t nh = min((int64_t)acc->n_huge, max_long);
-    const int n = (int)nh;
-    for (int q = threadIdx.x; q < n; q += 1024) { ng[q] = 0; ms[q] = 0; done[q] = 0; }
-    if (threadIdx.x == 0) *next = 0;
-    const int per = (n + 1023) / 1024;
-    const int q0 = min(n, (int)threadIdx.x * per), q1 = min(n, q0 + per);
-    int local = 0;
-    for (int q = q0; q < q1; ++q) {
-        const int row = long_rows[max_long - 1 - q];
-        local += (int)((rp[row + 1] - rp[row] + kChunk - 1) / kChunk);
-    }
-    part[threadIdx.x] = local;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-        const int t = threadIdx.x >= o ? part[threadIdx.x - o] : 0;
-        __syncthreads();
-        part[threadIdx.x] += t;
-        __syncthreads();
-    }
-    int run = part[threadIdx.x] - local;
-    for (int q = q0; q < q1; ++q) {
-        chunk_off[q] = run;
-        const int row = long_rows[max_long - 1 - q];
-        run += (int)((rp[row + 1] - rp[row] + kChunk - 1) / kChunk);
-    }
-    if (threadIdx.x == 1023) chunk_off[n] = part[1023];
-}
-
-// Chunks of kChunk nonzeros of the long rows: persistent warps take chunks
-// from an atomic counter, add the chunk's counts to the row's totals, and the
-// warp that completes a row's last chunk (a ticket per row) adds the row to
-// its aggregates.  Integer sums: the result does not depend on the order.
-struct LongScratch {
-    u64* ng;          // [max_long]
-    u64* ms;          // [max_long]
-    unsigned* done;   // [max_long] chunks finished
-    unsigned* next;   // work counter
-};
-
-template <bool FEATURES>
-__global__ void __launch_bounds__(256)
-k_feature_chunks(const int* __restrict__ long_rows, int64_t max_long, const int* __restrict__ chunk_off,
-                 int64_t n_cols, const int* __restrict__ rp, const int* __restrict__ ci,
-                 int64_t line_bytes, LongScratch w, FeatAcc* __restrict__ acc)
-{
-    __shared__ u64 s_red[8][kFields];
-    __shared__ u64 s_err;
-    if (threadIdx.x == 0) s_err = 0;
-    const int lane = threadIdx.x & 31;
-    const int n_mid = (int)min((int64_t)acc->n_long, max_long);
-    const int n_huge = (int)min((int64_t)acc->n_huge, max_long);
-    const int total = n_mid + (n_huge > 0 ? chunk_off[n_huge] : 0);
-    RowAgg r;
-    u64 bad = 0;
-    const ColTest t{(unsigned)n_cols, (int)(line_bytes >> 3)};
-    for (;;) {
-        int it = 0;
-        if (lane == 0) it = (int)atomicAdd(w.next, 1u);
-        it = __shfl_sync(FULL_MASK, it, 0);
-        if (it >= total) break;
-        if (it < n_mid) {
-            // a row of at most kChunk nonzeros: the whole row by this warp
-            const int row = long_rows[it];
-            const int64_t b = rp[row], e = rp[row + 1];
-            u64 ng = 0, ms = 0;
-            count_elements<4>(b, b + lane, e, 32, ci, t, ng, ms, bad);
-            ng = warp_sum_u64(ng);
-            ms = warp_sum_u64(ms);
-            if (FEATURES && lane == 0) r.add((u64)(e - b), (int64_t)ci[b], (int64_t)ci[e - 1], ng, ms);
-            continue;
-        }
-        const int ic = it - n_mid;
-        int lo = 0, hi = n_huge - 1;  // the huge row whose chunks include ic
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (chunk_off[mid] <= ic) lo = mid; else hi = mid - 1;
-        }
-        const int row = long_rows[max_long - 1 - lo];
-        const int64_t b = rp[row], e = rp[row + 1];
-        const int64_t c0 = b + (int64_t)(ic - chunk_off[lo]) * kChunk;
-        const int64_t c1 = min(e, c0 + kChunk);
-        u64 ng = 0, ms = 0;
-        count_elements<4>(b, c0 + lane, c1, 32, ci, t, ng, ms, bad);
-        ng = warp_sum_u64(ng);
-        ms = warp_sum_u64(ms);
-        if (lane == 0) {
-            atomicAdd(&w.ng[lo], ng);
-            atomicAdd(&w.ms[lo], ms);
-            __threadfence();
-            const unsigned n_chunks = (unsigned)(chunk_off[lo + 1] - chunk_off[lo]);
-            if (atomicAdd(&w.done[lo], 1u) == n_chunks - 1) {
-                __threadfence();
-                const u64 tng = atomicAdd(&w.ng[lo], 0ull), tms = atomicAdd(&w.ms[lo], 0ull);
-                if (FEATURES) r.add((u64)(e - b), (int64_t)ci[b], (int64_t)ci[e - 1], tng, tms);
-            }
-        }
-    }
-    flush_block<FEATURES>(r, bad, s_red, &s_err, acc);
+    if (top > 0 && top >= t.n_cols) err |= 8;
+    flush_block<FEATURES>(r, err, s_red, w.ctl);
+    if (last_to_flush(&w.ctl->done_long, gridDim.x)) publish(w.ctl, host);
 }
 
 double sd_from_sums(u64 n, u64 s1, u128 s2)
@@ -456,16 +542,20 @@ double sd_from_sums(u64 n, u64 s1, u128 s2)
     return sqrt((double)num) / (double)n;
 }
 
+// the 128-bit sum of digits of 32, 32 and 64 bits
+u128 digits(const u64 (&d)[3]) { return ((u128)d[2] << 64) + ((u128)d[1] << 32) + d[0]; }
+
 float lg1p(double v) { return (float)log2(1.0 + v); }
 
-// pinned host staging for the accumulator readback, one per host thread
+// page-locked result buffer the last block writes, one per host thread
 thread_local FeatAcc* t_host_acc = nullptr;
-thread_local FeatAcc* t_dev_acc = nullptr;
-thread_local int t_dev_acc_device = -1;
-// device scratch of the long-row kernels, per host thread; grows, never shrinks
+// device scratch of the pass (counters first), per host thread; grows, never
+// shrinks.  The counters are 0 between calls; after a failed call the scratch
+// is cleared again.
 thread_local void* t_scratch = nullptr;
 thread_local size_t t_scratch_bytes = 0;
 thread_local int t_scratch_device = -1;
+thread_local bool t_scratch_clean = false;
 
 }  // namespace
 
@@ -492,68 +582,53 @@ spmv_status run_feature_pass(const spmv_csr_t* A, int32_t line_bytes, spmv_featu
             return fail(SPMV_ERR_NOMEM, "cudaMallocHost for the feature readback failed");
         t_host_acc = static_cast<FeatAcc*>(p);
     }
-    // one device accumulator per host thread and device, kept for reuse
-    if (t_dev_acc_device != dev.device || !t_dev_acc) {
-        void* p = nullptr;
-        SPMV_CUDA_TRY(cudaMalloc(&p, sizeof(FeatAcc)));
-        t_dev_acc = static_cast<FeatAcc*>(p);
-        t_dev_acc_device = dev.device;
-    }
-    FeatAcc* acc = t_dev_acc;
-    cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(FeatAcc), s);
-    if (e == cudaSuccess && A->n_rows > 0) {
-        // scratch: per-long-row totals and tickets, the work counter, the
-        // long-row list and the chunk offsets
-        const int64_t max_long = std::min<int64_t>(A->n_rows, A->nnz / (kShortCap + 1) + 1);
-        const size_t bytes = sizeof(u64) * 2 * (size_t)max_long + sizeof(unsigned) * (size_t)(max_long + 1) +
-                             sizeof(int) * (size_t)(2 * max_long + 1) + 64;
-        if (t_scratch_device != dev.device || t_scratch_bytes < bytes) {
+    cudaError_t e = cudaSuccess;
+    if (A->n_rows > 0) {
+        const int64_t n_tiles = (A->n_rows + 31) / 32;
+        const int64_t resident = (int64_t)dev.sm_count * kFeatBlocks;
+        const unsigned blocks = (unsigned)std::min<int64_t>((n_tiles + kFT / 32 - 1) / (kFT / 32), resident);
+        // long rows and pieces a valid matrix can hold
+        const int64_t max_long = std::min<int64_t>(A->n_rows, A->nnz / (kLongRow + 1) + 1);
+        const int64_t max_pieces = A->nnz / kPiece + 2 * max_long;
+        const unsigned lblocks = (unsigned)std::min<int64_t>((max_pieces + kFT / 32 - 1) / (kFT / 32), resident);
+        LongScratch w;
+        size_t at = 0;
+        auto place = [&](size_t bytes) { const size_t p = at; at += (bytes + 15) / 16 * 16; return p; };
+        const size_t o_ctl = place(sizeof(FeatCtl)), o_piece = place(sizeof(int4) * max_pieces),
+                     o_row = place(sizeof(int2) * max_long), o_done = place(sizeof(unsigned) * max_long);
+        if (t_scratch_device != dev.device || t_scratch_bytes < at) {
             if (t_scratch) cudaFree(t_scratch);
             t_scratch = nullptr;
             t_scratch_bytes = 0;
-            e = cudaMalloc(&t_scratch, bytes);
-            if (e == cudaSuccess) { t_scratch_bytes = bytes; t_scratch_device = dev.device; }
+            t_scratch_clean = false;
+            e = cudaMalloc(&t_scratch, at);
+            if (e == cudaSuccess) { t_scratch_bytes = at; t_scratch_device = dev.device; }
         }
-        u64* ng = static_cast<u64*>(t_scratch);
-        u64* ms = ng + max_long;
-        unsigned* done = reinterpret_cast<unsigned*>(ms + max_long);
-        unsigned* next = done + max_long;
-        int* long_rows = reinterpret_cast<int*>(next + 1);
-        int* chunk_off = long_rows + max_long;
-        int64_t blocks = ((A->n_rows + 31) / 32 * 32 + 255) / 256;
-        const int64_t lim = (int64_t)dev.sm_count * 16;
-        if (blocks > lim) blocks = lim;
-        if (blocks < 1) blocks = 1;
-        const unsigned cgrid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(max_long, (int64_t)dev.sm_count * 2));
-        LongScratch w{ng, ms, done, next};
+        if (e == cudaSuccess && !t_scratch_clean) e = cudaMemsetAsync(t_scratch, 0, t_scratch_bytes, s);
+        t_scratch_clean = false;  // until this call has completed
+        unsigned char* base = static_cast<unsigned char*>(t_scratch);
+        w.ctl = reinterpret_cast<FeatCtl*>(base + o_ctl);
+        w.piece = reinterpret_cast<int4*>(base + o_piece);
+        w.row = reinterpret_cast<int2*>(base + o_row);
+        w.done = reinterpret_cast<unsigned*>(base + o_done);
+        w.max_long = (unsigned)max_long;
+        w.max_pieces = (unsigned)max_pieces;
         if (e == cudaSuccess) {
-            if (out)
-                k_feature_pass<true><<<(unsigned)blocks, 256, 0, s>>>(A->n_rows, A->n_cols, A->nnz, A->rowptr,
-                                                                      A->colind, line_bytes, long_rows, max_long, acc);
-            else
-                k_feature_pass<false><<<(unsigned)blocks, 256, 0, s>>>(A->n_rows, A->n_cols, A->nnz, A->rowptr,
-                                                                       A->colind, line_bytes, long_rows, max_long, acc);
+            if (out) k_feature_pass<true><<<blocks, kFT, 0, s>>>(A->n_rows, A->n_cols, A->nnz, A->rowptr, A->colind, line_bytes, w, t_host_acc);
+            else k_feature_pass<false><<<blocks, kFT, 0, s>>>(A->n_rows, A->n_cols, A->nnz, A->rowptr, A->colind, line_bytes, w, t_host_acc);
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) {
-            k_chunk_offsets<<<1, 1024, 0, s>>>(long_rows, max_long, A->rowptr, chunk_off, ng, ms, done,
-                                               next, acc);
+            if (out) k_feature_long<true><<<lblocks, kFT, 0, s>>>(A->n_cols, A->nnz, A->colind, line_bytes, w, t_host_acc);
+            else k_feature_long<false><<<lblocks, kFT, 0, s>>>(A->n_cols, A->nnz, A->colind, line_bytes, w, t_host_acc);
             e = cudaGetLastError();
         }
-        if (e == cudaSuccess) {
-            if (out)
-                k_feature_chunks<true><<<cgrid, 256, 0, s>>>(long_rows, max_long, chunk_off, A->n_cols, A->rowptr,
-                                                             A->colind, line_bytes, w, acc);
-            else
-                k_feature_chunks<false><<<cgrid, 256, 0, s>>>(long_rows, max_long, chunk_off, A->n_cols, A->rowptr,
-                                                              A->colind, line_bytes, w, acc);
-            e = cudaGetLastError();
-        }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return cuda_fail(e, "feature pass");
+        t_scratch_clean = true;
+    } else {
+        memset(t_host_acc, 0, sizeof(FeatAcc));
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(t_host_acc, acc, sizeof(FeatAcc),
-                                              cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_fail(e, "feature pass");
 
     const FeatAcc& h = *t_host_acc;
     u64 err = h.err;
@@ -583,11 +658,12 @@ spmv_status run_feature_pass(const spmv_csr_t* A, int32_t line_bytes, spmv_featu
     f.bw_min = N > 0 ? (int64_t)~h.bw_min_c : 0;
     f.bw_max = (int64_t)h.bw_max;
     f.bw_sum = h.bw_sum;
-    f.bw_sumsq_lo = h.bw_sq_lo;
-    f.bw_sumsq_hi = h.bw_sq_hi;
+    const u128 bw_s2 = digits(h.bw_sq), dq_s2 = digits(h.disp_sq);
+    f.bw_sumsq_lo = (uint64_t)bw_s2;
+    f.bw_sumsq_hi = (uint64_t)(bw_s2 >> 64);
     f.disp_sum = h.disp_sum;
-    f.disp_sumsq_lo = h.disp_sq_lo;
-    f.disp_sumsq_hi = h.disp_sq_hi;
+    f.disp_sumsq_lo = (uint64_t)dq_s2;
+    f.disp_sumsq_hi = (uint64_t)(dq_s2 >> 64);
     f.clust_sum = h.clust_sum;
     f.ngroups_sum = h.ngroups_sum;
     f.misses_sum = h.misses_sum;
@@ -597,8 +673,6 @@ spmv_status run_feature_pass(const spmv_csr_t* A, int32_t line_bytes, spmv_featu
     if (N > 0) {
         const double q32 = 1.0 / 4294967296.0;
         const double dn = (double)N;
-        const u128 bw_s2 = ((u128)f.bw_sumsq_hi << 64) | f.bw_sumsq_lo;
-        const u128 dq_s2 = ((u128)f.disp_sumsq_hi << 64) | f.disp_sumsq_lo;
         f.nnz_avg = (double)f.nnz_sum / dn;
         f.nnz_sd = sd_from_sums((u64)N, f.nnz_sum, (u128)f.nnz_sumsq_lo);
         f.bw_avg = (double)f.bw_sum / dn;
