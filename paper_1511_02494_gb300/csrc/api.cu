@@ -57,7 +57,116 @@ void persist_release(int d)
     cudaGetLastError();
     if (cur != d) cudaSetDevice(cur);
 }
+
+// one memory pool per device, with a stream of its own for the frees (the
+// legacy stream would order them with every other stream, and break captures)
+struct DevicePool {
+    cudaMemPool_t pool = nullptr;
+    cudaStream_t stream = nullptr;
+    int users = 0;
+};
+std::mutex g_pool_mu;
+DevicePool g_pool[kMaxDevices];
+
+// g_pool_mu held
+cudaError_t pool_open(int d)
+{
+    DevicePool& g = g_pool[d];
+    if (g.pool) return cudaSuccess;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = d;
+    cudaMemPool_t pool = nullptr;
+    cudaStream_t stream = nullptr;
+    cudaError_t e = cudaMemPoolCreate(&pool, &props);
+    // nothing is given back behind our back at a synchronisation: pool_free
+    // and pool_release keep the bound
+    uint64_t never = UINT64_MAX;
+    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &never);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking);
+    if (e != cudaSuccess) {
+        if (pool) cudaMemPoolDestroy(pool);
+        return e;
+    }
+    g.pool = pool;
+    g.stream = stream;
+    return cudaSuccess;
+}
+
+cudaError_t pool_get(int d, cudaMemPool_t* pool, cudaStream_t* stream)
+{
+    if (d < 0 || d >= kMaxDevices) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    cudaError_t e = pool_open(d);
+    *pool = g_pool[d].pool;
+    *stream = g_pool[d].stream;
+    return e;
+}
+
+// gives back what the pool holds beyond the memory in use and `keep`
+void pool_trim(cudaMemPool_t pool, size_t keep)
+{
+    uint64_t used = 0, reserved = 0;
+    if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess &&
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
+        reserved > used + keep)
+        cudaMemPoolTrimTo(pool, (size_t)used + keep);
+}
 }  // namespace
+
+cudaError_t pool_alloc(int device, void** p, size_t bytes)
+{
+    cudaMemPool_t pool;
+    cudaStream_t st;
+    cudaError_t e = pool_get(device, &pool, &st);
+    if (e != cudaSuccess) return e;
+    e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+    if (e == cudaErrorMemoryAllocation) {
+        // memory that is free but kept, or in pieces too small
+        cudaGetLastError();
+        cudaStreamSynchronize(st);
+        cudaMemPoolTrimTo(pool, 0);
+        e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+    }
+    return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+}
+
+void pool_free(int device, void* const* p, size_t count)
+{
+    if (count == 0) return;
+    cudaMemPool_t pool;
+    cudaStream_t st;
+    if (pool_get(device, &pool, &st) != cudaSuccess) return;
+    for (size_t i = 0; i < count; ++i) cudaFreeAsync(p[i], st);
+    cudaStreamSynchronize(st);
+    pool_trim(pool, kPoolKeep);
+}
+
+spmv_status pool_acquire(int device)
+{
+    if (device < 0 || device >= kMaxDevices) return fail(SPMV_ERR_CUDA, "device ordinal out of range");
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    SPMV_CUDA_TRY(pool_open(device));
+    ++g_pool[device].users;
+    return SPMV_OK;
+}
+
+void pool_release(int device)
+{
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (--g_pool[device].users == 0) cudaMemPoolTrimTo(g_pool[device].pool, 0);
+}
+
+cudaError_t work_alloc(int device, void** p, size_t bytes, cudaStream_t s)
+{
+    // large scratch does not stay mapped: the device's default pool
+    if (bytes > kPoolKeep / 4) return cudaMallocAsync(p, bytes, s);
+    cudaMemPool_t pool;
+    cudaStream_t st;
+    cudaError_t e = pool_get(device, &pool, &st);
+    return e == cudaSuccess ? cudaMallocFromPoolAsync(p, bytes, pool, s) : e;
+}
 
 void set_error(const std::string& msg) { t_last_error = msg; }
 void clear_error() { t_last_error.clear(); }
@@ -118,13 +227,13 @@ spmv_status prepared_alloc(spmv_prepared* P, void** p, int64_t bytes)
 {
     *p = nullptr;
     if (bytes <= 0) return SPMV_OK;
-    cudaError_t e = cudaMalloc(p, (size_t)bytes);
+    cudaError_t e = pool_alloc(P->device, p, (size_t)bytes);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         *p = nullptr;
-        return fail(SPMV_ERR_NOMEM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed");
+        return fail(SPMV_ERR_NOMEM, "allocation of " + std::to_string(bytes) + " device bytes failed");
     }
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc");
+    if (e != cudaSuccess) return cuda_fail(e, "device allocation");
     P->owned.push_back(*p);
     P->owned_bytes += bytes;
     return SPMV_OK;
@@ -150,28 +259,16 @@ bool merge_items_ok(int items)
 template <typename T>
 spmv_status dev_alloc(spmv_prepared_t* P, T** p, int64_t count)
 {
-    *p = nullptr;
-    if (count <= 0) return SPMV_OK;
-    const size_t bytes = sizeof(T) * (size_t)count;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
-    if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        *p = nullptr;
-        return fail(SPMV_ERR_NOMEM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed");
-    }
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc");
-    P->owned.push_back(*p);
-    P->owned_bytes += (int64_t)bytes;
-    return SPMV_OK;
+    return prepared_alloc(P, reinterpret_cast<void**>(p), (int64_t)sizeof(T) * count);
 }
 
 // Frees every device allocation the object made (each one registered itself
 // in P->owned when it was made), whatever the variant.
 void release(spmv_prepared_t* P)
 {
-    for (void* p : P->owned)
-        if (p) cudaFree(p);
+    pool_free(P->device, P->owned.data(), P->owned.size());
     P->owned.clear();
+    pool_release(P->device);
     if (P->persist_held) {
         persist_release(P->device);
         P->persist_held = false;
@@ -220,7 +317,7 @@ int64_t min_bytes_of(const spmv_prepared_t* P)
     return (int64_t)(vb + 2) * A.nnz + 4 * A.n_rows + vec + xconv;
 }
 
-spmv_status prepare_impl(spmv_prepared_t* P, cudaStream_t s)
+spmv_status prepare_impl(spmv_prepared_t* P, bool check, cudaStream_t s)
 {
     const spmv_csr_t& A = P->A;
     spmv_choice_t& c = P->c;
@@ -333,7 +430,7 @@ spmv_status prepare_impl(spmv_prepared_t* P, cudaStream_t s)
             return SPMV_OK;
         }
         case SPMV_V7_SLICED:
-            return sliced_prepare(P, s);
+            return sliced_prepare(P, check, s);
         default:
             return fail(SPMV_ERR_INVALID_ARG, "unknown variant");
     }
@@ -585,8 +682,10 @@ spmv_status spmv_prepare(const spmv_csr_t* A, const spmv_choice_t* c, int32_t tr
     if (st != SPMV_OK) return st;
     if ((st = check_choice(c)) != SPMV_OK) return st;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    // SLICED reads the verdict of the validation at the first wait of its own
+    const bool check_later = !trusted && c->variant == SPMV_V7_SLICED && A->n_rows > 0;
     if (!trusted) {
-        st = run_feature_pass(A, 128, nullptr, s);
+        st = check_later ? feature_pass_enqueue(A, 128, false, s) : run_feature_pass(A, 128, nullptr, s);
         if (st != SPMV_OK) return st;
     }
     DeviceInfo dev;
@@ -597,12 +696,22 @@ spmv_status spmv_prepare(const spmv_csr_t* A, const spmv_choice_t* c, int32_t tr
     P->c = *c;
     P->device = dev.device;
     P->sm_count = dev.sm_count;
-    st = prepare_impl(P, s);
-    if (st == SPMV_OK) {
+    if ((st = pool_acquire(dev.device)) != SPMV_OK) {
+        delete P;
+        return st;
+    }
+    st = prepare_impl(P, check_later, s);
+    if (st == SPMV_OK && (c->variant != SPMV_V7_SLICED || A->n_rows == 0)) {
         cudaError_t e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) st = cuda_fail(e, "spmv_prepare");
     }
-    if (st == SPMV_OK && A->n_rows > 0) {
+    if (st == SPMV_OK && A->n_rows > 0 && c->variant == SPMV_V7_SLICED) {
+        // load the variant's kernels now, so that later launches, including
+        // captured ones, load nothing
+        cudaError_t e = launch_sliced(P, nullptr, nullptr, s, true);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) st = cuda_fail(e, "spmv_prepare configure");
+    } else if (st == SPMV_OK && A->n_rows > 0) {
         // configure the variant's kernels now (one SpMV into scratch vectors),
         // so that later launches, including captured ones, make no
         // configuration call

@@ -65,6 +65,7 @@ struct spmv_batch {
     std::vector<spmv_csr_t> mats;
     std::vector<int32_t> tpr, rpi;   // lanes per row, rows per item
     std::vector<const spmv_prepared*> preps;  // SLICED matrices' prepared objects, else null
+    std::vector<std::vector<int32_t>> seg_row;  // their segments' rows, -1 where the row has several (empty: none has)
     std::vector<spmv_prepared*> owned;        // sliced forms the batch prepared itself
     std::vector<const double*> xs;
     std::vector<double*> ys;
@@ -175,13 +176,14 @@ std::vector<BatchItem> make_items(const spmv_batch* B, const std::vector<int32_t
                                   const std::vector<int32_t>& rpi)
 {
     std::vector<BatchItem> items;
+    auto several = [&](size_t m, int j) { return !B->seg_row[m].empty() && B->seg_row[m][j] < 0; };
     // the segments of rows that span several (the longest work, a row of
     // up to 2^31 nonzeros) of every sliced matrix first; then per matrix its
     // slices or row chunks, and the rows of a single segment
     for (size_t m = 0; m < B->mats.size(); ++m)
         if (const spmv_prepared* P = B->preps[m])
             for (int j = 0; j < P->sl.n_seg; ++j)
-                if (P->sl.seg_several[j]) items.push_back({(int32_t)m, j, j + 1, kSegItem});
+                if (several(m, j)) items.push_back({(int32_t)m, j, j + 1, kSegItem});
     for (size_t m = 0; m < B->mats.size(); ++m) {
         const spmv_prepared* P = B->preps[m];
         if (P) {
@@ -190,7 +192,7 @@ std::vector<BatchItem> make_items(const spmv_batch* B, const std::vector<int32_t
             const int k = std::max(1, rpi[m] / 32);
             for (int s0 = 0; s0 < ns; s0 += k) items.push_back({(int32_t)m, s0, std::min(ns, s0 + k), kSliceItem});
             for (int j = 0; j < P->sl.n_seg; ++j)
-                if (!P->sl.seg_several[j]) items.push_back({(int32_t)m, j, j + 1, kSegItem});
+                if (!several(m, j)) items.push_back({(int32_t)m, j, j + 1, kSegItem});
             continue;
         }
         const int n = (int)B->mats[m].n_rows;
@@ -223,6 +225,17 @@ spmv_status finish_create(spmv_batch* B, int32_t count, cudaStream_t s, spmv_bat
     if (e == cudaSuccess) e = cudaMemsetAsync(B->d_counter, 0, 8, s);
     if (e == cudaSuccess && count > 0)
         e = cudaMalloc(reinterpret_cast<void**>(&B->d_mats), sizeof(BatchMat) * count);
+    if (e != cudaSuccess) { spmv_batch_free(B); return cuda_fail(e, "spmv_batch_create"); }
+    // which segments belong to rows of several
+    B->seg_row.resize(count);
+    for (int m = 0; m < count && e == cudaSuccess; ++m)
+        if (const spmv_prepared* P = B->preps[m])
+            if (P->sl.n_fix > 0) {
+                B->seg_row[m].resize(P->sl.n_seg);
+                e = cudaMemcpyAsync(B->seg_row[m].data(), P->sl.seg_row, 4 * (size_t)P->sl.n_seg,
+                                    cudaMemcpyDeviceToHost, s);
+            }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) { spmv_batch_free(B); return cuda_fail(e, "spmv_batch_create"); }
     spmv_status st = build_items(B, s);
     if (st != SPMV_OK) { spmv_batch_free(B); return st; }

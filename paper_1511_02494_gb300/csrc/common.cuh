@@ -38,6 +38,24 @@ struct DeviceInfo {
 // Facts of the current device (queried once per device).
 spmv_status current_device(DeviceInfo* out);
 
+// ---- device memory ------------------------------------------------------------
+// The library's memory pool of a device.  Prepared objects live in it, and
+// while any does, up to kPoolKeep bytes that freed objects left stay mapped
+// for the next one (mapping and unmapping memory took 0.6 of the 1.5 ms that
+// a 100^3 27-point stencil spent from features to first product); when the
+// device's last object is freed, all of it goes back to the system.  Safe
+// from several threads.
+constexpr size_t kPoolKeep = (size_t)1 << 30;
+// usable on every stream once the call returns, like cudaMalloc
+cudaError_t pool_alloc(int device, void** p, size_t bytes);
+// with no work on p in flight
+void pool_free(int device, void* const* p, size_t count);
+// counts prepared objects (the last one to go empties the pool)
+spmv_status pool_acquire(int device);
+void pool_release(int device);
+// scratch of one call, ordered on its stream; freed with cudaFreeAsync
+cudaError_t work_alloc(int device, void** p, size_t bytes, cudaStream_t s);
+
 // ---- matrix checks on the host side of the ABI ----------------------------------
 spmv_status check_csr_args(const spmv_csr_t* A);
 spmv_status check_choice(const spmv_choice_t* c);
@@ -86,7 +104,6 @@ struct SlicedPlan {
     int* fix = nullptr;          // [n_fix] long rows (list indices) with several segments
     int* seg_fix = nullptr;      // [n_seg] index in fix of the segment's row, -1 for a single segment
     unsigned* ticket = nullptr;  // [n_fix] segments of the row finished in this call (0 between calls)
-    std::vector<uint8_t> seg_several;  // host, [n_seg]: 1 when the segment's row has several
     int n_fix = 0;
     int n_seg = 0;
     // low-precision values (FP32 / BF16), optionally 16-bit column offsets
@@ -97,7 +114,6 @@ struct SlicedPlan {
     uint16_t* off = nullptr;     // [tot] column - rowbase (off16)
     int* rowbase = nullptr;      // [32 n_slices] first column of each position's row (off16)
     float* x32 = nullptr;        // FP32 copy of x (acc32)
-    unsigned* count = nullptr;   // scratch counter
 };
 
 struct spmv_prepared {
@@ -163,8 +179,10 @@ cudaError_t launch_tile_fixup(int64_t n_tiles, int64_t n_rows, const int32_t* ca
 spmv_status prepared_alloc(spmv_prepared* P, void** p, int64_t bytes);
 spmv_status dyn_prepare(spmv_prepared* P, cudaStream_t s);
 cudaError_t launch_dyn(const spmv_prepared* P, const double* x, double* y, cudaStream_t s);
-spmv_status sliced_prepare(spmv_prepared* P, cudaStream_t s);
-cudaError_t launch_sliced(const spmv_prepared* P, const double* x, double* y, cudaStream_t s);
+// check: a validation pass of P->A is on the stream and its verdict is to be read
+spmv_status sliced_prepare(spmv_prepared* P, bool check, cudaStream_t s);
+// dry: the kernels that a call would launch, with nothing to do (loads them)
+cudaError_t launch_sliced(const spmv_prepared* P, const double* x, double* y, cudaStream_t s, bool dry = false);
 cudaError_t launch_latency(const spmv_csr_t& A, int T, const double* x, double* y,
                            int l2_window_bytes, cudaStream_t s);
 cudaError_t launch_compress(const spmv_csr_t& A, int32_t* rowbase, uint16_t* off16,
@@ -184,6 +202,12 @@ cudaError_t launch_compressed(const spmv_csr_t& A, int T, int value_type,
 // 8 column out of range, 16 columns not strictly increasing.
 spmv_status run_feature_pass(const spmv_csr_t* A, int32_t line_bytes,
                              spmv_features_t* features_out, cudaStream_t s);
+
+// The same without the wait: the pass of a matrix with rows is enqueued (the
+// arguments are checked), and once the stream has been waited for, by the
+// same host thread with no other pass in between, the verdict read.
+spmv_status feature_pass_enqueue(const spmv_csr_t* A, int32_t line_bytes, bool features, cudaStream_t s);
+spmv_status feature_pass_verdict(const spmv_csr_t* A);
 
 // Default lanes per row for a mean row length.
 int auto_threads_per_row(double mean_nnz);

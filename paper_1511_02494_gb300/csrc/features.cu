@@ -566,15 +566,13 @@ int auto_threads_per_row(double mean_nnz)
     return T;
 }
 
-spmv_status run_feature_pass(const spmv_csr_t* A, int32_t line_bytes, spmv_features_t* out,
-                             cudaStream_t s)
+spmv_status feature_pass_enqueue(const spmv_csr_t* A, int32_t line_bytes, bool features, cudaStream_t s)
 {
     spmv_status st = check_csr_args(A);
     if (st != SPMV_OK) return st;
     DeviceInfo dev;
     st = current_device(&dev);
     if (st != SPMV_OK) return st;
-    if (line_bytes <= 0) line_bytes = 128;
 
     if (!t_host_acc) {
         void* p = nullptr;
@@ -614,24 +612,26 @@ spmv_status run_feature_pass(const spmv_csr_t* A, int32_t line_bytes, spmv_featu
         w.max_long = (unsigned)max_long;
         w.max_pieces = (unsigned)max_pieces;
         if (e == cudaSuccess) {
-            if (out) k_feature_pass<true><<<blocks, kFT, 0, s>>>(A->n_rows, A->n_cols, A->nnz, A->rowptr, A->colind, line_bytes, w, t_host_acc);
+            if (features) k_feature_pass<true><<<blocks, kFT, 0, s>>>(A->n_rows, A->n_cols, A->nnz, A->rowptr, A->colind, line_bytes, w, t_host_acc);
             else k_feature_pass<false><<<blocks, kFT, 0, s>>>(A->n_rows, A->n_cols, A->nnz, A->rowptr, A->colind, line_bytes, w, t_host_acc);
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) {
-            if (out) k_feature_long<true><<<lblocks, kFT, 0, s>>>(A->n_cols, A->nnz, A->colind, line_bytes, w, t_host_acc);
+            if (features) k_feature_long<true><<<lblocks, kFT, 0, s>>>(A->n_cols, A->nnz, A->colind, line_bytes, w, t_host_acc);
             else k_feature_long<false><<<lblocks, kFT, 0, s>>>(A->n_cols, A->nnz, A->colind, line_bytes, w, t_host_acc);
             e = cudaGetLastError();
         }
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return cuda_fail(e, "feature pass");
-        t_scratch_clean = true;
     } else {
         memset(t_host_acc, 0, sizeof(FeatAcc));
     }
+    return SPMV_OK;
+}
 
-    const FeatAcc& h = *t_host_acc;
-    u64 err = h.err;
+spmv_status feature_pass_verdict(const spmv_csr_t* A)
+{
+    t_scratch_clean = true;
+    u64 err = t_host_acc->err;
     if (A->n_rows == 0 && A->nnz != 0) err |= 2;
     if (err) {
         std::string m = "invalid CSR:";
@@ -642,6 +642,20 @@ spmv_status run_feature_pass(const spmv_csr_t* A, int32_t line_bytes, spmv_featu
         if (err & 16) m += " columns not strictly increasing within a row;";
         return fail(SPMV_ERR_INVALID_CSR, m);
     }
+    return SPMV_OK;
+}
+
+spmv_status run_feature_pass(const spmv_csr_t* A, int32_t line_bytes, spmv_features_t* out,
+                             cudaStream_t s)
+{
+    if (line_bytes <= 0) line_bytes = 128;
+    spmv_status st = feature_pass_enqueue(A, line_bytes, out != nullptr, s);
+    if (st != SPMV_OK) return st;
+    SPMV_CUDA_TRY(cudaStreamSynchronize(s));
+    if ((st = feature_pass_verdict(A)) != SPMV_OK) return st;
+    const FeatAcc& h = *t_host_acc;
+    DeviceInfo dev;
+    if ((st = current_device(&dev)) != SPMV_OK) return st;
     if (!out) return SPMV_OK;
 
     spmv_features_t f = {};

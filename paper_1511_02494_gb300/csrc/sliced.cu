@@ -22,6 +22,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <utility>
 #include <vector>
 
 #include "common.cuh"
@@ -33,109 +34,431 @@ namespace {
 
 using namespace dev;
 constexpr int kSB = 256;       // threads per block: 8 slices
-constexpr int kSortT = 1024;   // threads of the window sort
 
-__global__ void k_sl_rowlen_identity(int64_t n_rows, const int* __restrict__ rp, int cap,
-                                     int* __restrict__ rowlen, unsigned* __restrict__ n_long)
-{
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n_rows;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const int len = rp[p + 1] - rp[p];
-        if (len > cap) {
-            rowlen[p] = -1;
-            atomicAdd(n_long, 1u);
-        } else {
-            rowlen[p] = len;
+// ---- layout (prepare) --------------------------------------------------------
+// What the layout kernels find out about the matrix; the scan writes it to
+// page-locked host memory, so that a layout costs one wait and no copy.
+struct SlStats {
+    unsigned long long slots;   // sum of 32 x slice length: padding by unequal rows only
+    unsigned long long tot;     // element slots (slices rounded up to `vec` elements a row)
+    unsigned n_long, n_seg, n_fix;
+    int longest;                // longest slice
+    unsigned shortest_c;        // maximum of ~length over the rows
+    unsigned reach;             // for the column-width questions
+};
+// The slices are cut into at most kTiles tiles of equal length (whole sort
+// windows); per tile the element slots and the long rows, their segments and
+// those with several segments.  A tile's place is the sum of the tiles before
+// it, which every block of the next kernel forms for itself: no block waits
+// for another.
+constexpr int kTiles = 1024;
+struct SlTile {
+    unsigned long long len;
+    unsigned n_long, n_seg, n_fix, pad;
+};
+struct SlScratch {
+    SlStats stats;
+    SlTile tile[kTiles];
+};
+
+// a thread's share of a tile
+struct TileAcc {
+    unsigned long long len = 0, slots = 0;
+    unsigned n_long = 0, n_seg = 0, n_fix = 0, shortest_c = 0;
+    int longest = 0;
+
+    // one row: its length in the slices, -1 when it is long
+    __device__ __forceinline__ int row(int n, int cap) {
+        if (n > cap) {
+            ++n_long;
+            n_seg += (unsigned)(n + kSlicedSeg - 1) / kSlicedSeg;
+            n_fix += n > kSlicedSeg;
+            n = -1;
+        }
+        shortest_c = max(shortest_c, ~(unsigned)n);
+        return n;
+    }
+    // one slice (called by one lane)
+    __device__ __forceinline__ void slice(int m, int vec) {
+        len += 32ull * (unsigned)((m + vec - 1) / vec * vec);
+        slots += 32ull * (unsigned)m;
+        longest = max(longest, m);
+    }
+    // adds the block's share to its tile and to the totals
+    __device__ __forceinline__ void flush(SlScratch* w, int64_t tile) {
+        __shared__ SlTile t;
+        __shared__ SlStats g;
+        if (threadIdx.x == 0) { t = SlTile{}; g = SlStats{}; }
+        __syncthreads();
+        const unsigned nl = __reduce_add_sync(FULL, n_long), ns = __reduce_add_sync(FULL, n_seg),
+                       nf = __reduce_add_sync(FULL, n_fix), sc = __reduce_max_sync(FULL, shortest_c);
+        const int lo = __reduce_max_sync(FULL, longest);
+        unsigned long long l = len, q = slots;
+        for (int o = 16; o > 0; o >>= 1) {
+            l += __shfl_xor_sync(FULL, l, o);
+            q += __shfl_xor_sync(FULL, q, o);
+        }
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd(&t.len, l);
+            atomicAdd(&g.slots, q);
+            atomicMax(&g.longest, lo);
+            atomicMax(&g.shortest_c, sc);
+            if (nl) { atomicAdd(&t.n_long, nl); atomicAdd(&t.n_seg, ns); atomicAdd(&t.n_fix, nf); }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            SlTile* T = w->tile + tile;
+            SlStats* S = &w->stats;
+            atomicAdd(&T->len, t.len);
+            atomicAdd(&S->slots, g.slots);
+            atomicMax(&S->longest, g.longest);
+            atomicMax(&S->shortest_c, g.shortest_c);
+            if (t.n_long) {
+                atomicAdd(&T->n_long, t.n_long); atomicAdd(&T->n_seg, t.n_seg); atomicAdd(&T->n_fix, t.n_fix);
+                atomicAdd(&S->n_long, t.n_long); atomicAdd(&S->n_seg, t.n_seg); atomicAdd(&S->n_fix, t.n_fix);
+            }
         }
     }
+};
+
+// Rows in order: row lengths and slice lengths, a block per tile, a warp per
+// slice, four slices' row pointers in flight.
+__global__ void __launch_bounds__(kSB)
+k_sl_layout(int64_t n_rows, int64_t n_slices, const int* __restrict__ rp, int cap, int vec, int64_t tile_slices,
+            int* __restrict__ rowlen, int* __restrict__ slice_len, SlScratch* __restrict__ w)
+{
+    constexpr int U = 4;
+    const int lane = threadIdx.x & 31;
+    const int64_t t0 = blockIdx.x * tile_slices, t1 = min(n_slices, t0 + tile_slices);
+    TileAcc acc;
+    for (int64_t s0 = t0 + (threadIdx.x >> 5) * U; s0 < t1; s0 += (kSB / 32) * U) {
+        int b[U], e[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t row = (s0 + u) * 32 + lane;
+            const bool in = s0 + u < t1 && row < n_rows;
+            b[u] = in ? rp[row] : 0;
+            e[u] = in ? rp[row + 1] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (s0 + u >= t1) break;  // whole warps
+            const int64_t p = (s0 + u) * 32 + lane;
+            const int n = p < n_rows ? acc.row(e[u] - b[u], cap) : -1;
+            rowlen[p] = n;
+            const int m = __reduce_max_sync(FULL, max(n, 0));
+            if (lane == 0) {
+                slice_len[s0 + u] = m;
+                acc.slice(m, vec);
+            }
+        }
+    }
+    acc.flush(w, blockIdx.x);
 }
 
-// One CTA per window of sigma rows (sigma a power of two, 32..4096): bitonic
-// sort of keys (0xFFFFFFFF - key length) << 32 | index in window, so rows come
-// out by key length descending, ties by row index ascending; slots past the
-// last row carry the largest key and end last.
-__global__ void __launch_bounds__(kSortT)
-k_sl_sort(int64_t n_rows, const int* __restrict__ rp, int sigma, int cap, int* __restrict__ perm,
-          int* __restrict__ rowlen, unsigned* __restrict__ n_long)
+// Rows sorted by length inside windows of sigma rows (a power of two,
+// 32..4096), longest first, ties by row index, long rows as of length 0: a
+// block per window, four rows per thread.  A stable radix sort of (longest -
+// length, index) in 5-bit digits over only the bits that the window's lengths
+// differ in -- one pass for a stencil's rows, two for a cap of 32 -- ranks by
+// warp votes (a warp owns 128 consecutive places) and a scan over (digit,
+// warp).  A bitonic sort of 64-bit keys, 78 steps with a block barrier each,
+// took 70 us for 1M rows in windows of 4096; this takes 17.6.
+constexpr int kSortItems = 4;
+constexpr int kSortMax = 4096;
+__global__ void __launch_bounds__(kSortMax / kSortItems)
+k_sl_sort(int64_t n_rows, int64_t n_slices, const int* __restrict__ rp, int sigma, int cap, int vec,
+          int64_t tile_slices, int* __restrict__ perm, int* __restrict__ rowlen, int* __restrict__ slice_len,
+          SlScratch* __restrict__ w)
 {
-    extern __shared__ unsigned long long keys[];
+    __shared__ unsigned buf[kSortMax];
+    __shared__ unsigned hist[kSortMax / kSortItems / 32][32];
+    __shared__ unsigned warp_sum[32];
+    __shared__ unsigned s_max, s_min;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     const int64_t w0 = (int64_t)blockIdx.x * sigma;
-    for (int i = threadIdx.x; i < sigma; i += kSortT) {
-        const int64_t r = w0 + i;
-        unsigned long long key = ~0ull;
-        if (r < n_rows) {
-            const int len = rp[r + 1] - rp[r];
-            const unsigned klen = len > cap ? 0u : (unsigned)len;
-            key = ((unsigned long long)(0xFFFFFFFFu - klen) << 32) | (unsigned)i;
+    TileAcc acc;
+    if (threadIdx.x == 0) { s_max = 0; s_min = 0xffffffffu; }
+    __syncthreads();
+    // place i of the window: warp * 128 + 32 u + lane
+    unsigned klen[kSortItems], lo = 0xffffffffu, hi = 0;
+#pragma unroll
+    for (int u = 0; u < kSortItems; ++u) {
+        const int i = warp * 128 + u * 32 + lane;
+        klen[u] = 0xffffffffu;  // no row
+        if (i < sigma && w0 + i < n_rows) {
+            const int n = acc.row(rp[w0 + i + 1] - rp[w0 + i], cap);
+            klen[u] = (unsigned)max(n, 0);
+            lo = min(lo, klen[u]);
+            hi = max(hi, klen[u]);
         }
-        keys[i] = key;
+    }
+    lo = __reduce_min_sync(FULL, lo);
+    hi = __reduce_max_sync(FULL, hi);
+    if (lane == 0) { atomicMin(&s_min, lo); atomicMax(&s_max, hi); }
+    __syncthreads();
+    const unsigned longest = s_max, none = longest - min(s_min, longest) + 1;  // places without a row sort last
+    const int bits = 32 - __clz((int)none);
+    unsigned val[kSortItems];  // key << 12 | index in the window
+#pragma unroll
+    for (int u = 0; u < kSortItems; ++u) {
+        const int i = warp * 128 + u * 32 + lane;
+        val[u] = ((klen[u] == 0xffffffffu ? none : longest - klen[u]) << 12) | (unsigned)i;
+    }
+    for (int shift = 12; shift < 12 + bits; shift += 5) {
+        hist[warp][lane] = 0;
+        __syncwarp();
+        unsigned rank[kSortItems];
+#pragma unroll
+        for (int u = 0; u < kSortItems; ++u) {
+            const bool in = warp * 128 + u * 32 < sigma;  // whole warps
+            if (in) {
+                const unsigned digit = (val[u] >> shift) & 31u;
+                const unsigned peers = __match_any_sync(FULL, digit);
+                const unsigned before = hist[warp][digit];
+                rank[u] = before + __popc(peers & ((1u << lane) - 1u));
+                __syncwarp();
+                if ((peers & ((1u << lane) - 1u)) == 0) hist[warp][digit] = before + __popc(peers);
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+        // exclusive scan over (digit, warp), an entry per thread
+        const int e_digit = threadIdx.x / n_warps, e_warp = threadIdx.x % n_warps;
+        const unsigned own = hist[e_warp][e_digit];
+        unsigned incl = own;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned t = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) warp_sum[warp] = incl;
+        __syncthreads();
+        unsigned base = 0;
+        for (int k = 0; k < warp; ++k) base += warp_sum[k];
+        hist[e_warp][e_digit] = base + incl - own;
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kSortItems; ++u)
+            if (warp * 128 + u * 32 < sigma) buf[hist[warp][(val[u] >> shift) & 31u] + rank[u]] = val[u];
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kSortItems; ++u)
+            if (warp * 128 + u * 32 < sigma) val[u] = buf[warp * 128 + u * 32 + lane];
+    }
+#pragma unroll
+    for (int u = 0; u < kSortItems; ++u) {
+        const int i = warp * 128 + u * 32;
+        const int64_t p = w0 + i + lane;
+        if (i >= sigma || p - lane >= 32 * n_slices) continue;  // whole warps
+        int n = -1;
+        if (p < n_rows) {
+            const int64_t r = w0 + (val[u] & 4095u);
+            n = (int)(longest - (val[u] >> 12));
+            if (n == 0 && rp[r + 1] - rp[r] > cap) n = -1;
+            perm[p] = (int)r;
+        }
+        rowlen[p] = n;
+        const int m = __reduce_max_sync(FULL, max(n, 0));
+        if (lane == 0) {
+            slice_len[p / 32] = m;
+            acc.slice(m, vec);
+        }
+    }
+    acc.flush(w, w0 / 32 / tile_slices);
+}
+
+// sums over the tiles before this block's: element slots, long rows,
+// segments, rows with several segments (valid in every thread)
+__device__ __forceinline__ SlTile tiles_before(const SlScratch* __restrict__ w)
+{
+    __shared__ SlTile t;
+    if (threadIdx.x == 0) t = SlTile{};
+    __syncthreads();
+    unsigned long long l = 0;
+    unsigned nl = 0, ns = 0, nf = 0;
+    for (int k = threadIdx.x; k < (int)blockIdx.x; k += kSB) {
+        l += w->tile[k].len;
+        nl += w->tile[k].n_long;
+        ns += w->tile[k].n_seg;
+        nf += w->tile[k].n_fix;
+    }
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(FULL, l, o);
+    nl = __reduce_add_sync(FULL, nl);
+    ns = __reduce_add_sync(FULL, ns);
+    nf = __reduce_add_sync(FULL, nf);
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&t.len, l);
+        atomicAdd(&t.n_long, nl);
+        atomicAdd(&t.n_seg, ns);
+        atomicAdd(&t.n_fix, nf);
     }
     __syncthreads();
-    for (int k = 2; k <= sigma; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < sigma; i += kSortT) {
-                const int ixj = i ^ j;
-                if (ixj > i) {
-                    const unsigned long long a = keys[i], b = keys[ixj];
-                    const bool up = (i & k) == 0;
-                    if ((a > b) == up) {
-                        keys[i] = b;
-                        keys[ixj] = a;
-                    }
-                }
-            }
-            __syncthreads();
-        }
+    return t;
+}
+
+// block-wide exclusive scan of one value per thread (below 2^31 in total)
+__device__ __forceinline__ unsigned block_scan(unsigned v, unsigned* total)
+{
+    __shared__ unsigned part[kSB / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned incl = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned t = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += t;
     }
-    for (int i = threadIdx.x; i < sigma; i += kSortT) {
-        const int64_t p = w0 + i;
-        if (p >= n_rows) continue;
-        const int r = (int)(w0 + (int64_t)(keys[i] & 0xFFFFFFFFull));
-        perm[p] = r;
-        const int len = rp[r + 1] - rp[r];
-        if (len > cap) {
-            rowlen[p] = -1;
-            atomicAdd(n_long, 1u);
-        } else {
-            rowlen[p] = len;
-        }
+    __syncthreads();  // part may still be read from the scan before
+    if (lane == 31) part[warp] = incl;
+    __syncthreads();
+    unsigned base = 0, all = 0;
+    for (int k = 0; k < kSB / 32; ++k) {
+        if (k < warp) base += part[k];
+        all += part[k];
+    }
+    *total = all;
+    return base + incl - v;
+}
+
+// slice starts from the slice lengths, a block per tile; the last block also
+// hands the totals to the host
+__global__ void __launch_bounds__(kSB)
+k_sl_scan(int64_t n_slices, int64_t tile_slices, int vec, const int* __restrict__ slice_len,
+          int64_t* __restrict__ slice_ptr, const SlScratch* __restrict__ w, SlStats* __restrict__ host)
+{
+    int64_t at = (int64_t)tiles_before(w).len;
+    const int64_t t0 = blockIdx.x * tile_slices, t1 = min(n_slices, t0 + tile_slices);
+    for (int64_t s0 = t0; s0 < t1; s0 += kSB) {
+        const int64_t s = s0 + threadIdx.x;
+        const unsigned n = s < t1 ? 32u * (unsigned)((slice_len[s] + vec - 1) / vec * vec) : 0u;
+        unsigned all;
+        const unsigned before = block_scan(n, &all);
+        if (s < t1) slice_ptr[s] = at + before;
+        at += all;
+    }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+        slice_ptr[n_slices] = at;
+        SlStats t = w->stats;
+        t.tot = (unsigned long long)at;
+        *host = t;
     }
 }
 
-// slice_len[s] = max(0, max over the slice's 32 positions of rowlen)
-__global__ void k_sl_slice_len(int64_t n_slices, const int* __restrict__ rowlen,
-                               int* __restrict__ slice_len)
+// Contents of the slices.  A warp per slice reads its rows' elements with T
+// lanes per row (T the power of two that covers the chunk's longest row, at
+// most 8), so that a load instruction covers runs of the CSR arrays, straight
+// into shared memory (cp.async, no registers held), turned around there (rows
+// of 33: no bank conflicts), and writes the chunk column-major, padding
+// included: every slot is written, so nothing is zeroed beforehand.  `Out`
+// writes the elements of one lane's row in row order, `vec` at a time.
+// Bound by HBM: 108 us for a 100^3 27-point stencil (26.5 M nonzeros, 5.9
+// TB/s).  A lane per row, as the SpMV walks them, reads 32 places per
+// instruction; that and the memsets took 132 + 57 us.  Chunks of 16 or 32
+// elements leave fewer blocks resident (125 us either way), 40 registers a
+// thread for 48 warps spill (114 us), and warps striding over the slices with
+// the next header loaded ahead are slower than many short blocks (138 us).
+constexpr int kFillK = 8, kFillWarps = 4;
+template <int B>
+__device__ __forceinline__ void cp_async(void* dst, const void* src)
 {
-    const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (s >= n_slices) return;
-    const int lane = threadIdx.x & 31;
-    const int m = __reduce_max_sync(FULL, max(rowlen[s * 32 + lane], 0));
-    if (lane == 0) slice_len[s] = m;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;"
+                 :: "r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "n"(B) : "memory");
 }
-
-// column-major contents of each slice (padding was zeroed beforehand)
-// FP64 contents: CT int stores the columns, int16_t / int8_t the column
-// minus the row index (the range was checked by k_sl_reach)
-template <typename CT>
-__global__ void k_sl_fill(int64_t n_slices, const int* __restrict__ rp, const int* __restrict__ ci,
-                          const double* __restrict__ v, const int* __restrict__ perm,
-                          const int* __restrict__ rowlen, const int64_t* __restrict__ slice_ptr,
-                          CT* __restrict__ col, double* __restrict__ val)
+template <typename Out>
+__global__ void __launch_bounds__(32 * kFillWarps)
+k_sl_fill(int64_t n_slices, const int* __restrict__ rp, const int* __restrict__ ci, const double* __restrict__ v,
+          const int* __restrict__ perm, const int* __restrict__ rowlen, const int* __restrict__ slice_len,
+          const int64_t* __restrict__ slice_ptr, Out out)
 {
-    const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (s >= n_slices) return;
+    __shared__ int s_col[kFillWarps][kFillK * 33];
+    __shared__ double s_val[kFillWarps][kFillK * 33];
     const int lane = threadIdx.x & 31;
+    int* tc = s_col[threadIdx.x >> 5];
+    double* tv = s_val[threadIdx.x >> 5];
+    const int64_t s = (int64_t)blockIdx.x * kFillWarps + (threadIdx.x >> 5);
+    if (s >= n_slices) return;  // whole warps
     const int64_t p = s * 32 + lane;
-    const int len = rowlen[p];
-    if (len <= 0) return;
-    const int r = perm ? perm[p] : (int)p;
-    const int64_t b = rp[r];
-    const int64_t q0 = slice_ptr[s] + lane;
-    for (int k = 0; k < len; ++k) {
-        col[q0 + (int64_t)k * 32] = sizeof(CT) == 4 ? (CT)ci[b + k] : (CT)(ci[b + k] - r);
-        val[q0 + (int64_t)k * 32] = v[b + k];
+    const int len = max(rowlen[p], 0);
+    const int r = len > 0 ? (perm ? perm[p] : (int)p) : 0;
+    const int b = len > 0 ? rp[r] : 0;
+    const int L = slice_len[s], Lp = (L + Out::vec - 1) / Out::vec * Out::vec;
+    const int64_t q0 = slice_ptr[s];
+    typename Out::Row row;
+    out.begin(row, p, r, len > 0 ? ci[b] : 0, len > 0);
+    for (int kc = 0; kc < Lp; kc += kFillK) {
+        const int width = min(kFillK, L - kc);
+        const int lg = width > 1 ? 32 - __clz(width - 1) : 0, T = 1 << lg;
+        const int sub = lane >> lg, k = lane & (T - 1);
+#pragma unroll 4
+        for (int i = 0; i < T; ++i) {
+            const int row_of = i * (32 >> lg) + sub;
+            const int rb = __shfl_sync(FULL, b, row_of), rl = __shfl_sync(FULL, len, row_of);
+            if (kc + k < rl) {
+                const int at = k * 33 + row_of;
+                cp_async<4>(tc + at, ci + (int64_t)rb + kc + k);
+                cp_async<8>(tv + at, v + (int64_t)rb + kc + k);
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+        for (int k0 = 0; k0 < kFillK && kc + k0 < Lp; k0 += Out::vec) {
+            int c[Out::vec];
+            double a[Out::vec];
+            bool ok[Out::vec];
+#pragma unroll
+            for (int e = 0; e < Out::vec; ++e) {
+                ok[e] = kc + k0 + e < len;
+                c[e] = ok[e] ? tc[(k0 + e) * 33 + lane] : 0;
+                a[e] = ok[e] ? tv[(k0 + e) * 33 + lane] : 0.0;
+            }
+            out.put(row, q0 + (int64_t)(kc + k0) * 32 + Out::vec * lane, c, a, ok);
+        }
+        __syncwarp();
     }
 }
+
+// FP64 values; CT int stores the columns, int16_t / int8_t the column minus
+// the row index (the range was checked by k_sl_reach)
+template <typename CT>
+struct OutF64 {
+    static constexpr int vec = 1;
+    CT* col;
+    double* val;
+    struct Row { int r; };
+    __device__ __forceinline__ void begin(Row& w, int64_t, int r, int, bool) const { w.r = r; }
+    __device__ __forceinline__ void put(Row& w, int64_t q, const int* c, const double* a, const bool* ok) const
+    {
+        col[q] = sizeof(CT) == 4 ? (CT)c[0] : (CT)(ok[0] ? c[0] - w.r : 0);
+        val[q] = a[0];
+    }
+};
+
+// FP64 values with coded columns: MODE 1 deltas and row bases, MODE 2 panel
+// offsets and steps
+template <int MODE, typename DT>
+struct OutCoded {
+    static constexpr int vec = 1;
+    DT* cs;
+    uint8_t* step;
+    int* rowbase;
+    double* val;
+    struct Row { int prev; };
+    __device__ __forceinline__ void begin(Row& w, int64_t p, int, int first, bool has) const
+    {
+        w.prev = MODE == 1 && has ? first : 0;
+        if (MODE == 1) rowbase[p] = has ? first : 0;
+    }
+    __device__ __forceinline__ void put(Row& w, int64_t q, const int* c, const double* a, const bool* ok) const
+    {
+        const int x = ok[0] ? c[0] : w.prev;
+        if (MODE == 1) {
+            cs[q] = (DT)(x - w.prev);
+        } else {
+            cs[q] = ok[0] ? (DT)(x & 0xffff) : (DT)0;
+            step[q] = (uint8_t)((x >> 16) - (w.prev >> 16));
+        }
+        val[q] = a[0];
+        w.prev = x;
+    }
+};
 
 // largest |column - row| over the rows in the slices (the first or the last
 // column of a row, its columns being increasing)
@@ -177,70 +500,6 @@ __global__ void k_sl_code_reach(int64_t n_slices, const int* __restrict__ rp, co
         prev = c;
     }
     atomicMax(reach, m);
-}
-
-// coded contents (padding was zeroed beforehand): MODE 1 deltas and row
-// bases, MODE 2 panel offsets and steps; a warp per slice, a lane per row
-template <int MODE, typename DT>
-__global__ void k_sl_fill_coded(int64_t n_slices, const int* __restrict__ rp, const int* __restrict__ ci,
-                                const double* __restrict__ v, const int* __restrict__ perm,
-                                const int* __restrict__ rowlen, const int64_t* __restrict__ slice_ptr,
-                                DT* __restrict__ cs, uint8_t* __restrict__ step, int* __restrict__ rowbase,
-                                double* __restrict__ val)
-{
-    const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (s >= n_slices) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t p = s * 32 + lane;
-    const int len = rowlen[p];
-    if (len <= 0) return;
-    const int64_t b = rp[perm ? perm[p] : (int)p];
-    const int64_t q0 = slice_ptr[s] + lane;
-    if (MODE == 1) rowbase[p] = ci[b];
-    int prev = MODE == 1 ? ci[b] : 0;
-    for (int k = 0; k < len; ++k) {
-        const int c = ci[b + k];
-        const int64_t q = q0 + (int64_t)k * 32;
-        if (MODE == 1) {
-            cs[q] = (DT)(c - prev);
-        } else {
-            cs[q] = (DT)(c & 0xffff);
-            step[q] = (uint8_t)((c >> 16) - (prev >> 16));
-        }
-        prev = c;
-        val[q] = v[b + k];
-    }
-}
-
-// the shortest row length over the positions holding rows (min into *out,
-// which starts at INT_MAX)
-__global__ void k_sl_min_len(int64_t n_rows, const int* __restrict__ rowlen, int* __restrict__ out)
-{
-    int m = 0x7fffffff;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n_rows;
-         p += (int64_t)gridDim.x * blockDim.x)
-        m = min(m, rowlen[p]);
-    m = __reduce_min_sync(FULL, m);
-    if ((threadIdx.x & 31) == 0) atomicMin(out, m);
-}
-
-// rows longer than cap, appended with one atomic per warp
-__global__ void k_sl_long_list(int64_t n_rows, const int* __restrict__ rp, int cap,
-                               int* __restrict__ list, unsigned* __restrict__ count)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t n_iter = (n_rows + stride - 1) / stride;
-    for (int64_t it = 0; it < n_iter; ++it) {
-        const int64_t i = it * stride + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-        const bool is_long = i < n_rows && rp[i + 1] - rp[i] > cap;
-        const unsigned m = __ballot_sync(FULL, is_long);
-        if (m == 0) continue;
-        unsigned base = 0;
-        if (lane == 0) base = atomicAdd(count, (unsigned)__popc(m));
-        base = __shfl_sync(FULL, base, 0);
-        if (is_long) list[base + __popc(m & ((1u << lane) - 1u))] = (int)i;
-    }
 }
 
 // 8 blocks of 256 per SM (32 registers): measured faster than the 40-register
@@ -318,30 +577,49 @@ k_sliced_multi(int64_t n_slices, const int* __restrict__ rowlen, const int* __re
                                y);
 }
 
-__global__ void k_sl_row_lengths(int n, const int* __restrict__ list, const int* __restrict__ rp,
-                                 int* __restrict__ len)
+// Long rows in ascending order, split into segments of kSlicedSeg nonzeros:
+// the list, its segment offsets, each segment's CSR begin and end, its row
+// when it is the row's only one (that segment writes y itself; else -1), and
+// the rows with several segments with their tickets.  A block per tile.
+struct LongTables {
+    int* rows; int* seg_off; int64_t* seg_be; int* seg_row; int* seg_fix; int* fix; unsigned* ticket;
+};
+__global__ void __launch_bounds__(kSB)
+k_sl_long_tables(int64_t n_rows, const int* __restrict__ rp, int cap, int64_t tile_slices,
+                 const SlScratch* __restrict__ w, int n_long, LongTables o)
 {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q < n) len[q] = rp[list[q] + 1] - rp[list[q]];
-}
-
-// Long rows are split into segments of kSlicedSeg nonzeros; seg_be holds
-// each segment's CSR begin and end, seg_row the row of a segment that is its
-// row's only one (that segment writes y itself) and -1 otherwise.
-__global__ void k_sl_seg_table(int n_long, const int* __restrict__ list, const int* __restrict__ seg_off,
-                               const int* __restrict__ rp, int64_t* __restrict__ seg_be,
-                               int* __restrict__ seg_row)
-{
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n_long) return;
-    const int r = list[q];
-    const int64_t b0 = rp[r], e0 = rp[r + 1];
-    const bool single = seg_off[q + 1] - seg_off[q] == 1;
-    for (int j = seg_off[q]; j < seg_off[q + 1]; ++j) {
-        const int64_t b = b0 + (int64_t)(j - seg_off[q]) * kSlicedSeg;
-        seg_be[2 * (int64_t)j] = b;
-        seg_be[2 * (int64_t)j + 1] = min(e0, b + kSlicedSeg);
-        seg_row[j] = single ? r : -1;
+    if (w->tile[blockIdx.x].n_long == 0) return;
+    const SlTile at = tiles_before(w);
+    unsigned q0 = at.n_long, j0 = at.n_seg, f0 = at.n_fix;
+    const int64_t r0 = blockIdx.x * tile_slices * 32, r1 = min(n_rows, r0 + tile_slices * 32);
+    for (int64_t base = r0; base < r1; base += kSB) {
+        const int64_t r = base + threadIdx.x;
+        const int b = r < r1 ? rp[r] : 0, e = r < r1 ? rp[r + 1] : 0;
+        const bool is_long = e - b > cap, several = is_long && e - b > kSlicedSeg;
+        if (!__syncthreads_or(is_long)) continue;
+        const unsigned segs = is_long ? (unsigned)(e - b + kSlicedSeg - 1) / kSlicedSeg : 0u;
+        unsigned nq, nj, nf;
+        const unsigned q = q0 + block_scan(is_long, &nq), j = j0 + block_scan(segs, &nj),
+                       f = f0 + block_scan(several, &nf);
+        if (is_long) {
+            o.rows[q] = (int)r;
+            o.seg_off[q] = (int)j;
+            if ((int)q == n_long - 1) o.seg_off[n_long] = (int)(j + segs);
+            if (several) {
+                o.fix[f] = (int)q;
+                o.ticket[f] = 0u;
+            }
+            for (unsigned i = 0; i < segs; ++i) {
+                const int64_t sb = b + (int64_t)i * kSlicedSeg;
+                o.seg_be[2 * (int64_t)(j + i)] = sb;
+                o.seg_be[2 * (int64_t)(j + i) + 1] = min((int64_t)e, sb + kSlicedSeg);
+                o.seg_row[j + i] = several ? -1 : (int)r;
+                o.seg_fix[j + i] = several ? (int)f : -1;
+            }
+        }
+        q0 += nq;
+        j0 += nj;
+        f0 += nf;
     }
 }
 
@@ -446,43 +724,56 @@ __device__ __forceinline__ float widen32(__nv_bfloat16 a) { return __bfloat162fl
 
 __global__ void k_sl_span(int64_t n_slices, const int* __restrict__ rp, const int* __restrict__ ci,
                           const int* __restrict__ perm, const int* __restrict__ rowlen,
-                          int* __restrict__ span)
+                          unsigned* __restrict__ span)
 {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= 32 * n_slices) return;
     const int len = rowlen[p];
     if (len <= 0) return;
     const int64_t b = rp[perm ? perm[p] : (int)p];
-    atomicMax(span, ci[b + len - 1] - ci[b]);
+    atomicMax(span, (unsigned)(ci[b + len - 1] - ci[b]));
 }
 
 // low-precision contents, four elements of a row side by side (element k
 // at slice_ptr[s] + 128 (k / 4) + 4 l + k % 4); OFF16: offsets from the
 // row's first column (rowbase per position), else 32-bit columns
-template <typename VT, bool OFF16>
-__global__ void k_sl_fill_lp(int64_t n_slices, const int* __restrict__ rp, const int* __restrict__ ci,
-                             const double* __restrict__ v, const int* __restrict__ perm,
-                             const int* __restrict__ rowlen, const int64_t* __restrict__ slice_ptr,
-                             int* __restrict__ col, uint16_t* __restrict__ off,
-                             int* __restrict__ rowbase, VT* __restrict__ val)
+__device__ __forceinline__ void store4(float* p, const float* a) { *reinterpret_cast<float4*>(p) = make_float4(a[0], a[1], a[2], a[3]); }
+__device__ __forceinline__ void store4(__nv_bfloat16* p, const __nv_bfloat16* a)
 {
-    const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (s >= n_slices) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t p = s * 32 + lane;
-    const int len = rowlen[p];
-    if (len <= 0) return;
-    const int64_t b = rp[perm ? perm[p] : (int)p];
-    const int64_t q0 = slice_ptr[s] + 4 * lane;
-    const int first = ci[b];
-    if (OFF16) rowbase[p] = first;
-    for (int k = 0; k < len; ++k) {
-        const int64_t q = q0 + (int64_t)(k >> 2) * 128 + (k & 3);
-        if (OFF16) off[q] = (uint16_t)(ci[b + k] - first);
-        else col[q] = ci[b + k];
-        val[q] = round_to(v[b + k], (VT*)nullptr);
-    }
+    uint2 w;
+    w.x = __bfloat16_as_ushort(a[0]) | ((unsigned)__bfloat16_as_ushort(a[1]) << 16);
+    w.y = __bfloat16_as_ushort(a[2]) | ((unsigned)__bfloat16_as_ushort(a[3]) << 16);
+    *reinterpret_cast<uint2*>(p) = w;
 }
+template <typename VT, bool OFF16>
+struct OutLp {
+    static constexpr int vec = 4;
+    int* col;
+    uint16_t* off;
+    int* rowbase;
+    VT* val;
+    struct Row { int first; };
+    __device__ __forceinline__ void begin(Row& w, int64_t p, int, int first, bool has) const
+    {
+        w.first = has ? first : 0;
+        if (OFF16) rowbase[p] = w.first;
+    }
+    __device__ __forceinline__ void put(Row& w, int64_t q, const int* c, const double* a, const bool* ok) const
+    {
+        VT x[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[e] = round_to(a[e], (VT*)nullptr);
+        store4(val + q, x);
+        if (OFF16) {
+            unsigned o[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[e] = ok[e] ? (unsigned)(c[e] - w.first) & 0xffffu : 0u;
+            *reinterpret_cast<uint2*>(off + q) = make_uint2(o[0] | (o[1] << 16), o[2] | (o[3] << 16));
+        } else {
+            *reinterpret_cast<int4*>(col + q) = make_int4(c[0], c[1], c[2], c[3]);
+        }
+    }
+};
 
 __global__ void k_sl_x_to_f32(int64_t n, const double* __restrict__ x, float* __restrict__ x32)
 {
@@ -564,57 +855,86 @@ unsigned grid_of(int64_t threads, int64_t cap_blocks)
 
 }  // namespace
 
-spmv_status sliced_prepare(spmv_prepared* P, cudaStream_t s)
+namespace {
+
+// page-locked buffer the layout's totals are written to, one per host thread
+thread_local SlStats* t_host_stats = nullptr;
+
+// Places arrays in one allocation, each on a 256-byte boundary.
+struct Arena {
+    int64_t bytes = 0;
+    std::vector<std::pair<void**, int64_t>> at;
+    template <typename T>
+    void add(T** p, int64_t count)
+    {
+        at.push_back({reinterpret_cast<void**>(p), bytes});
+        bytes += ((int64_t)sizeof(T) * std::max<int64_t>(count, 1) + 255) / 256 * 256;
+    }
+    spmv_status allocate(spmv_prepared* P)
+    {
+        void* base = nullptr;
+        spmv_status st = prepared_alloc(P, &base, bytes);
+        if (st != SPMV_OK) return st;
+        for (auto& a : at) *a.first = static_cast<char*>(base) + a.second;
+        return SPMV_OK;
+    }
+};
+
+// check: the matrix's validation pass is on the stream; its verdict is read
+// at the first wait (what runs before that reads row pointers only, each as
+// a number)
+spmv_status sliced_build(spmv_prepared* P, SlScratch* w, bool check, cudaStream_t s)
 {
     const spmv_csr_t& A = P->A;
     SlicedPlan& d = P->sl;
+    SlStats* const host = t_host_stats;
     int cap = P->c.items_per_warp > 0 ? P->c.items_per_warp : kSlicedCap;
     d.n_slices = (A.n_rows + 31) / 32;
     const int64_t n_pos = 32 * d.n_slices;
+    const bool f64 = P->c.value_type == SPMV_VAL_F64;
+    // FP64 values: one element per slot row; FP32/BF16: four side by side
+    d.vec = f64 ? 1 : 4;
     spmv_status st;
-    if ((st = prepared_alloc(P, reinterpret_cast<void**>(&d.rowlen), 4 * std::max<int64_t>(n_pos, 1))) != SPMV_OK ||
-        (st = prepared_alloc(P, reinterpret_cast<void**>(&d.slice_len), 4 * std::max<int64_t>(d.n_slices, 1))) != SPMV_OK ||
-        (st = prepared_alloc(P, reinterpret_cast<void**>(&d.slice_ptr), 8 * (d.n_slices + 1))) != SPMV_OK ||
-        (st = prepared_alloc(P, reinterpret_cast<void**>(&d.count), 4)) != SPMV_OK)
-        return st;
-    const unsigned rows_grid = grid_of(A.n_rows, (int64_t)P->sm_count * 16);
-    const unsigned slice_grid = grid_of(n_pos, INT32_MAX);
-    std::vector<int> slen((size_t)std::max<int64_t>(d.n_slices, 1));
-    std::vector<int64_t> sptr((size_t)d.n_slices + 1, 0);
-    unsigned n_long = 0;
-    int64_t slots = 0;  // sum of 32 x slice length: padding by unequal rows only
+    Arena head;
+    head.add(&d.rowlen, n_pos);
+    head.add(&d.slice_len, d.n_slices);
+    head.add(&d.slice_ptr, d.n_slices + 1);
+    if ((st = head.allocate(P)) != SPMV_OK) return st;
+    SlStats f = {};
+    int64_t tile_slices = 1;
+    unsigned n_tiles = 0;
     // one layout pass for window length sigma (1 = rows in order)
     auto layout = [&](int sigma) -> spmv_status {
-        SPMV_CUDA_TRY(cudaMemsetAsync(d.rowlen, 0xFF, 4 * std::max<int64_t>(n_pos, 1), s));
-        SPMV_CUDA_TRY(cudaMemsetAsync(d.count, 0, 4, s));
-        if (A.n_rows > 0) {
-            if (sigma == 1) {
-                k_sl_rowlen_identity<<<rows_grid, kSB, 0, s>>>(A.n_rows, A.rowptr, cap, d.rowlen, d.count);
-            } else {
-                if (!d.perm) {
-                    spmv_status st2 = prepared_alloc(P, reinterpret_cast<void**>(&d.perm), 4 * A.n_rows);
-                    if (st2 != SPMV_OK) return st2;
-                }
-                const int64_t n_win = (A.n_rows + sigma - 1) / sigma;
-                k_sl_sort<<<(unsigned)n_win, kSortT, sizeof(unsigned long long) * sigma, s>>>(
-                    A.n_rows, A.rowptr, sigma, cap, d.perm, d.rowlen, d.count);
+        if (d.n_slices == 0) {
+            SPMV_CUDA_TRY(cudaMemsetAsync(d.slice_ptr, 0, 8, s));
+            return SPMV_OK;
+        }
+        const int64_t unit = sigma > 1 ? sigma / 32 : 32;  // whole windows
+        tile_slices = ((d.n_slices + kTiles - 1) / kTiles + unit - 1) / unit * unit;
+        n_tiles = (unsigned)((d.n_slices + tile_slices - 1) / tile_slices);
+        SPMV_CUDA_TRY(cudaMemsetAsync(w, 0, sizeof(SlStats) + sizeof(SlTile) * n_tiles, s));
+        if (sigma == 1) {
+            k_sl_layout<<<n_tiles, kSB, 0, s>>>(A.n_rows, d.n_slices, A.rowptr, cap, d.vec, tile_slices, d.rowlen,
+                                                d.slice_len, w);
+        } else {
+            if (!d.perm) {
+                st = prepared_alloc(P, reinterpret_cast<void**>(&d.perm), 4 * A.n_rows);
+                if (st != SPMV_OK) return st;
             }
-            SPMV_CUDA_TRY(cudaGetLastError());
-            k_sl_slice_len<<<slice_grid, kSB, 0, s>>>(d.n_slices, d.rowlen, d.slice_len);
-            SPMV_CUDA_TRY(cudaGetLastError());
-            SPMV_CUDA_TRY(cudaMemcpyAsync(slen.data(), d.slice_len, 4 * d.n_slices, cudaMemcpyDeviceToHost, s));
+            const unsigned n_win = (unsigned)((A.n_rows + sigma - 1) / sigma);
+            k_sl_sort<<<n_win, std::max(32, sigma / kSortItems), 0, s>>>(A.n_rows, d.n_slices, A.rowptr, sigma, cap,
+                                                                         d.vec, tile_slices, d.perm, d.rowlen,
+                                                                         d.slice_len, w);
         }
-        SPMV_CUDA_TRY(cudaMemcpyAsync(&n_long, d.count, 4, cudaMemcpyDeviceToHost, s));
+        SPMV_CUDA_TRY(cudaGetLastError());
+        k_sl_scan<<<n_tiles, kSB, 0, s>>>(d.n_slices, tile_slices, d.vec, d.slice_len, d.slice_ptr, w, host);
+        SPMV_CUDA_TRY(cudaGetLastError());
         SPMV_CUDA_TRY(cudaStreamSynchronize(s));
-        slots = 0;
-        for (int64_t i = 0; i < d.n_slices; ++i) {
-            sptr[i + 1] = sptr[i] + 32 * (int64_t)((slen[i] + d.vec - 1) / d.vec * d.vec);
-            slots += 32 * (int64_t)slen[i];
-        }
+        f = *host;
+        if (check && (st = feature_pass_verdict(&A)) != SPMV_OK) return st;
+        check = false;
         return SPMV_OK;
     };
-    // FP64 values: one element per slot row; FP32/BF16: four side by side
-    d.vec = P->c.value_type == SPMV_VAL_F64 ? 1 : 4;
     int sigma = P->c.block_nnz;
     if (sigma == 0) {
         // rows in order unless that pads the slices by more than a quarter;
@@ -622,7 +942,7 @@ spmv_status sliced_prepare(spmv_prepared* P, cudaStream_t s)
         // was chosen) every row above 32 nonzeros computed by a warp, so that
         // no lane's chain is longer than one element per lane of a warp
         if ((st = layout(1)) != SPMV_OK) return st;
-        if (slots > A.nnz + A.nnz / 4) {
+        if ((int64_t)f.slots > A.nnz + A.nnz / 4) {
             sigma = 4096;
             if (P->c.items_per_warp == 0) cap = 32;
             if ((st = layout(sigma)) != SPMV_OK) return st;
@@ -639,237 +959,165 @@ spmv_status sliced_prepare(spmv_prepared* P, cudaStream_t s)
     // elements (a lane's few loads leave a warp waiting on latency, so one
     // warp takes four slices), else 1 (longer slices keep four elements of
     // one row in flight instead)
-    if (P->c.value_type != SPMV_VAL_F64) {
-        P->c.threads_per_row = 1;
-    } else if (P->c.threads_per_row == 0) {
-        const int longest = d.n_slices > 0 ? *std::max_element(slen.begin(), slen.begin() + d.n_slices) : 0;
-        P->c.threads_per_row = longest <= 4 ? 4 : 1;
-    }
-    d.n_long = (int)n_long;
-    d.tot = sptr[d.n_slices];
+    if (!f64) P->c.threads_per_row = 1;
+    else if (P->c.threads_per_row == 0) P->c.threads_per_row = f.longest <= 4 ? 4 : 1;
+    d.n_long = (int)f.n_long;
+    d.n_seg = (int)f.n_seg;
+    d.n_fix = (int)f.n_fix;
+    d.tot = (int64_t)f.tot;
     // rows all of one length, in order, none long: the slice header is implied
-    d.uniform_len = -1;
-    if (sigma == 1 && n_long == 0 && A.n_rows > 0) {
-        int shortest = 0x7fffffff;
-        SPMV_CUDA_TRY(cudaMemsetAsync(d.count, 0x7f, 4, s));
-        k_sl_min_len<<<rows_grid, kSB, 0, s>>>(A.n_rows, d.rowlen, reinterpret_cast<int*>(d.count));
-        SPMV_CUDA_TRY(cudaGetLastError());
-        SPMV_CUDA_TRY(cudaMemcpyAsync(&shortest, d.count, 4, cudaMemcpyDeviceToHost, s));
-        SPMV_CUDA_TRY(cudaStreamSynchronize(s));
-        const int longest = *std::max_element(slen.begin(), slen.begin() + d.n_slices);
-        if (shortest == longest) d.uniform_len = longest;
-    }
-    SPMV_CUDA_TRY(cudaMemcpyAsync(d.slice_ptr, sptr.data(), 8 * (d.n_slices + 1), cudaMemcpyHostToDevice, s));
+    d.uniform_len = sigma == 1 && d.n_long == 0 && A.n_rows > 0 && (int)~f.shortest_c == f.longest ? f.longest : -1;
     const int64_t tot1 = std::max<int64_t>(d.tot, 1);
     const int* permp = sigma > 1 ? d.perm : nullptr;
     d.value_type = P->c.value_type;
-    if (P->c.accumulate == 0) P->c.accumulate = d.value_type == SPMV_VAL_F64 ? 1 : 2;
+    if (P->c.accumulate == 0) P->c.accumulate = f64 ? 1 : 2;
     d.acc32 = P->c.accumulate == 2;
-    if (d.value_type == SPMV_VAL_F64) {
-        // columns as offsets from the row index in 8 or 16 bits when the
-        // caller allows it and every row in the slices stays that close to
-        // its diagonal, else 32-bit
+    // a question about the columns of the rows in the slices (0 without rows)
+    auto ask = [&](auto kernel, unsigned* out) -> spmv_status {
+        *out = 0;
+        if (d.n_slices == 0) return SPMV_OK;
+        SPMV_CUDA_TRY(cudaMemsetAsync(&w->stats.reach, 0, 4, s));
+        kernel<<<(unsigned)((n_pos + kSB - 1) / kSB), kSB, 0, s>>>(d.n_slices, A.rowptr, A.colind, permp, d.rowlen,
+                                                                    &w->stats.reach);
+        SPMV_CUDA_TRY(cudaGetLastError());
+        SPMV_CUDA_TRY(cudaMemcpyAsync(&host->reach, &w->stats.reach, 4, cudaMemcpyDeviceToHost, s));
+        SPMV_CUDA_TRY(cudaStreamSynchronize(s));
+        *out = host->reach;
+        return SPMV_OK;
+    };
+    Arena body;
+    unsigned r = 0;
+    if (f64) {
         // coded columns (Table 2's deltas, or panels) when asked for and
         // every row in the slices fits: deltas in 8 bits, else 16, else (or
         // when panels were asked for) 16-bit panel offsets with 8-bit steps
         d.coding = 0;
         if (P->c.index_coding != 0 && d.n_slices > 0) {
-            auto code_reach = [&](int mode, unsigned* out) -> spmv_status {
-                SPMV_CUDA_TRY(cudaMemsetAsync(d.count, 0, 4, s));
-                const unsigned g = (unsigned)((32 * d.n_slices + kSB - 1) / kSB);
-                if (mode == 1) k_sl_code_reach<1><<<g, kSB, 0, s>>>(d.n_slices, A.rowptr, A.colind, permp, d.rowlen, d.count);
-                else k_sl_code_reach<2><<<g, kSB, 0, s>>>(d.n_slices, A.rowptr, A.colind, permp, d.rowlen, d.count);
-                SPMV_CUDA_TRY(cudaGetLastError());
-                SPMV_CUDA_TRY(cudaMemcpyAsync(out, d.count, 4, cudaMemcpyDeviceToHost, s));
-                SPMV_CUDA_TRY(cudaStreamSynchronize(s));
-                return SPMV_OK;
-            };
-            unsigned r = 0;
             if (P->c.index_coding == 1) {
-                if ((st = code_reach(1, &r)) != SPMV_OK) return st;
+                if ((st = ask(k_sl_code_reach<1>, &r)) != SPMV_OK) return st;
                 if (r <= 255) { d.coding = 1; d.cbytes = 1; }
                 else if (r <= 65535) { d.coding = 1; d.cbytes = 2; }
             }
             if (d.coding == 0) {
-                if ((st = code_reach(2, &r)) != SPMV_OK) return st;
+                if ((st = ask(k_sl_code_reach<2>, &r)) != SPMV_OK) return st;
                 if (r <= 255) { d.coding = 2; d.cbytes = 3; }
             }
         }
         // index_bytes 0: the narrowest form that fits when the rows are all of
         // one length and in order (k_sliced_uniform, where the narrower column
-        // stream shortens the launch), else 32-bit columns
+        // stream shortens the launch), else 32-bit columns.  Columns as
+        // offsets from the row index in 8 or 16 bits when the caller allows it
+        // and every row in the slices stays that close to its diagonal
         const int allowed = d.coding != 0 ? 4
                             : P->c.index_bytes != 0 ? P->c.index_bytes
                             : d.uniform_len >= 0 ? 1 : 4;
-        unsigned reach = 0;
-        if (d.n_slices > 0 && allowed < 4) {
-            SPMV_CUDA_TRY(cudaMemsetAsync(d.count, 0, 4, s));
-            k_sl_reach<<<(unsigned)((32 * d.n_slices + kSB - 1) / kSB), kSB, 0, s>>>(
-                d.n_slices, A.rowptr, A.colind, permp, d.rowlen, d.count);
-            SPMV_CUDA_TRY(cudaGetLastError());
-            SPMV_CUDA_TRY(cudaMemcpyAsync(&reach, d.count, 4, cudaMemcpyDeviceToHost, s));
-            SPMV_CUDA_TRY(cudaStreamSynchronize(s));
-        }
-        if (d.coding == 0) d.cbytes = std::max(allowed, reach <= 127 ? 1 : (reach <= 32767 ? 2 : 4));
+        r = 0;
+        if (allowed < 4 && (st = ask(k_sl_reach, &r)) != SPMV_OK) return st;
+        if (d.coding == 0) d.cbytes = std::max(allowed, r <= 127 ? 1 : (r <= 32767 ? 2 : 4));
         P->c.index_bytes = d.cbytes;
         P->c.index_coding = d.coding;
         if (d.coding != 0) P->c.threads_per_row = 1;  // coded columns: one slice per warp
         const int64_t sbytes = d.coding == 2 ? 2 : d.cbytes;  // panel offsets are 16-bit
-        if ((st = prepared_alloc(P, &d.scol, sbytes * tot1)) != SPMV_OK ||
-            (st = prepared_alloc(P, reinterpret_cast<void**>(&d.val), 8 * tot1)) != SPMV_OK)
-            return st;
-        if (d.cbytes == 4) d.col = static_cast<int*>(d.scol);
-        SPMV_CUDA_TRY(cudaMemsetAsync(d.scol, 0, sbytes * tot1, s));
-        SPMV_CUDA_TRY(cudaMemsetAsync(d.val, 0, 8 * tot1, s));
-        if (d.coding == 2) {
-            if ((st = prepared_alloc(P, reinterpret_cast<void**>(&d.step), tot1)) != SPMV_OK) return st;
-            SPMV_CUDA_TRY(cudaMemsetAsync(d.step, 0, tot1, s));
-        }
-        if (d.coding == 1) {
-            if ((st = prepared_alloc(P, reinterpret_cast<void**>(&d.rowbase), 4 * std::max<int64_t>(n_pos, 1))) != SPMV_OK)
-                return st;
-            SPMV_CUDA_TRY(cudaMemsetAsync(d.rowbase, 0, 4 * std::max<int64_t>(n_pos, 1), s));
-        }
-        if (d.n_slices > 0 && d.coding != 0) {
-#define SPMV_SL_FILL_CODED(MODE, DT)                                                                  \
-    k_sl_fill_coded<MODE, DT><<<slice_grid, kSB, 0, s>>>(d.n_slices, A.rowptr, A.colind, A.val, permp, \
-                                                        d.rowlen, d.slice_ptr, static_cast<DT*>(d.scol), \
-                                                        d.step, d.rowbase, d.val)
-            if (d.coding == 1 && d.cbytes == 1) SPMV_SL_FILL_CODED(1, uint8_t);
-            else if (d.coding == 1) SPMV_SL_FILL_CODED(1, uint16_t);
-            else SPMV_SL_FILL_CODED(2, uint16_t);
-#undef SPMV_SL_FILL_CODED
-            SPMV_CUDA_TRY(cudaGetLastError());
-        } else if (d.n_slices > 0) {
-#define SPMV_SL_FILL64(CT)                                                                           \
-    k_sl_fill<CT><<<slice_grid, kSB, 0, s>>>(d.n_slices, A.rowptr, A.colind, A.val, permp, d.rowlen, \
-                                             d.slice_ptr, static_cast<CT*>(d.scol), d.val)
-            if (d.cbytes == 1) SPMV_SL_FILL64(int8_t);
-            else if (d.cbytes == 2) SPMV_SL_FILL64(int16_t);
-            else SPMV_SL_FILL64(int);
-#undef SPMV_SL_FILL64
-            SPMV_CUDA_TRY(cudaGetLastError());
-        }
+        body.add(reinterpret_cast<char**>(&d.scol), sbytes * tot1);
+        body.add(&d.val, tot1);
+        if (d.coding == 2) body.add(&d.step, tot1);
+        if (d.coding == 1) body.add(&d.rowbase, n_pos);
     } else {
         // 16-bit offsets when every row in the slices spans fewer than 65536 columns
-        int span = 0;
-        if (d.n_slices > 0) {
-            SPMV_CUDA_TRY(cudaMemsetAsync(d.count, 0, 4, s));
-            k_sl_span<<<(unsigned)((32 * d.n_slices + kSB - 1) / kSB), kSB, 0, s>>>(
-                d.n_slices, A.rowptr, A.colind, permp, d.rowlen, reinterpret_cast<int*>(d.count));
-            SPMV_CUDA_TRY(cudaGetLastError());
-            SPMV_CUDA_TRY(cudaMemcpyAsync(&span, d.count, 4, cudaMemcpyDeviceToHost, s));
-            SPMV_CUDA_TRY(cudaStreamSynchronize(s));
-        }
-        d.off16 = span < 65536;
-        const int vb = d.value_type == SPMV_VAL_F32 ? 4 : 2;
-        if ((st = prepared_alloc(P, &d.lowval, vb * tot1)) != SPMV_OK) return st;
-        SPMV_CUDA_TRY(cudaMemsetAsync(d.lowval, 0, vb * tot1, s));
+        if ((st = ask(k_sl_span, &r)) != SPMV_OK) return st;
+        d.off16 = r < 65536;
+        body.add(reinterpret_cast<char**>(&d.lowval), (d.value_type == SPMV_VAL_F32 ? 4 : 2) * tot1);
         if (d.off16) {
-            if ((st = prepared_alloc(P, reinterpret_cast<void**>(&d.off), 2 * tot1)) != SPMV_OK ||
-                (st = prepared_alloc(P, reinterpret_cast<void**>(&d.rowbase), 4 * std::max<int64_t>(n_pos, 1))) != SPMV_OK)
-                return st;
-            SPMV_CUDA_TRY(cudaMemsetAsync(d.off, 0, 2 * tot1, s));
-            SPMV_CUDA_TRY(cudaMemsetAsync(d.rowbase, 0, 4 * std::max<int64_t>(n_pos, 1), s));
+            body.add(&d.off, tot1);
+            body.add(&d.rowbase, n_pos);
         } else {
-            if ((st = prepared_alloc(P, reinterpret_cast<void**>(&d.col), 4 * tot1)) != SPMV_OK) return st;
-            SPMV_CUDA_TRY(cudaMemsetAsync(d.col, 0, 4 * tot1, s));
-        }
-        if (d.n_slices > 0) {
-#define SPMV_SL_FILL(VT, O16)                                                                      \
-    k_sl_fill_lp<VT, O16><<<slice_grid, kSB, 0, s>>>(d.n_slices, A.rowptr, A.colind, A.val, permp, \
-                                                     d.rowlen, d.slice_ptr, d.col, d.off,          \
-                                                     d.rowbase, static_cast<VT*>(d.lowval))
-            if (d.value_type == SPMV_VAL_F32) {
-                if (d.off16) SPMV_SL_FILL(float, true); else SPMV_SL_FILL(float, false);
-            } else {
-                if (d.off16) SPMV_SL_FILL(__nv_bfloat16, true); else SPMV_SL_FILL(__nv_bfloat16, false);
-            }
-#undef SPMV_SL_FILL
-            SPMV_CUDA_TRY(cudaGetLastError());
+            body.add(&d.col, tot1);
         }
     }
-    if (d.acc32 &&
-        (st = prepared_alloc(P, reinterpret_cast<void**>(&d.x32), 4 * std::max<int64_t>(A.n_cols, 1))) != SPMV_OK)
-        return st;
+    if (d.acc32) body.add(&d.x32, A.n_cols);
+    LongTables lt = {};
     if (d.n_long > 0) {
-        if ((st = prepared_alloc(P, reinterpret_cast<void**>(&d.long_rows), 4 * (int64_t)d.n_long)) != SPMV_OK ||
-            (st = prepared_alloc(P, reinterpret_cast<void**>(&d.seg_off), 4 * ((int64_t)d.n_long + 1))) != SPMV_OK)
-            return st;
-        SPMV_CUDA_TRY(cudaMemsetAsync(d.count, 0, 4, s));
-        k_sl_long_list<<<rows_grid, kSB, 0, s>>>(A.n_rows, A.rowptr, cap, d.long_rows, d.count);
-        SPMV_CUDA_TRY(cudaGetLastError());
-        // long rows in ascending order (host sort), their lengths (device,
-        // into seg_off as scratch), then their segment offsets (host scan)
-        std::vector<int> lr(d.n_long), len(d.n_long), off(d.n_long + 1);
-        SPMV_CUDA_TRY(cudaMemcpyAsync(lr.data(), d.long_rows, 4 * (size_t)d.n_long, cudaMemcpyDeviceToHost, s));
-        SPMV_CUDA_TRY(cudaStreamSynchronize(s));
-        std::sort(lr.begin(), lr.end());
-        SPMV_CUDA_TRY(cudaMemcpyAsync(d.long_rows, lr.data(), 4 * (size_t)d.n_long, cudaMemcpyHostToDevice, s));
-        k_sl_row_lengths<<<(unsigned)((d.n_long + 255) / 256), 256, 0, s>>>(d.n_long, d.long_rows, A.rowptr,
-                                                                            d.seg_off);
-        SPMV_CUDA_TRY(cudaGetLastError());
-        SPMV_CUDA_TRY(cudaMemcpyAsync(len.data(), d.seg_off, 4 * (size_t)d.n_long, cudaMemcpyDeviceToHost, s));
-        SPMV_CUDA_TRY(cudaStreamSynchronize(s));
-        off[0] = 0;
-        for (int q = 0; q < d.n_long; ++q) off[q + 1] = off[q] + (len[q] + kSlicedSeg - 1) / kSlicedSeg;
-        d.n_seg = off[d.n_long];
-        SPMV_CUDA_TRY(cudaMemcpyAsync(d.seg_off, off.data(), 4 * ((size_t)d.n_long + 1), cudaMemcpyHostToDevice, s));
-        // the rows with several segments, summed by the fix-up
-        std::vector<int> fix;
-        for (int q = 0; q < d.n_long; ++q)
-            if (off[q + 1] - off[q] > 1) fix.push_back(q);
-        d.n_fix = (int)fix.size();
-        // per segment the index of its row in the fix list (-1: the row's only segment)
-        std::vector<int> seg_fix((size_t)d.n_seg, -1);
-        d.seg_several.assign((size_t)d.n_seg, 0);
-        for (int t = 0; t < d.n_fix; ++t)
-            for (int j = off[fix[t]]; j < off[fix[t] + 1]; ++j) {
-                seg_fix[j] = t;
-                d.seg_several[j] = 1;
-            }
-        if ((st = prepared_alloc(P, reinterpret_cast<void**>(&d.partial), 8 * (int64_t)d.n_seg)) != SPMV_OK ||
-            (st = prepared_alloc(P, reinterpret_cast<void**>(&d.seg_be), 16 * (int64_t)d.n_seg)) != SPMV_OK ||
-            (st = prepared_alloc(P, reinterpret_cast<void**>(&d.seg_row), 4 * (int64_t)d.n_seg)) != SPMV_OK ||
-            (st = prepared_alloc(P, reinterpret_cast<void**>(&d.seg_fix), 4 * (int64_t)d.n_seg)) != SPMV_OK ||
-            (st = prepared_alloc(P, reinterpret_cast<void**>(&d.fix), 4 * std::max<int64_t>(d.n_fix, 1))) != SPMV_OK ||
-            (st = prepared_alloc(P, reinterpret_cast<void**>(&d.ticket), 4 * std::max<int64_t>(d.n_fix, 1))) != SPMV_OK)
-            return st;
-        if (d.n_fix > 0)
-            SPMV_CUDA_TRY(cudaMemcpyAsync(d.fix, fix.data(), 4 * (size_t)d.n_fix, cudaMemcpyHostToDevice, s));
-        SPMV_CUDA_TRY(cudaMemsetAsync(d.ticket, 0, 4 * std::max<int64_t>(d.n_fix, 1), s));
-        SPMV_CUDA_TRY(cudaMemcpyAsync(d.seg_fix, seg_fix.data(), 4 * (size_t)d.n_seg, cudaMemcpyHostToDevice, s));
-        k_sl_seg_table<<<(unsigned)((d.n_long + 255) / 256), 256, 0, s>>>(d.n_long, d.long_rows, d.seg_off,
-                                                                          A.rowptr, d.seg_be, d.seg_row);
-        SPMV_CUDA_TRY(cudaGetLastError());
-        SPMV_CUDA_TRY(cudaStreamSynchronize(s));
+        body.add(&d.long_rows, d.n_long);
+        body.add(&d.seg_off, (int64_t)d.n_long + 1);
+        body.add(&d.partial, d.n_seg);
+        body.add(&d.seg_be, 2 * (int64_t)d.n_seg);
+        body.add(&d.seg_row, d.n_seg);
+        body.add(&d.seg_fix, d.n_seg);
+        body.add(&d.fix, d.n_fix);
+        body.add(&d.ticket, d.n_fix);
     }
-    SPMV_CUDA_TRY(cudaStreamSynchronize(s));  // host vectors go out of scope
+    if ((st = body.allocate(P)) != SPMV_OK) return st;
+    if (f64 && d.cbytes == 4) d.col = static_cast<int*>(d.scol);
+    if (d.n_slices > 0) {
+        const unsigned grid = (unsigned)((d.n_slices + kFillWarps - 1) / kFillWarps);
+        auto fill = [&](auto out) {
+            k_sl_fill<<<grid, 32 * kFillWarps, 0, s>>>(d.n_slices, A.rowptr, A.colind, A.val, permp, d.rowlen,
+                                                       d.slice_len, d.slice_ptr, out);
+        };
+        if (d.coding == 1 && d.cbytes == 1) fill(OutCoded<1, uint8_t>{static_cast<uint8_t*>(d.scol), nullptr, d.rowbase, d.val});
+        else if (d.coding == 1) fill(OutCoded<1, uint16_t>{static_cast<uint16_t*>(d.scol), nullptr, d.rowbase, d.val});
+        else if (d.coding == 2) fill(OutCoded<2, uint16_t>{static_cast<uint16_t*>(d.scol), d.step, nullptr, d.val});
+        else if (f64 && d.cbytes == 1) fill(OutF64<int8_t>{static_cast<int8_t*>(d.scol), d.val});
+        else if (f64 && d.cbytes == 2) fill(OutF64<int16_t>{static_cast<int16_t*>(d.scol), d.val});
+        else if (f64) fill(OutF64<int>{d.col, d.val});
+        else if (d.value_type == SPMV_VAL_F32 && d.off16) fill(OutLp<float, true>{nullptr, d.off, d.rowbase, static_cast<float*>(d.lowval)});
+        else if (d.value_type == SPMV_VAL_F32) fill(OutLp<float, false>{d.col, nullptr, nullptr, static_cast<float*>(d.lowval)});
+        else if (d.off16) fill(OutLp<__nv_bfloat16, true>{nullptr, d.off, d.rowbase, static_cast<__nv_bfloat16*>(d.lowval)});
+        else fill(OutLp<__nv_bfloat16, false>{d.col, nullptr, nullptr, static_cast<__nv_bfloat16*>(d.lowval)});
+        SPMV_CUDA_TRY(cudaGetLastError());
+    }
+    if (d.n_long > 0) {
+        lt = {d.long_rows, d.seg_off, d.seg_be, d.seg_row, d.seg_fix, d.fix, d.ticket};
+        k_sl_long_tables<<<n_tiles, kSB, 0, s>>>(A.n_rows, A.rowptr, cap, tile_slices, w, d.n_long, lt);
+        SPMV_CUDA_TRY(cudaGetLastError());
+    }
     P->n_blocks = d.n_slices;
     return SPMV_OK;
 }
 
-cudaError_t launch_sliced(const spmv_prepared* P, const double* x, double* y, cudaStream_t s)
+}  // namespace
+
+spmv_status sliced_prepare(spmv_prepared* P, bool check, cudaStream_t s)
+{
+    if (!t_host_stats) {
+        void* p = nullptr;
+        if (cudaMallocHost(&p, sizeof(SlStats)) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(SPMV_ERR_NOMEM, "cudaMallocHost for the layout's totals failed");
+        }
+        t_host_stats = static_cast<SlStats*>(p);
+    }
+    SlScratch* w = nullptr;
+    SPMV_CUDA_TRY(work_alloc(P->device, reinterpret_cast<void**>(&w), sizeof(SlScratch), s));
+    const spmv_status st = sliced_build(P, w, check, s);
+    cudaFreeAsync(w, s);
+    return st;
+}
+
+cudaError_t launch_sliced(const spmv_prepared* P, const double* x, double* y, cudaStream_t s, bool dry)
 {
     const spmv_csr_t& A = P->A;
     const SlicedPlan& d = P->sl;
     if (A.n_rows == 0) return cudaSuccess;
-    const unsigned grid = grid_of(32 * d.n_slices, INT32_MAX);
+    // dry: the same kernels with nothing to do, one block each
+    const int64_t n_slices = dry ? 0 : d.n_slices, n_cols = dry ? 0 : A.n_cols;
+    const int n_seg = dry ? 0 : d.n_seg;
+    const unsigned grid = grid_of(32 * n_slices, INT32_MAX);
     const int* perm = d.sigma > 1 ? d.perm : nullptr;
     cudaError_t e;
     if (d.acc32 && A.n_cols > 0) {
-        k_sl_x_to_f32<<<(unsigned)((A.n_cols + kSB - 1) / kSB), kSB, 0, s>>>(A.n_cols, x, d.x32);
+        k_sl_x_to_f32<<<grid_of(n_cols, INT32_MAX), kSB, 0, s>>>(n_cols, x, d.x32);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (d.value_type == SPMV_VAL_F64 && d.n_long > 0) {
         // slices and long-row segments in one launch, segments first
-        const unsigned seg_blocks = (unsigned)((d.n_seg + kLB / 32 - 1) / (kLB / 32));
+        const unsigned seg_blocks = (unsigned)((n_seg + kLB / 32 - 1) / (kLB / 32));
         const int R = P->c.threads_per_row == 2 || P->c.threads_per_row == 4 ? P->c.threads_per_row : 1;
-        const int64_t slice_warps = (d.n_slices + R - 1) / R;
-        const unsigned blocks = seg_blocks + (unsigned)((slice_warps + kLB / 32 - 1) / (kLB / 32));
+        const int64_t slice_warps = (n_slices + R - 1) / R;
+        const unsigned blocks = std::max(1u, seg_blocks + (unsigned)((slice_warps + kLB / 32 - 1) / (kLB / 32)));
 #define SPMV_SL_LONG(U, RR, B, CT)                                                                  \
     k_sliced_long<U, RR, B, CT><<<blocks, kLB, 0, s>>>(                                           \
-        d.n_seg, seg_blocks, d.n_slices, d.seg_be, d.seg_row, d.seg_fix, d.fix, d.long_rows,       \
+        n_seg, seg_blocks, n_slices, d.seg_be, d.seg_row, d.seg_fix, d.fix, d.long_rows,       \
         d.seg_off, d.ticket, d.partial, A.colind, A.val, d.rowlen, d.slice_len, d.slice_ptr, perm,  \
         static_cast<const CT*>(d.scol), d.val, x, y, nullptr, nullptr)
 #define SPMV_SL_LONG_CT(CT)                                                                          \
@@ -877,7 +1125,7 @@ cudaError_t launch_sliced(const spmv_prepared* P, const double* x, double* y, cu
         else SPMV_SL_LONG(4, 1, 8, CT);
 #define SPMV_SL_LONG_CODED(MODE, DT)                                                                \
     k_sliced_long<4, 1, 8, int, MODE, DT><<<blocks, kLB, 0, s>>>(                                   \
-        d.n_seg, seg_blocks, d.n_slices, d.seg_be, d.seg_row, d.seg_fix, d.fix, d.long_rows,       \
+        n_seg, seg_blocks, n_slices, d.seg_be, d.seg_row, d.seg_fix, d.fix, d.long_rows,       \
         d.seg_off, d.ticket, d.partial, A.colind, A.val, d.rowlen, d.slice_len, d.slice_ptr, perm,  \
         static_cast<const int*>(d.scol), d.val, x, y, d.step, d.rowbase)
         if (d.coding == 1 && d.cbytes == 1) { SPMV_SL_LONG_CODED(1, uint8_t); }
@@ -893,7 +1141,7 @@ cudaError_t launch_sliced(const spmv_prepared* P, const double* x, double* y, cu
     }
     if (d.value_type == SPMV_VAL_F64 && d.coding != 0) {
 #define SPMV_SL_CODED(MODE, DT)                                                                     \
-    k_sliced_coded<4, MODE, DT><<<grid, kSB, 0, s>>>(d.n_slices, d.rowlen, d.slice_len, d.slice_ptr,  \
+    k_sliced_coded<4, MODE, DT><<<grid, kSB, 0, s>>>(n_slices, d.rowlen, d.slice_len, d.slice_ptr,  \
                                                      perm, static_cast<const DT*>(d.scol), d.step,    \
                                                      d.rowbase, d.val, x, y)
         if (d.coding == 1 && d.cbytes == 1) SPMV_SL_CODED(1, uint8_t);
@@ -905,9 +1153,9 @@ cudaError_t launch_sliced(const spmv_prepared* P, const double* x, double* y, cu
     if (d.value_type == SPMV_VAL_F64 && d.uniform_len >= 0) {
         // rows of one length: no slice header (k_sliced_uniform)
         const int R = P->c.threads_per_row == 2 || P->c.threads_per_row == 4 ? P->c.threads_per_row : 1;
-        const unsigned ugrid = grid_of(32 * ((d.n_slices + R - 1) / R), R == 4 ? (int64_t)P->sm_count * 4 : INT32_MAX);
+        const unsigned ugrid = grid_of(32 * ((n_slices + R - 1) / R), R == 4 ? (int64_t)P->sm_count * 4 : INT32_MAX);
 #define SPMV_SL_U(U, RR, B, CT)                                                                    \
-    k_sliced_uniform<U, RR, B, CT><<<ugrid, kSB, 0, s>>>(A.n_rows, d.n_slices, d.uniform_len,      \
+    k_sliced_uniform<U, RR, B, CT><<<ugrid, kSB, 0, s>>>(A.n_rows, n_slices, d.uniform_len,      \
                                                          static_cast<const CT*>(d.scol), d.val, x, y)
 #define SPMV_SL_U_CT(CT)                                                                           \
         if (R == 4) SPMV_SL_U(1, 4, 4, CT); else if (R == 2) SPMV_SL_U(2, 2, 6, CT);               \
@@ -923,15 +1171,15 @@ cudaError_t launch_sliced(const spmv_prepared* P, const double* x, double* y, cu
         // R slices per warp (sliced_prepare chose R, or the caller did);
         // columns stored as CT (sliced_prepare chose the width)
 #define SPMV_SL_M(U, RR, B, CT)                                                                    \
-    k_sliced_multi<U, RR, B, CT><<<grid_of(32 * ((d.n_slices + RR - 1) / RR), INT32_MAX), kSB, 0, s>>>( \
-        d.n_slices, d.rowlen, d.slice_len, d.slice_ptr, perm, static_cast<const CT*>(d.scol), d.val, x, y)
+    k_sliced_multi<U, RR, B, CT><<<grid_of(32 * ((n_slices + RR - 1) / RR), INT32_MAX), kSB, 0, s>>>( \
+        n_slices, d.rowlen, d.slice_len, d.slice_ptr, perm, static_cast<const CT*>(d.scol), d.val, x, y)
 #define SPMV_SL_CT(CT)                                                                             \
         switch (P->c.threads_per_row) {                                                            \
             case 2: SPMV_SL_M(2, 2, 6, CT); break;                                                 \
             case 4: SPMV_SL_M(1, 4, 4, CT); break;                                                 \
             default:                                                                               \
-                k_sliced<4, CT><<<(unsigned)((d.n_slices + kOB / 32 - 1) / (kOB / 32)), kOB, 0, s>>>( \
-                    d.n_slices, d.rowlen, d.slice_len, d.slice_ptr, \
+                k_sliced<4, CT><<<std::max(1u, (unsigned)((n_slices + kOB / 32 - 1) / (kOB / 32))), kOB, 0, s>>>( \
+                    n_slices, d.rowlen, d.slice_len, d.slice_ptr, \
                                                      perm, static_cast<const CT*>(d.scol), d.val, x, y); \
         }
         if (d.cbytes == 1) { SPMV_SL_CT(int8_t) }
@@ -941,11 +1189,11 @@ cudaError_t launch_sliced(const spmv_prepared* P, const double* x, double* y, cu
 #undef SPMV_SL_M
     } else if (d.n_long > 0) {
         // FP32/BF16 values with long rows: slices and segments in one launch
-        const unsigned seg_blocks = (unsigned)((d.n_seg + kSB / 32 - 1) / (kSB / 32));
-        const unsigned blocks = seg_blocks + (unsigned)((d.n_slices + kSB / 32 - 1) / (kSB / 32));
+        const unsigned seg_blocks = (unsigned)((n_seg + kSB / 32 - 1) / (kSB / 32));
+        const unsigned blocks = std::max(1u, seg_blocks + (unsigned)((n_slices + kSB / 32 - 1) / (kSB / 32)));
 #define SPMV_SL_LONG_LP(VT, O16, A32)                                                                 \
     k_sliced_long_lp<VT, O16, A32><<<blocks, kSB, 0, s>>>(                                          \
-        d.n_seg, seg_blocks, d.n_slices, d.seg_be, d.seg_row, d.seg_fix, d.fix, d.long_rows,         \
+        n_seg, seg_blocks, n_slices, d.seg_be, d.seg_row, d.seg_fix, d.fix, d.long_rows,         \
         d.seg_off, d.ticket, d.partial, A.colind, A.val, d.rowlen, d.slice_len, d.slice_ptr, perm,    \
         d.col, d.off, d.rowbase, static_cast<const VT*>(d.lowval), x, d.x32, y)
 #define SPMV_SL_LONG_LP_VT(VT)                                                                         \
@@ -956,7 +1204,7 @@ cudaError_t launch_sliced(const spmv_prepared* P, const double* x, double* y, cu
 #undef SPMV_SL_LONG_LP
     } else {
 #define SPMV_SL_LP(VT, O16, A32)                                                                   \
-    k_sliced_lp<4, VT, O16, A32><<<grid, kSB, 0, s>>>(d.n_slices, d.rowlen, d.slice_len,          \
+    k_sliced_lp<4, VT, O16, A32><<<grid, kSB, 0, s>>>(n_slices, d.rowlen, d.slice_len,          \
                                                       d.slice_ptr, perm, d.col, d.off, d.rowbase,  \
                                                       static_cast<const VT*>(d.lowval), x, d.x32, y)
 #define SPMV_SL_LP_VT(VT)                                                        \
