@@ -54,6 +54,26 @@ __device__ __forceinline__ double widen_f32_bits(uint32_t f)
 }
 __device__ __forceinline__ double widen_f32(float a) { return widen_f32_bits(__float_as_uint(a)); }
 
+// FP64 -> FP32, to nearest even, in integer arithmetic for the same reason
+// (one conversion a row costs as much FP64 time as one of the row's DFMAs):
+// for a result with a normal exponent the top 23 mantissa bits, rounded up
+// when the 29 dropped ones exceed a half or equal it with the last kept bit
+// odd; the carry runs into the exponent, up to infinity.  Zeros and FP64
+// subnormals give the zero of the same sign; the rest (FP32 subnormals,
+// overflow, infinities, NaN) takes the conversion instruction.
+__device__ __forceinline__ float round_f32(double v)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t sign = hi & 0x80000000u, mag = hi & 0x7fffffffu;
+    if (mag - 0x38100000u < 0x0fe00000u) {  // exponents 897..1150: 2^-126 to 2^127
+        uint32_t f = ((mag - 0x38000000u) << 3) | (lo >> 29);
+        f += ((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29;
+        return __uint_as_float(sign | f);
+    }
+    if (mag < 0x00100000u) return __uint_as_float(sign);
+    return __double2float_rn(v);
+}
+
 __device__ __forceinline__ double ldval(const double* p) { return __ldcs(p); }
 __device__ __forceinline__ double ldval(const float* p) { return widen_f32(__ldcs(p)); }
 __device__ __forceinline__ double ldval(const __nv_bfloat16* p) {

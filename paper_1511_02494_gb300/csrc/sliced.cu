@@ -778,7 +778,7 @@ struct OutLp {
 __global__ void k_sl_x_to_f32(int64_t n, const double* __restrict__ x, float* __restrict__ x32)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) x32[i] = __double2float_rn(x[i]);
+    if (i < n) x32[i] = round_f32(x[i]);
 }
 
 // One slice with low-precision values (slice_value_lp).

@@ -25,7 +25,21 @@ __device__ __forceinline__ int column_of(CT stored, int row)
     else return row + (int)stored;
 }
 
-template <int U, typename CT = int>
+// FRESH: x is written by other blocks of the same kernel (with a barrier in
+// between), so it is read with ordinary loads instead of the read-only path.
+template <bool FRESH>
+__device__ __forceinline__ double ldx_of(const double* p)
+{
+    if constexpr (FRESH) {
+        double v;
+        asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+        return v;
+    } else {
+        return ldx(p);
+    }
+}
+
+template <int U, typename CT = int, bool FRESH = false>
 __device__ __forceinline__ double slice_value(int64_t s, int lane, const int* __restrict__ rowlen,
                                               const int* __restrict__ slice_len,
                                               const int64_t* __restrict__ slice_ptr,
@@ -55,7 +69,7 @@ __device__ __forceinline__ double slice_value(int64_t s, int lane, const int* __
             a[u] = ok ? __ldcs(vp + (k + u) * 32) : 0.0;
         }
 #pragma unroll
-        for (int u = 0; u < U; ++u) xv[u] = k + u < len ? ldx(x + c[u]) : 0.0;
+        for (int u = 0; u < U; ++u) xv[u] = k + u < len ? ldx_of<FRESH>(x + c[u]) : 0.0;
 #pragma unroll
         for (int u = 0; u < U; ++u)
             if (k + u < len) acc = fma(a[u], xv[u], acc);
@@ -332,7 +346,7 @@ __device__ __forceinline__ double slice_value_lp(int64_t s, int lane, const int*
         }
     }
     *row = len >= 0 ? (perm ? perm[p] : (int)p) : -1;
-    return ACC32 ? (double)acc32 : acc64;
+    return ACC32 ? widen_f32(acc32) : acc64;
 }
 
 }  // namespace dev

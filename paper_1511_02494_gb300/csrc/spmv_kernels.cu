@@ -372,7 +372,7 @@ k_compressed(int64_t n_rows, const int* __restrict__ rp, const int32_t* __restri
 __global__ void k_x_to_f32(int64_t n, const double* __restrict__ x, float* __restrict__ x32)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) x32[i] = __double2float_rn(x[i]);
+    if (i < n) x32[i] = round_f32(x[i]);
 }
 
 template <int T, typename VT, bool ALL_WIDE>
@@ -396,7 +396,7 @@ k_compressed32(int64_t n_rows, const int* __restrict__ rp, const int32_t* __rest
     else
         p = row_partial32<T, 4>(b, e, lane, ColOff16{off, base}, v, x32);
     const float s = group_sum32(p, T);
-    if (lane == 0 && row < n_rows) y[row] = (double)s;
+    if (lane == 0 && row < n_rows) y[row] = widen_f32(s);
 }
 
 inline unsigned grid_for(int64_t threads) {
