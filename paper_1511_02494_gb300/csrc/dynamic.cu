@@ -198,7 +198,7 @@ spmv_status dyn_prepare(spmv_prepared* P, cudaStream_t s)
     // 1. row-length histogram -> lanes per short row
     unsigned long long* dh = nullptr;
     unsigned long long hh[33] = {0};
-    SPMV_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&dh), sizeof(hh), s));
+    SPMV_CUDA_TRY(work_alloc(P->device, reinterpret_cast<void**>(&dh), sizeof(hh), s));
     cudaError_t e = cudaMemsetAsync(dh, 0, sizeof(hh), s);
     const unsigned grid = (unsigned)std::min<int64_t>((A.n_rows + 255) / 256, (int64_t)P->sm_count * 8);
     if (e == cudaSuccess && A.n_rows > 0) {
