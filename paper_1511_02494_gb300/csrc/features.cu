@@ -455,7 +455,7 @@ k_feature_pass(int64_t n_rows, int64_t n_cols, int64_t nnz, const int* __restric
             // this row's elements in the batch, without the row's first
             const int64_t k1 = k0 + len;
             unsigned any_bad = 0;
-            if (e > b) count_bits<FEATURES>(bits, (int)(max((int64_t)max(b + 1, cur), k0) - k0), (int)(min((int64_t)e, k1) - k0), ng, ms, any_bad);
+            if (e > b && (int64_t)b + 1 < k1) count_bits<FEATURES>(bits, (int)(max((int64_t)max(b + 1, cur), k0) - k0), (int)(min((int64_t)e, k1) - k0), ng, ms, any_bad);
             if (any_bad) err |= 16;
             __syncwarp();
             cur = (int)k1;
