@@ -575,6 +575,33 @@ double* host_target(const spmv_prepared* P, double* y_host)
     return static_cast<double*>(a.devicePointer);
 }
 
+// spmv_host's work on stream s.  `alone` (the caller waits for this call):
+// the kernels use the caller's page-locked memory themselves where they can.
+// Calls that the caller pipelines over several streams go through the staging
+// vectors: the copy engines then move one call's vectors while another's
+// kernel has the SMs, which kernels that hold the SMs for as long as the
+// link takes prevent (four matrices on eight streams, both directions of the
+// link busy: 2967 GB/s of matrix against 2286).
+spmv_status host_enqueue(spmv_prepared* P, const double* x_host, double* y_host, bool alone, cudaStream_t s)
+{
+    clear_error();
+    if (!P || (!x_host && P->A.n_cols > 0) || (!y_host && P->A.n_rows > 0))
+        return fail(SPMV_ERR_INVALID_ARG, "spmv_host: NULL argument");
+    spmv_status st;
+    if (!P->x_stage && P->A.n_cols > 0 && (st = dev_alloc(P, &P->x_stage, P->A.n_cols)) != SPMV_OK)
+        return st;
+    double* const y_direct = alone ? host_target(P, y_host) : nullptr;
+    if (!y_direct && !P->y_stage && P->A.n_rows > 0 && (st = dev_alloc(P, &P->y_stage, P->A.n_rows)) != SPMV_OK)
+        return st;
+    if (P->A.n_cols > 0)
+        SPMV_CUDA_TRY(cudaMemcpyAsync(P->x_stage, x_host, 8 * P->A.n_cols, cudaMemcpyHostToDevice, s));
+    st = run_impl(P, P->x_stage, y_direct ? y_direct : P->y_stage, s);
+    if (st != SPMV_OK) return st;
+    if (!y_direct && P->A.n_rows > 0)
+        SPMV_CUDA_TRY(cudaMemcpyAsync(y_host, P->y_stage, 8 * P->A.n_rows, cudaMemcpyDeviceToHost, s));
+    return SPMV_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -792,32 +819,17 @@ spmv_status spmv(const spmv_prepared_t* P, const double* x, double* y, spmv_stre
 spmv_status spmv_host(spmv_prepared_t* P, const double* x_host, double* y_host,
                       spmv_stream_t stream)
 {
-    spmv_status st = spmv_host_async(P, x_host, y_host, stream);
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    spmv_status st = host_enqueue(P, x_host, y_host, true, s);
     if (st != SPMV_OK) return st;
-    SPMV_CUDA_TRY(cudaStreamSynchronize(reinterpret_cast<cudaStream_t>(stream)));
+    SPMV_CUDA_TRY(cudaStreamSynchronize(s));
     return SPMV_OK;
 }
 
 spmv_status spmv_host_async(spmv_prepared_t* P, const double* x_host, double* y_host,
                             spmv_stream_t stream)
 {
-    clear_error();
-    if (!P || (!x_host && P->A.n_cols > 0) || (!y_host && P->A.n_rows > 0))
-        return fail(SPMV_ERR_INVALID_ARG, "spmv_host: NULL argument");
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    spmv_status st;
-    if (!P->x_stage && P->A.n_cols > 0 && (st = dev_alloc(P, &P->x_stage, P->A.n_cols)) != SPMV_OK)
-        return st;
-    double* const y_direct = host_target(P, y_host);
-    if (!y_direct && !P->y_stage && P->A.n_rows > 0 && (st = dev_alloc(P, &P->y_stage, P->A.n_rows)) != SPMV_OK)
-        return st;
-    if (P->A.n_cols > 0)
-        SPMV_CUDA_TRY(cudaMemcpyAsync(P->x_stage, x_host, 8 * P->A.n_cols, cudaMemcpyHostToDevice, s));
-    st = run_impl(P, P->x_stage, y_direct ? y_direct : P->y_stage, s);
-    if (st != SPMV_OK) return st;
-    if (!y_direct && P->A.n_rows > 0)
-        SPMV_CUDA_TRY(cudaMemcpyAsync(y_host, P->y_stage, 8 * P->A.n_rows, cudaMemcpyDeviceToHost, s));
-    return SPMV_OK;
+    return host_enqueue(P, x_host, y_host, false, reinterpret_cast<cudaStream_t>(stream));
 }
 
 spmv_status spmv_prepared_info(const spmv_prepared_t* P, spmv_prepared_info_t* info)
