@@ -553,8 +553,10 @@ spmv_status spmv(const spmv_prepared_t *P, const double *x, double *y, spmv_stre
 
 /* End-to-end form of spmv for host vectors: copies x_host [n_cols] to the
  * device, runs spmv, copies y back to y_host [n_rows] and synchronizes
- * `stream`.  Page-locked host buffers give full copy bandwidth.  The device
- * staging vectors are allocated on the first call and owned by P. */
+ * `stream`.  Page-locked host buffers give full copy bandwidth, and let the
+ * kernels of some forms write y into y_host themselves and pull x from x_host
+ * while they multiply, so that the transfers pass beside the product.  The
+ * device staging vectors are allocated on the first call and owned by P. */
 spmv_status spmv_host(spmv_prepared_t *P, const double *x_host, double *y_host,
                       spmv_stream_t stream);
 

@@ -542,6 +542,21 @@ spmv_status run_impl(const spmv_prepared_t* P, const double* x, double* y, cudaS
     return SPMV_OK;
 }
 
+// The device's address of n doubles of page-locked host memory, mapped from
+// the first to the last; null for other memory.
+double* mapped(double* host, int64_t n)
+{
+    cudaPointerAttributes a, b;
+    if (cudaPointerGetAttributes(&a, host) != cudaSuccess || cudaPointerGetAttributes(&b, host + n - 1) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer ||
+        static_cast<double*>(b.devicePointer) != static_cast<double*>(a.devicePointer) + n - 1)
+        return nullptr;
+    return static_cast<double*>(a.devicePointer);
+}
+
 // Where the kernels of P can write y into the caller's host memory
 // themselves, so that its download passes behind the product instead of after
 // it (27-point stencil 128^3, 16.8 MB of y: 217 us for the call against 315):
@@ -562,17 +577,22 @@ double* host_target(const spmv_prepared* P, double* y_host)
         case SPMV_V7_SLICED: in_order = P->sl.sigma == 1; break;
         default: break;
     }
-    if (!in_order || P->A.n_rows == 0) return nullptr;
-    cudaPointerAttributes a, b;
-    const int64_t last = P->A.n_rows - 1;
-    if (cudaPointerGetAttributes(&a, y_host) != cudaSuccess || cudaPointerGetAttributes(&b, y_host + last) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer ||
-        static_cast<double*>(b.devicePointer) != static_cast<double*>(a.devicePointer) + last)
-        return nullptr;
-    return static_cast<double*>(a.devicePointer);
+    return in_order && P->A.n_rows > 0 ? mapped(y_host, P->A.n_rows) : nullptr;
+}
+
+// The same for x, which a form of the SLICED kernel pulls while it multiplies
+// (k_sliced_host, sliced_host_form): page-locked, and apart from a y that the
+// kernel writes.  27-point stencil 128^3, 16.8 MB of x: 158 us for the call
+// against 216 with the copy first.
+const double* host_source(const spmv_prepared* P, const double* x_host, const double* y_host, const double* y_direct)
+{
+    if (!sliced_host_form(P)) return nullptr;
+    const double* x = mapped(const_cast<double*>(x_host), P->A.n_cols);
+    auto apart = [&](const double* a, const double* b) {
+        const uintptr_t u = (uintptr_t)a, v = (uintptr_t)b;
+        return u + 8 * (uintptr_t)P->A.n_cols <= v || v + 8 * (uintptr_t)P->A.n_rows <= u;
+    };
+    return x && (!y_direct || (apart(x_host, y_host) && apart(x, y_direct))) ? x : nullptr;
 }
 
 // spmv_host's work on stream s.  `alone` (the caller waits for this call):
@@ -593,10 +613,19 @@ spmv_status host_enqueue(spmv_prepared* P, const double* x_host, double* y_host,
     double* const y_direct = alone ? host_target(P, y_host) : nullptr;
     if (!y_direct && !P->y_stage && P->A.n_rows > 0 && (st = dev_alloc(P, &P->y_stage, P->A.n_rows)) != SPMV_OK)
         return st;
-    if (P->A.n_cols > 0)
-        SPMV_CUDA_TRY(cudaMemcpyAsync(P->x_stage, x_host, 8 * P->A.n_cols, cudaMemcpyHostToDevice, s));
-    st = run_impl(P, P->x_stage, y_direct ? y_direct : P->y_stage, s);
-    if (st != SPMV_OK) return st;
+    double* const y = y_direct ? y_direct : P->y_stage;
+    if (const double* x_direct = alone ? host_source(P, x_host, y_host, y_direct) : nullptr) {
+        if (!P->x_count && (st = dev_alloc(P, &P->x_count, sliced_host_words())) != SPMV_OK) return st;
+        if (!P->status) {
+            if ((st = dev_alloc(P, &P->status, 1)) != SPMV_OK) return st;
+            SPMV_CUDA_TRY(cudaMemsetAsync(P->status, 0, sizeof(unsigned), s));
+        }
+        SPMV_CUDA_TRY(launch_sliced_host(P, x_direct, y, s));
+    } else {
+        if (P->A.n_cols > 0)
+            SPMV_CUDA_TRY(cudaMemcpyAsync(P->x_stage, x_host, 8 * P->A.n_cols, cudaMemcpyHostToDevice, s));
+        if ((st = run_impl(P, P->x_stage, y, s)) != SPMV_OK) return st;
+    }
     if (!y_direct && P->A.n_rows > 0)
         SPMV_CUDA_TRY(cudaMemcpyAsync(y_host, P->y_stage, 8 * P->A.n_rows, cudaMemcpyDeviceToHost, s));
     return SPMV_OK;

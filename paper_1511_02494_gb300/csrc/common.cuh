@@ -84,6 +84,7 @@ constexpr int kSlicedSeg = 2048;
 struct SlicedPlan {
     int64_t n_slices = 0, tot = 0;
     int sigma = 1, n_long = 0;
+    unsigned ahead = 0;          // sigma 1: columns by which rows (one in 32, sampled) reach ahead of the diagonal
     int uniform_len = -1;        // >= 0: every row has this many nonzeros, rows in order, none long
     int* rowlen = nullptr;       // [32 n_slices] row length per position, -1: long or absent
     int* slice_len = nullptr;    // [n_slices]
@@ -132,6 +133,7 @@ struct spmv_prepared {
     int64_t n_wide = 0;
     double* x_stage = nullptr;     // spmv_host staging
     double* y_stage = nullptr;
+    unsigned* x_count = nullptr;   // spmv_host: stages of x that have arrived
     int64_t owned_bytes = 0;
     int sm_count = 0;
     int l2_window_bytes = 0;       // LATENCY: bytes of x kept persisting in L2
@@ -183,6 +185,12 @@ cudaError_t launch_dyn(const spmv_prepared* P, const double* x, double* y, cudaS
 spmv_status sliced_prepare(spmv_prepared* P, bool check, cudaStream_t s);
 // dry: the kernels that a call would launch, with nothing to do (loads them)
 cudaError_t launch_sliced(const spmv_prepared* P, const double* x, double* y, cudaStream_t s, bool dry = false);
+// The product with x pulled from page-locked host memory beside it: for
+// prepared objects of this form, with x_stage, x_count (sliced_host_words()
+// words) and status allocated.
+bool sliced_host_form(const spmv_prepared* P);
+size_t sliced_host_words();
+cudaError_t launch_sliced_host(const spmv_prepared* P, const double* x_host, double* y, cudaStream_t s);
 cudaError_t launch_latency(const spmv_csr_t& A, int T, const double* x, double* y,
                            int l2_window_bytes, cudaStream_t s);
 cudaError_t launch_compress(const spmv_csr_t& A, int32_t* rowbase, uint16_t* off16,

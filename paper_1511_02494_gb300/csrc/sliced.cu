@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "ptx.cuh"
 #include "rowdot.cuh"
 #include "sliced.cuh"
 
@@ -44,7 +45,7 @@ struct SlStats {
     unsigned n_long, n_seg, n_fix;
     int longest;                // longest slice
     unsigned shortest_c;        // maximum of ~length over the rows
-    unsigned reach;             // for the column-width questions
+    unsigned reach;             // columns ahead of the diagonal (sampled), then the column-width questions' answers
 };
 // The slices are cut into at most kTiles tiles of equal length (whole sort
 // windows); per tile the element slots and the long rows, their segments and
@@ -64,7 +65,7 @@ struct SlScratch {
 // a thread's share of a tile
 struct TileAcc {
     unsigned long long len = 0, slots = 0;
-    unsigned n_long = 0, n_seg = 0, n_fix = 0, shortest_c = 0;
+    unsigned n_long = 0, n_seg = 0, n_fix = 0, shortest_c = 0, reach = 0;
     int longest = 0;
 
     // one row: its length in the slices, -1 when it is long
@@ -91,7 +92,7 @@ struct TileAcc {
         if (threadIdx.x == 0) { t = SlTile{}; g = SlStats{}; }
         __syncthreads();
         const unsigned nl = __reduce_add_sync(FULL, n_long), ns = __reduce_add_sync(FULL, n_seg),
-                       nf = __reduce_add_sync(FULL, n_fix), sc = __reduce_max_sync(FULL, shortest_c);
+                       nf = __reduce_add_sync(FULL, n_fix), sc = __reduce_max_sync(FULL, shortest_c), re = __reduce_max_sync(FULL, reach);
         const int lo = __reduce_max_sync(FULL, longest);
         unsigned long long l = len, q = slots;
         for (int o = 16; o > 0; o >>= 1) {
@@ -103,6 +104,7 @@ struct TileAcc {
             atomicAdd(&g.slots, q);
             atomicMax(&g.longest, lo);
             atomicMax(&g.shortest_c, sc);
+            if (re) atomicMax(&g.reach, re);
             if (nl) { atomicAdd(&t.n_long, nl); atomicAdd(&t.n_seg, ns); atomicAdd(&t.n_fix, nf); }
         }
         __syncthreads();
@@ -113,6 +115,7 @@ struct TileAcc {
             atomicAdd(&S->slots, g.slots);
             atomicMax(&S->longest, g.longest);
             atomicMax(&S->shortest_c, g.shortest_c);
+            if (g.reach) atomicMax(&S->reach, g.reach);
             if (t.n_long) {
                 atomicAdd(&T->n_long, t.n_long); atomicAdd(&T->n_seg, t.n_seg); atomicAdd(&T->n_fix, t.n_fix);
                 atomicAdd(&S->n_long, t.n_long); atomicAdd(&S->n_seg, t.n_seg); atomicAdd(&S->n_fix, t.n_fix);
@@ -124,12 +127,14 @@ struct TileAcc {
 // Rows in order: row lengths and slice lengths, a block per tile, a warp per
 // slice, four slices' row pointers in flight.
 __global__ void __launch_bounds__(kSB)
-k_sl_layout(int64_t n_rows, int64_t n_slices, const int* __restrict__ rp, int cap, int vec, int64_t tile_slices,
+k_sl_layout(int64_t n_rows, int64_t n_cols, int64_t nnz, int64_t n_slices, const int* __restrict__ rp,
+            const int* __restrict__ ci, int cap, int vec, int64_t tile_slices,
             int* __restrict__ rowlen, int* __restrict__ slice_len, SlScratch* __restrict__ w)
 {
     constexpr int U = 4;
     const int lane = threadIdx.x & 31;
     const int64_t t0 = blockIdx.x * tile_slices, t1 = min(n_slices, t0 + tile_slices);
+    const float ahead = (float)n_cols / (float)n_rows;
     TileAcc acc;
     for (int64_t s0 = t0 + (threadIdx.x >> 5) * U; s0 < t1; s0 += (kSB / 32) * U) {
         int b[U], e[U];
@@ -150,6 +155,12 @@ k_sl_layout(int64_t n_rows, int64_t n_slices, const int* __restrict__ rp, int ca
             if (lane == 0) {
                 slice_len[s0 + u] = m;
                 acc.slice(m, vec);
+                // how far ahead of the corner-to-corner diagonal the slice's
+                // first row reaches (the matrix need not be a valid one yet)
+                if (b[u] >= 0 && e[u] > b[u] && e[u] <= nnz) {
+                    const int64_t over = (int64_t)__ldg(ci + e[u] - 1) - (int64_t)((float)p * ahead);
+                    acc.reach = max(acc.reach, (unsigned)max((int64_t)0, min(over, (int64_t)INT32_MAX)));
+                }
             }
         }
     }
@@ -520,6 +531,142 @@ k_sliced(int64_t n_slices, const int* __restrict__ rowlen, const int* __restrict
     const int64_t s = ((int64_t)blockIdx.x * kOB + threadIdx.x) >> 5;
     if (s >= n_slices) return;  // whole warps only
     slice_rows<U, CT>(s, threadIdx.x & 31, rowlen, slice_len, slice_ptr, perm, col, val, x, y);
+}
+
+// The product with x still in the caller's page-locked memory: the first
+// blocks pull x over the link into the staging vector, stage by stage in
+// ascending order, and the others, a slice per warp as in k_sliced, gather a
+// batch of elements once the stage of its largest column is complete.  So the
+// upload passes beside the product instead of before it.  A waiting warp
+// holds up nothing: the copying blocks come first in the grid and wait for
+// nobody.  Every wait is bounded all the same; one that gives up sets
+// *status.  x is read with ordinary loads after an acquire: a sector enters
+// L1 only when its stage is complete, so none is stale.
+// Bound by the link: pulling 16.8 MB takes 87 us (512 warps with 4 x 16
+// bytes a lane in flight; 2 x 16 are slower, 8 x 16 or 1024 warps no faster).
+// What the waits cost is the looking: 9700 resident warps that look at one
+// counter every 0.2 us keep its L2 slice from taking the copies' own counts
+// (980 us for the 27-point stencil 128^3), every 1 us 162 us, every 2 us
+// 145, every 8 us 138 but longer where the product keeps pace with the link
+// (7-point 128^3: 191 us for the call against 167).
+constexpr int kXStages = 64;          // at most
+constexpr int kXShift = 15;           // columns of a stage, at least (log2)
+constexpr unsigned kXWarps = 512;     // copying warps: 64 columns each of a stage's 32768
+constexpr int kXStride = 32;          // words from one stage's counter to the next: a line each
+constexpr unsigned kXSleepNs = 2048;  // between two looks at a counter
+constexpr uint64_t kXLimitNs = 2000000000ull;
+struct HostX {
+    const double* src;  // device address of the host vector
+    double* dst;
+    int64_t n;
+    int shift;          // log2 of the columns of a stage
+    unsigned* count;    // [kXStages kXStride] warps that have finished a stage (each finishes them in order)
+    unsigned* status;
+};
+
+__device__ __forceinline__ void pull_x(const HostX& h, unsigned w, int lane)
+{
+    constexpr int U = 4;  // 16 bytes each, in flight per lane
+    const int lg = h.shift - kXShift;  // log2 of a warp's items of a stage
+    const unsigned n = (unsigned)h.n, per = 1u << lg;
+    const unsigned items = (((n - 1) >> h.shift) + 1) << lg;
+    const bool wide = ((uintptr_t)h.src & 15) == 0;
+    // the lane's first column of item t (item t of a stage: 32768 columns on)
+    auto column = [&](unsigned t) { return (t >> lg << h.shift) + ((t & (per - 1)) << kXShift) + w * 64 + 2 * lane; };
+    for (unsigned t0 = 0; t0 < items; t0 += U) {
+        double2 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const unsigned c = column(t0 + u);
+            const bool in = t0 + u < items;
+            if (wide && in && c + 1 < n) {
+                v[u] = __ldcs(reinterpret_cast<const double2*>(h.src + c));
+            } else {
+                v[u].x = in && c < n ? __ldcs(h.src + c) : 0.0;
+                v[u].y = in && c + 1 < n ? __ldcs(h.src + c + 1) : 0.0;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const unsigned c = column(t0 + u);
+            if (t0 + u < items && c + 1 < n) *reinterpret_cast<double2*>(h.dst + c) = v[u];
+            else if (t0 + u < items && c < n) h.dst[c] = v[u].x;
+        }
+        __threadfence();
+        __syncwarp();
+        if (lane == 0)
+            for (unsigned t = t0; t < t0 + U && t < items; ++t)
+                if (((t + 1) & (per - 1)) == 0)
+                    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(h.count + kXStride * (t >> lg)) : "memory");
+    }
+}
+
+// true once all warps have finished the stage (for the whole warp)
+__device__ __forceinline__ bool stage_in(const HostX& h, int stage)
+{
+    unsigned v = 0;
+    if ((threadIdx.x & 31) == 0) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(h.count + kXStride * stage) : "memory");
+    }
+    v = __shfl_sync(FULL, v, 0);
+    __syncwarp();
+    return v == kXWarps;
+}
+
+template <int U, typename CT>
+__global__ void __launch_bounds__(kOB, 32)
+k_sliced_host(HostX h, unsigned copy_blocks, int64_t n_slices, const int* __restrict__ rowlen,
+              const int* __restrict__ slice_len, const int64_t* __restrict__ slice_ptr,
+              const CT* __restrict__ col, const double* __restrict__ val, double* __restrict__ y)
+{
+    const int lane = threadIdx.x & 31;
+    if (blockIdx.x < copy_blocks) {
+        pull_x(h, blockIdx.x * (kOB / 32) + (threadIdx.x >> 5), lane);
+        return;
+    }
+    const int64_t s = ((int64_t)(blockIdx.x - copy_blocks) * kOB + threadIdx.x) >> 5;
+    if (s >= n_slices) return;  // whole warps only
+    const int last = (int)((h.n - 1) >> h.shift);
+    const int64_t p = s * 32 + lane;
+    const int len = rowlen[p], L = slice_len[s];
+    const int64_t q0 = slice_ptr[s] + lane;
+    unsigned ready = stage_in(h, last) ? 0xffffffffu : 0u;  // columns below it are in
+    const CT* __restrict__ cp = col + q0;
+    const double* __restrict__ vp = val + q0;
+    double acc = 0.0;
+    for (int k = 0; k < L; k += U) {
+        int c[U];
+        double a[U], xv[U];
+        int top = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool ok = k + u < len;
+            c[u] = ok ? column_of(__ldcs(cp + (k + u) * 32), (int)p) : 0;
+            a[u] = ok ? __ldcs(vp + (k + u) * 32) : 0.0;
+            top = max(top, c[u]);
+        }
+        top = __reduce_max_sync(FULL, top);
+        if ((unsigned)top >= ready) {
+            const int stage = top >> h.shift;
+            uint64_t t0 = 0;
+            while (!stage_in(h, stage)) {
+                const uint64_t now = __shfl_sync(FULL, ptx::global_ns(), 0);
+                if (t0 == 0) t0 = now;
+                if (now - t0 > kXLimitNs) {
+                    if (lane == 0) *h.status = 1u;
+                    break;
+                }
+                __nanosleep(kXSleepNs);
+            }
+            ready = stage == last ? 0xffffffffu : (unsigned)(stage + 1) << h.shift;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) xv[u] = k + u < len ? ldx_of<true>(h.dst + c[u]) : 0.0;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (k + u < len) acc = fma(a[u], xv[u], acc);
+    }
+    if (len >= 0) y[p] = acc;
 }
 
 // One slice per warp with coded columns (slice_value_coded).
@@ -914,8 +1061,8 @@ spmv_status sliced_build(spmv_prepared* P, SlScratch* w, bool check, cudaStream_
         n_tiles = (unsigned)((d.n_slices + tile_slices - 1) / tile_slices);
         SPMV_CUDA_TRY(cudaMemsetAsync(w, 0, sizeof(SlStats) + sizeof(SlTile) * n_tiles, s));
         if (sigma == 1) {
-            k_sl_layout<<<n_tiles, kSB, 0, s>>>(A.n_rows, d.n_slices, A.rowptr, cap, d.vec, tile_slices, d.rowlen,
-                                                d.slice_len, w);
+            k_sl_layout<<<n_tiles, kSB, 0, s>>>(A.n_rows, A.n_cols, A.nnz, d.n_slices, A.rowptr, A.colind, cap, d.vec,
+                                                tile_slices, d.rowlen, d.slice_len, w);
         } else {
             if (!d.perm) {
                 st = prepared_alloc(P, reinterpret_cast<void**>(&d.perm), 4 * A.n_rows);
@@ -955,6 +1102,7 @@ spmv_status sliced_build(spmv_prepared* P, SlScratch* w, bool check, cudaStream_
     P->c.block_nnz = sigma;
     P->c.items_per_warp = cap;
     d.sigma = sigma;
+    d.ahead = sigma == 1 ? f.reach : 0;
     // FP64 values: slices per warp, 4 when no slice is longer than four
     // elements (a lane's few loads leave a warp waiting on latency, so one
     // warp takes four slices), else 1 (longer slices keep four elements of
@@ -1092,6 +1240,42 @@ spmv_status sliced_prepare(spmv_prepared* P, bool check, cudaStream_t s)
     const spmv_status st = sliced_build(P, w, check, s);
     cudaFreeAsync(w, s);
     return st;
+}
+
+// Where k_sliced_host pays: x of at least half a million columns and rows
+// that reach no further than a quarter of them ahead of the diagonal (a
+// sample, one row in 32: the speed depends on it, the result does not).  Call
+// with the copy first and so, in us: 27-point stencil 96^3 112 and 88, 128^3
+// 216 and 158, 160^3 390 and 305; 7-point 128^3 195 and 167; a band of 6 per
+// row, 1M rows 104 and 99, 4M 344 and 288; below the limits 27-point 48^3 34
+// and 40, 64^3 52 and 53, random columns 1M x 20 136 and 153, 2M x 20 244
+// and 276 (nothing passes beside the upload, and the header costs where rows
+// are of one length).
+bool sliced_host_form(const spmv_prepared* P)
+{
+    const SlicedPlan& d = P->sl;
+    return P->c.variant == SPMV_V7_SLICED && d.value_type == SPMV_VAL_F64 && d.coding == 0 && d.n_long == 0 &&
+           d.sigma == 1 && P->A.n_cols >= 1 << 19 && (int64_t)d.ahead * 4 <= P->A.n_cols && P->c.threads_per_row != 2 && P->c.threads_per_row != 4 && P->A.n_rows > 0 && P->A.n_cols > 0;
+}
+
+size_t sliced_host_words() { return kXStride * kXStages; }
+
+cudaError_t launch_sliced_host(const spmv_prepared* P, const double* x_host, double* y, cudaStream_t s)
+{
+    const SlicedPlan& d = P->sl;
+    HostX h{x_host, P->x_stage, P->A.n_cols, kXShift, P->x_count, P->status};
+    while (((h.n - 1) >> h.shift) >= kXStages) ++h.shift;
+    cudaError_t e = cudaMemsetAsync(P->x_count, 0, sizeof(unsigned) * kXStride * kXStages, s);
+    if (e != cudaSuccess) return e;
+    const unsigned copy = kXWarps / (kOB / 32), blocks = copy + (unsigned)((d.n_slices + kOB / 32 - 1) / (kOB / 32));
+#define SPMV_SL_HOST(CT)                                                                            \
+    k_sliced_host<4, CT><<<blocks, kOB, 0, s>>>(h, copy, d.n_slices, d.rowlen, d.slice_len, d.slice_ptr, \
+                                                static_cast<const CT*>(d.scol), d.val, y)
+    if (d.cbytes == 1) SPMV_SL_HOST(int8_t);
+    else if (d.cbytes == 2) SPMV_SL_HOST(int16_t);
+    else SPMV_SL_HOST(int);
+#undef SPMV_SL_HOST
+    return cudaGetLastError();
 }
 
 cudaError_t launch_sliced(const spmv_prepared* P, const double* x, double* y, cudaStream_t s, bool dry)
