@@ -30,6 +30,7 @@ typedef unsigned __int128 u128;
 // 32, 32 and 64 bits, whose sums over blocks need no carries.
 constexpr int kFT = 256;        // threads per block of both kernels
 constexpr int kFeatBlocks = 3;  // their resident blocks per SM (80 registers)
+constexpr int kShortRow = 8;
 constexpr int64_t kLongRow = 1024;
 constexpr int64_t kPiece = 2048;
 constexpr int kFields = 18;
@@ -79,7 +80,7 @@ __device__ __forceinline__ u64 warp_sum_u64(u64 v) {
 // gives a correction, and the remainder is brought into [0, b).  The
 // reciprocal and the three products are each off by at most 2 ulp, so the
 // first estimate is within 2^10 of the quotient, |remainder| < 2^42 and the
-// second within one; the final steps run at most once (capped at four).
+// second within one, which the last line settles.
 // Arguments outside that range come only from rows the pass flags as invalid
 // (columns not strictly increasing or out of range), whose results are
 // discarded: they give 0.
@@ -94,18 +95,26 @@ __device__ __forceinline__ unsigned fixq32(unsigned a, unsigned b)
     const int c = __float2int_rd(__fmul_rn(rf, rb));
     q += (unsigned)c;
     rem -= (int64_t)c * b;
-    for (int i = 0; i < 4 && rem < 0; ++i) { --q; rem += b; }
-    for (int i = 0; i < 4 && rem >= (int64_t)b; ++i) { ++q; rem -= b; }
-    return q;
+    return rem < 0 ? q - 1 : rem >= (int64_t)b ? q + 1 : q;
 }
 
+// A sum of 64-bit terms of which one thread adds fewer than 2^32.
+struct Sum96 {
+    u64 lo = 0;
+    unsigned hi = 0;
+    __device__ __forceinline__ void add(u64 v) {
+        asm("add.cc.u64 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+l"(lo), "+r"(hi) : "l"(v));
+    }
+    __device__ __forceinline__ u128 value() const { return ((u128)hi << 64) | lo; }
+};
+
 // Per-thread partial aggregates of the rows a thread finalizes.  A ratio of
-// exactly 1 (2^32 in fixed point, one bit too wide) is counted apart, so that
-// every per-row quantity fits 32 bits and its square 64.
+// exactly 1 (2^32 in fixed point, one bit too wide) is added to the sums'
+// upper words, so that every per-row quantity fits 32 bits and its square 64.
 struct RowAgg {
-    unsigned nnz_min = 0xffffffffu, nnz_max = 0, bw_min = 0xffffffffu, bw_max = 0, disp_ones = 0, clust_ones = 0;
+    unsigned nnz_min = 0xffffffffu, nnz_max = 0, bw_min = 0xffffffffu, bw_max = 0;
     u64 nnz_sum = 0, nnz_sq = 0, bw_sum = 0, disp_sum = 0, clust_sum = 0, ng_sum = 0, ms_sum = 0;
-    u128 bw_sq = 0, disp_sq = 0;
+    Sum96 bw_sq, disp_sq;
 
     // one row: nz nonzeros, columns first..last, ng / ms counted over its
     // elements after the first (the first element adds one to each)
@@ -117,8 +126,8 @@ struct RowAgg {
             ms += 1;
             dq = fixq32(nz, bw + 1);
             cq = fixq32(ng, nz);
-            disp_ones += nz == bw + 1;
-            clust_ones += ng == nz;
+            if (nz == bw + 1) { disp_sum += 1ull << 32; ++disp_sq.hi; }
+            if (ng == nz) clust_sum += 1ull << 32;
         }
         nnz_min = min(nnz_min, nz);
         nnz_max = max(nnz_max, nz);
@@ -127,26 +136,26 @@ struct RowAgg {
         bw_min = min(bw_min, bw);
         bw_max = max(bw_max, bw);
         bw_sum += bw;
-        bw_sq += (u64)bw * bw;
+        bw_sq.add((u64)bw * bw);
         disp_sum += dq;
-        disp_sq += (u64)dq * dq;
+        disp_sq.add((u64)dq * dq);
         clust_sum += cq;
         ng_sum += ng;
         ms_sum += ms;
     }
 
-    // minima as complements and the ratios of 1 folded in
-    __device__ __forceinline__ void words(u64* t, unsigned err) {
+    // minima as complements; the 128-bit sums apart
+    __device__ __forceinline__ void words(u64* t, unsigned err, u128 bw_sq, u128 disp_sq) {
         const u64 m32 = 0xffffffffull;
         t[0] = nnz_min == 0xffffffffu ? 0 : ~(u64)nnz_min;
         t[1] = nnz_max; t[2] = nnz_sum; t[3] = nnz_sq;
         t[4] = bw_min == 0xffffffffu ? 0 : ~(u64)bw_min;
         t[5] = bw_max; t[6] = bw_sum;
-        t[7] = disp_sum + ((u64)disp_ones << 32);
-        t[8] = clust_sum + ((u64)clust_ones << 32);
+        t[7] = disp_sum;
+        t[8] = clust_sum;
         t[9] = ng_sum; t[10] = ms_sum; t[11] = err;
         t[12] = (u64)bw_sq & m32; t[13] = (u64)bw_sq >> 32; t[14] = (u64)(bw_sq >> 64);
-        t[15] = (u64)disp_sq & m32; t[16] = (u64)disp_sq >> 32; t[17] = (u64)(disp_sq >> 64) + disp_ones;
+        t[15] = (u64)disp_sq & m32; t[16] = (u64)disp_sq >> 32; t[17] = (u64)(disp_sq >> 64);
     }
 };
 
@@ -165,24 +174,23 @@ __device__ void flush_block(RowAgg& r, unsigned err, u64 (*s_red)[kFields], Feat
 {
     err = __reduce_or_sync(FULL_MASK, err);
     const int w = threadIdx.x >> 5;
+    u128 bw_sq = 0, disp_sq = 0;
     if (FEATURES) {
         r.nnz_min = __reduce_min_sync(FULL_MASK, r.nnz_min);
         r.nnz_max = __reduce_max_sync(FULL_MASK, r.nnz_max);
         r.bw_min = __reduce_min_sync(FULL_MASK, r.bw_min);
         r.bw_max = __reduce_max_sync(FULL_MASK, r.bw_max);
-        r.disp_ones = __reduce_add_sync(FULL_MASK, r.disp_ones);
-        r.clust_ones = __reduce_add_sync(FULL_MASK, r.clust_ones);
         r.nnz_sum = warp_sum_u64(r.nnz_sum);
         r.nnz_sq = warp_sum_u64(r.nnz_sq);
         r.bw_sum = warp_sum_u64(r.bw_sum);
-        r.bw_sq = warp_sum_u128(r.bw_sq);
+        bw_sq = warp_sum_u128(r.bw_sq.value());
         r.disp_sum = warp_sum_u64(r.disp_sum);
-        r.disp_sq = warp_sum_u128(r.disp_sq);
+        disp_sq = warp_sum_u128(r.disp_sq.value());
         r.clust_sum = warp_sum_u64(r.clust_sum);
         r.ng_sum = warp_sum_u64(r.ng_sum);
         r.ms_sum = warp_sum_u64(r.ms_sum);
     }
-    if ((threadIdx.x & 31) == 0) r.words(s_red[w], err);
+    if ((threadIdx.x & 31) == 0) r.words(s_red[w], err, bw_sq, disp_sq);
     __syncthreads();
     const int f = threadIdx.x;
     if (f < kFields && (FEATURES || f == 11)) {
@@ -439,6 +447,30 @@ k_feature_pass(int64_t n_rows, int64_t n_cols, int64_t nnz, const int* __restric
         if (!row_ok) b = e = 0;
         unsigned ng = 0, ms = 0;
         int first = 0, last = 0;
+        // A tile of rows of at most kShortRow: a lane's few loads, in flight
+        // together, cover what the streaming would, without its batches and
+        // shared memory (bound by issue: 8M rows of 2, the call 188 us
+        // streamed and 125 so; 7-point stencil 128^3 70 and 56; of at most 4:
+        // 118 and 71; more than 8 gains nothing).
+        if (__reduce_max_sync(FULL_MASK, (unsigned)(e - b)) <= kShortRow) {
+            int c[kShortRow];
+#pragma unroll
+            for (int u = 0; u < kShortRow; ++u) c[u] = b + u < e ? __ldg(ci + b + u) : 0;
+            first = last = c[0];
+#pragma unroll
+            for (int u = 0; u < kShortRow; ++u) {
+                top = max(top, (unsigned)c[u]);
+                if (u > 0 && b + u < e) {
+                    const int d = (int)((unsigned)c[u] - (unsigned)last);
+                    if (d <= 0) err |= 16;
+                    ng += d > 1;
+                    ms += d > t.lb8;
+                    last = c[u];
+                }
+            }
+            if (FEATURES && row_ok) r.add((unsigned)(e - b), first, last, ng, ms);
+            continue;
+        }
         if (FEATURES && e > b) {
             first = ci[b];
             last = ci[e - 1];
