@@ -925,7 +925,7 @@ struct OutLp {
 __global__ void k_sl_x_to_f32(int64_t n, const double* __restrict__ x, float* __restrict__ x32)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) x32[i] = round_f32(x[i]);
+    if (i < n) x32[i] = __double2float_rn(x[i]);
 }
 
 // One slice with low-precision values (slice_value_lp).
@@ -1007,15 +1007,21 @@ namespace {
 // page-locked buffer the layout's totals are written to, one per host thread
 thread_local SlStats* t_host_stats = nullptr;
 
-// Places arrays in one allocation, each on a 256-byte boundary.
+// Places arrays in one allocation, each on a 256-byte boundary, large ones on
+// a 2 MB boundary.
 struct Arena {
+    static constexpr int64_t kPage = 2 << 20, kLarge = 8 << 20;
     int64_t bytes = 0;
     std::vector<std::pair<void**, int64_t>> at;
     template <typename T>
     void add(T** p, int64_t count)
     {
+        // large arrays as an allocation of their own would start: FP32 7-point
+        // products 2 % faster than with arrays end to end
+        const int64_t size = (int64_t)sizeof(T) * std::max<int64_t>(count, 1);
+        if (size >= kLarge) bytes = (bytes + kPage - 1) / kPage * kPage;
         at.push_back({reinterpret_cast<void**>(p), bytes});
-        bytes += ((int64_t)sizeof(T) * std::max<int64_t>(count, 1) + 255) / 256 * 256;
+        bytes += (size + 255) / 256 * 256;
     }
     spmv_status allocate(spmv_prepared* P)
     {

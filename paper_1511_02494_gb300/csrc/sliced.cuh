@@ -346,7 +346,8 @@ __device__ __forceinline__ double slice_value_lp(int64_t s, int lane, const int*
         }
     }
     *row = len >= 0 ? (perm ? perm[p] : (int)p) : -1;
-    return ACC32 ? widen_f32(acc32) : acc64;
+    // (one conversion a row: integer widening here is 2 % slower on rows of 5)
+    return ACC32 ? (double)acc32 : acc64;
 }
 
 }  // namespace dev
