@@ -1010,7 +1010,7 @@ thread_local SlStats* t_host_stats = nullptr;
 // Places arrays in one allocation, each on a 256-byte boundary, large ones on
 // a 2 MB boundary.
 struct Arena {
-    static constexpr int64_t kPage = 2 << 20, kLarge = 8 << 20;
+    static constexpr int64_t kPage = 2 << 20, kLarge = 4 << 20;
     int64_t bytes = 0;
     std::vector<std::pair<void**, int64_t>> at;
     template <typename T>
