@@ -580,8 +580,9 @@ spmv_status spmv_prepared_info(const spmv_prepared_t *P, spmv_prepared_info_t *i
 spmv_status spmv_prepared_export(const spmv_prepared_t *P, int32_t which, void *dst,
                                  int64_t bytes, spmv_stream_t stream);
 
-/* SPMV_ERR_TIMEOUT when a bounded device-side wait of an earlier spmv() on P
- * gave up (that call's y is then incomplete), else SPMV_OK; clears the flag.
+/* SPMV_ERR_TIMEOUT when a bounded device-side wait of an earlier spmv() or
+ * spmv_host() on P gave up (that call's y is then not to be used), else
+ * SPMV_OK; clears the flag.
  * Synchronizes `stream`. */
 spmv_status spmv_prepared_status(const spmv_prepared_t *P, spmv_stream_t stream);
 
