@@ -704,7 +704,8 @@ spmv_status spmv_stream_noalloc(const spmv_csr_t *A, const double *x, double *y,
  * nothing.  The next spmv_stream_noalloc call clears the word. */
 spmv_status spmv_stream_noalloc_status(spmv_stream_t stream);
 
-/* Releases everything P owns (device sync first).  NULL is ignored.  A
+/* Releases everything P owns (waits for the device P was prepared on first,
+ * whichever device is current).  NULL is ignored.  A
  * LATENCY object whose x exceeds half the L2 raised this process's
  * persisting-L2 carve-out when it was prepared; freeing the last such object
  * on the device releases the persisting lines and puts the carve-out back, so

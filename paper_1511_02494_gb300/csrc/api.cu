@@ -68,7 +68,7 @@ struct DevicePool {
 std::mutex g_pool_mu;
 DevicePool g_pool[kMaxDevices];
 
-// g_pool_mu held
+// g_pool_mu held; d is the current device (its stream is made here)
 cudaError_t pool_open(int d)
 {
     DevicePool& g = g_pool[d];
@@ -1039,8 +1039,14 @@ spmv_status spmv_prepared_status(const spmv_prepared_t* P, spmv_stream_t stream)
 void spmv_prepared_free(spmv_prepared_t* P)
 {
     if (!P) return;
+    // the pool orders a free with no stream of the caller's, so P's own
+    // device, which need not be the current one, is waited for
+    int cur = P->device;
+    cudaGetDevice(&cur);
+    if (cur != P->device) cudaSetDevice(P->device);
     cudaDeviceSynchronize();
     release(P);
+    if (cur != P->device) cudaSetDevice(cur);
     delete P;
 }
 

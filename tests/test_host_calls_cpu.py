@@ -1,0 +1,85 @@
+"""The library's host code on a CUDA runtime without a GPU (fake_cuda.cpp):
+which device waits before memory is freed, what an error leaves behind, which
+form a call takes.  Kernels do nothing here; their results are the GPU tests'."""
+import ctypes as C
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_1511_02494_gb300 import _abi, build as lib_build
+import paper_1511_02494_gb300 as sp
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+OK, NOMEM, CUDA = 0, 4, 5
+CUDA_ERROR_MEMORY = 2
+
+
+@pytest.fixture(scope="module")
+def linked(tmp_path_factory):
+    """The library's objects with the fake runtime in the place of CUDA's."""
+    lib_build.build()
+    objs = sorted(os.path.join(lib_build.OBJ, f) for f in os.listdir(lib_build.OBJ) if f.endswith(".cu.o"))
+    objs = [o for o in objs if os.path.exists(os.path.join(lib_build.CSRC, os.path.basename(o)[:-2]))]
+    out = str(tmp_path_factory.mktemp("fake") / "lib.so")
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(lib_build._nvcc()))), "include")
+    r = subprocess.run(["g++", "-std=c++17", "-fPIC", "-shared", "-I", inc, "-o", out,
+                        os.path.join(HERE, "fake_cuda.cpp"), *objs, "-Wl,-Bsymbolic"], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return out
+
+
+class Fake:
+    """A fresh instance of the library with its own runtime state."""
+
+    def __init__(self, path, devices=1):
+        self.lib = _abi.declare(C.CDLL(path))
+        self.lib.fake_log.restype = C.c_char_p
+        self.lib.fake_live.restype = self.lib.fake_reserved.restype = C.c_longlong
+        self.lib.fake_lock.argtypes = [C.c_void_p, C.c_size_t]
+        self.lib.fake_reset(devices)
+
+    def fail(self, fn, code, after=0):
+        self.lib.fake_fail(fn.encode(), after, code)
+
+    def log(self):
+        return self.lib.fake_log().decode().splitlines()
+
+    def matrix(self, n, per_row=1):
+        """n rows of per_row columns on the diagonal and after it."""
+        self.rp = np.arange(n + 1, dtype=np.int32) * per_row
+        self.ci = (np.arange(n, dtype=np.int32)[:, None] + np.arange(per_row, dtype=np.int32)).reshape(-1) % n
+        self.ci = np.ascontiguousarray(self.ci)
+        self.v = np.ones(n * per_row)
+        return _abi.CSR(n, n, self.ci.size, self.rp.ctypes.data, self.ci.ctypes.data, self.v.ctypes.data)
+
+    def prepare(self, A, variant="sliced", trusted=1, **kw):
+        h, ch = C.c_void_p(), sp.make_choice(variant, **kw)
+        st = self.lib.spmv_prepare(C.byref(A), C.byref(ch), trusted, C.byref(h), None)
+        return st, h
+
+
+@pytest.fixture
+def fake(linked, tmp_path):
+    def make(devices=1):
+        path = str(tmp_path / f"lib{len(os.listdir(tmp_path))}.so")
+        shutil.copy(linked, path)
+        return Fake(path, devices)
+    return make
+
+
+def test_free_waits_for_the_device_that_owns_the_object(fake):
+    f = fake(devices=2)
+    st, h = f.prepare(f.matrix(1000))
+    assert st == OK
+    f.lib.cudaSetDevice(1)
+    f.lib.fake_clear()
+    f.lib.spmv_prepared_free(h)
+    log = f.log()
+    frees = [i for i, ln in enumerate(log) if ln.startswith("free ")]
+    assert frees and "device 0 synchronize" in log[:frees[0]], log
+    d = C.c_int(-1)
+    f.lib.cudaGetDevice(C.byref(d))
+    assert d.value == 1 and f.lib.fake_live() == 0
