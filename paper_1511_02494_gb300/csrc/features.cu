@@ -452,15 +452,17 @@ k_feature_pass(int64_t n_rows, int64_t n_cols, int64_t nnz, const int* __restric
         // shared memory (bound by issue: 8M rows of 2, the call 188 us
         // streamed and 125 so; 7-point stencil 128^3 70 and 56; of at most 4:
         // 118 and 71; more than 8 gains nothing).
-        if (__reduce_max_sync(FULL_MASK, (unsigned)(e - b)) <= kShortRow) {
+        const int nz = e - b;
+        if (__reduce_max_sync(FULL_MASK, (unsigned)nz) <= kShortRow) {
+            // counted within the row: b + u can pass 2^31 - 1 in the last rows
             int c[kShortRow];
 #pragma unroll
-            for (int u = 0; u < kShortRow; ++u) c[u] = b + u < e ? __ldg(ci + b + u) : 0;
+            for (int u = 0; u < kShortRow; ++u) c[u] = u < nz ? __ldg(ci + b + u) : 0;
             first = last = c[0];
 #pragma unroll
             for (int u = 0; u < kShortRow; ++u) {
                 top = max(top, (unsigned)c[u]);
-                if (u > 0 && b + u < e) {
+                if (u > 0 && u < nz) {
                     const int d = (int)((unsigned)c[u] - (unsigned)last);
                     if (d <= 0) err |= 16;
                     ng += d > 1;
@@ -468,7 +470,7 @@ k_feature_pass(int64_t n_rows, int64_t n_cols, int64_t nnz, const int* __restric
                     last = c[u];
                 }
             }
-            if (FEATURES && row_ok) r.add((unsigned)(e - b), first, last, ng, ms);
+            if (FEATURES && row_ok) r.add((unsigned)nz, first, last, ng, ms);
             continue;
         }
         if (FEATURES && e > b) {
