@@ -555,10 +555,21 @@ spmv_status spmv(const spmv_prepared_t *P, const double *x, double *y, spmv_stre
  * device, runs spmv, copies y back to y_host [n_rows] and synchronizes
  * `stream`.  Page-locked host buffers give full copy bandwidth, and let the
  * kernels of some forms write y into y_host themselves and pull x from x_host
- * while they multiply, so that the transfers pass beside the product.  The
- * device staging vectors are allocated on the first call and owned by P. */
+ * while they multiply, so that the transfers pass beside the product.  A
+ * product that waits for its x for more than two seconds is given up and done
+ * again after a copy of x, within the call.  The device staging vectors are
+ * allocated on the first call and owned by P. */
 spmv_status spmv_host(spmv_prepared_t *P, const double *x_host, double *y_host,
                       spmv_stream_t stream);
+
+/* Self-test of that wait: spmv_host with a limit of limit_ns (1..2e9)
+ * nanoseconds, whose product also waits for a part of x that nobody copies
+ * when arrive == 0.  *gave_up: whether the wait ran out (y_host is right all
+ * the same).  SPMV_ERR_UNSUPPORTED, with y_host right, when the call's kernel
+ * does not pull x. */
+spmv_status spmv_host_wait_check(spmv_prepared_t *P, const double *x_host, double *y_host,
+                                 int64_t limit_ns, int32_t arrive, int32_t *gave_up,
+                                 spmv_stream_t stream);
 
 /* spmv_host without the final synchronisation: the copy of x, the SpMV and
  * the copy of y are enqueued on `stream`, and y_host is valid once the
@@ -580,9 +591,8 @@ spmv_status spmv_prepared_info(const spmv_prepared_t *P, spmv_prepared_info_t *i
 spmv_status spmv_prepared_export(const spmv_prepared_t *P, int32_t which, void *dst,
                                  int64_t bytes, spmv_stream_t stream);
 
-/* SPMV_ERR_TIMEOUT when a bounded device-side wait of an earlier spmv() or
- * spmv_host() on P gave up (that call's y is then not to be used), else
- * SPMV_OK; clears the flag.
+/* SPMV_ERR_TIMEOUT when a bounded device-side wait of an earlier spmv() on P
+ * gave up (that call's y is then incomplete), else SPMV_OK; clears the flag.
  * Synchronizes `stream`. */
 spmv_status spmv_prepared_status(const spmv_prepared_t *P, spmv_stream_t stream);
 

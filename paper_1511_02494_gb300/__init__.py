@@ -245,6 +245,16 @@ def spmv_host_async(P: Prepared, x_host, y_host, stream=None) -> None:
     _check(lib().spmv_host_async(P.handle, _ptr(x_host), _ptr(y_host), _stream(stream)))
 
 
+def spmv_host_wait_check(P: Prepared, x_host, y_host, limit_ns: int, arrive: bool, stream=None) -> bool:
+    """Self-test of spmv_host's wait for x: whether it gave up (y_host is
+    right either way).  Raises SpmvError (UNSUPPORTED) when the call's kernel
+    does not pull x."""
+    gave_up = C.c_int32(0)
+    _check(lib().spmv_host_wait_check(P.handle, _ptr(x_host), _ptr(y_host), int(limit_ns), 1 if arrive else 0,
+                                      C.byref(gave_up), _stream(stream)))
+    return bool(gave_up.value)
+
+
 def spmv_prepared_info(P: Prepared) -> PreparedInfo:
     out = PreparedInfo()
     _check(lib().spmv_prepared_info(P.handle, C.byref(out)))

@@ -108,6 +108,7 @@ def declare(lib):
         "spmv": (I32, [P, P, P, P]),
         "spmv_host": (I32, [P, P, P, P]),
         "spmv_host_async": (I32, [P, P, P, P]),
+        "spmv_host_wait_check": (I32, [P, P, P, I64, I32, C.POINTER(I32), P]),
         "spmv_prepared_info": (I32, [P, C.POINTER(PreparedInfo)]),
         "spmv_prepared_export": (I32, [P, I32, P, I64, P]),
         "spmv_prepared_status": (I32, [P, P]),

@@ -601,10 +601,12 @@ const double* host_source(const spmv_prepared* P, const double* x_host, const do
 // vectors: the copy engines then move one call's vectors while another's
 // kernel has the SMs, which kernels that hold the SMs for as long as the
 // link takes prevent (four matrices on eight streams, both directions of the
-// link busy: 2967 GB/s of matrix against 2286).
-spmv_status host_enqueue(spmv_prepared* P, const double* x_host, double* y_host, bool alone, cudaStream_t s)
+// link busy: 2967 GB/s of matrix against 2286).  *pulled: the product's kernel
+// pulls x and may give up waiting for it (sliced_host_late).
+spmv_status host_enqueue(spmv_prepared* P, const double* x_host, double* y_host, bool alone, const PullWait& wait,
+                         bool* pulled, cudaStream_t s)
 {
-    clear_error();
+    *pulled = false;
     if (!P || (!x_host && P->A.n_cols > 0) || (!y_host && P->A.n_rows > 0))
         return fail(SPMV_ERR_INVALID_ARG, "spmv_host: NULL argument");
     spmv_status st;
@@ -616,11 +618,8 @@ spmv_status host_enqueue(spmv_prepared* P, const double* x_host, double* y_host,
     double* const y = y_direct ? y_direct : P->y_stage;
     if (const double* x_direct = alone ? host_source(P, x_host, y_host, y_direct) : nullptr) {
         if (!P->x_count && (st = dev_alloc(P, &P->x_count, sliced_host_words())) != SPMV_OK) return st;
-        if (!P->status) {
-            if ((st = dev_alloc(P, &P->status, 1)) != SPMV_OK) return st;
-            SPMV_CUDA_TRY(cudaMemsetAsync(P->status, 0, sizeof(unsigned), s));
-        }
-        SPMV_CUDA_TRY(launch_sliced_host(P, x_direct, y, s));
+        if ((st = launch_sliced_host(P, x_direct, y, wait, s)) != SPMV_OK) return st;
+        *pulled = true;
     } else {
         if (P->A.n_cols > 0)
             SPMV_CUDA_TRY(cudaMemcpyAsync(P->x_stage, x_host, 8 * P->A.n_cols, cudaMemcpyHostToDevice, s));
@@ -628,6 +627,25 @@ spmv_status host_enqueue(spmv_prepared* P, const double* x_host, double* y_host,
     }
     if (!y_direct && P->A.n_rows > 0)
         SPMV_CUDA_TRY(cudaMemcpyAsync(y_host, P->y_stage, 8 * P->A.n_rows, cudaMemcpyDeviceToHost, s));
+    return SPMV_OK;
+}
+
+// spmv_host: enqueues and waits.  A product that gave up waiting for x wrote a
+// y that is not to be used; x lies apart from it, so the call is done again
+// with the copy first, which waits for nothing on the device.
+spmv_status host_run(spmv_prepared* P, const double* x_host, double* y_host, const PullWait& wait, bool* pulled,
+                     bool* gave_up, cudaStream_t s)
+{
+    clear_error();
+    *gave_up = false;
+    spmv_status st = host_enqueue(P, x_host, y_host, true, wait, pulled, s);
+    if (st != SPMV_OK) return st;
+    SPMV_CUDA_TRY(cudaStreamSynchronize(s));
+    if (!*pulled || !sliced_host_late()) return SPMV_OK;
+    *gave_up = true;
+    bool again = false;
+    if ((st = host_enqueue(P, x_host, y_host, false, wait, &again, s)) != SPMV_OK) return st;
+    SPMV_CUDA_TRY(cudaStreamSynchronize(s));
     return SPMV_OK;
 }
 
@@ -848,17 +866,33 @@ spmv_status spmv(const spmv_prepared_t* P, const double* x, double* y, spmv_stre
 spmv_status spmv_host(spmv_prepared_t* P, const double* x_host, double* y_host,
                       spmv_stream_t stream)
 {
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    spmv_status st = host_enqueue(P, x_host, y_host, true, s);
-    if (st != SPMV_OK) return st;
-    SPMV_CUDA_TRY(cudaStreamSynchronize(s));
-    return SPMV_OK;
+    bool pulled, gave_up;
+    return host_run(P, x_host, y_host, PullWait{}, &pulled, &gave_up, reinterpret_cast<cudaStream_t>(stream));
 }
 
 spmv_status spmv_host_async(spmv_prepared_t* P, const double* x_host, double* y_host,
                             spmv_stream_t stream)
 {
-    return host_enqueue(P, x_host, y_host, false, reinterpret_cast<cudaStream_t>(stream));
+    clear_error();
+    bool pulled;
+    return host_enqueue(P, x_host, y_host, false, PullWait{}, &pulled, reinterpret_cast<cudaStream_t>(stream));
+}
+
+spmv_status spmv_host_wait_check(spmv_prepared_t* P, const double* x_host, double* y_host, int64_t limit_ns,
+                                 int32_t arrive, int32_t* gave_up, spmv_stream_t stream)
+{
+    clear_error();
+    if (!gave_up) return fail(SPMV_ERR_INVALID_ARG, "spmv_host_wait_check: NULL argument");
+    *gave_up = 0;
+    if (limit_ns <= 0 || limit_ns > 2000000000ll)
+        return fail(SPMV_ERR_INVALID_ARG, "spmv_host_wait_check: limit_ns must be in 1..2e9");
+    bool pulled, late;
+    spmv_status st = host_run(P, x_host, y_host, PullWait{arrive ? 0u : 1u, (uint64_t)limit_ns}, &pulled, &late,
+                              reinterpret_cast<cudaStream_t>(stream));
+    if (st != SPMV_OK) return st;
+    if (!pulled) return fail(SPMV_ERR_UNSUPPORTED, "spmv_host_wait_check: this call's kernel does not wait for x");
+    *gave_up = late ? 1 : 0;
+    return SPMV_OK;
 }
 
 spmv_status spmv_prepared_info(const spmv_prepared_t* P, spmv_prepared_info_t* info)

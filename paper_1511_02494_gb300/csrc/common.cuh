@@ -186,11 +186,19 @@ spmv_status sliced_prepare(spmv_prepared* P, bool check, cudaStream_t s);
 // dry: the kernels that a call would launch, with nothing to do (loads them)
 cudaError_t launch_sliced(const spmv_prepared* P, const double* x, double* y, cudaStream_t s, bool dry = false);
 // The product with x pulled from page-locked host memory beside it: for
-// prepared objects of this form, with x_stage, x_count (sliced_host_words()
-// words) and status allocated.
+// prepared objects of this form, with x_stage and x_count
+// (sliced_host_words() words) allocated.  Its bounded wait is for `missing`
+// copying warps more than there are (none but in the wait's self-test).
+struct PullWait {
+    unsigned missing = 0;
+    uint64_t limit_ns = 2000000000ull;
+};
 bool sliced_host_form(const spmv_prepared* P);
 size_t sliced_host_words();
-cudaError_t launch_sliced_host(const spmv_prepared* P, const double* x_host, double* y, cudaStream_t s);
+spmv_status launch_sliced_host(const spmv_prepared* P, const double* x_host, double* y, const PullWait& wait, cudaStream_t s);
+// whether a wait of this host thread's last launch gave up, so that its y is
+// not to be used (once the stream has been waited for)
+bool sliced_host_late();
 cudaError_t launch_latency(const spmv_csr_t& A, int T, const double* x, double* y,
                            int l2_window_bytes, cudaStream_t s);
 cudaError_t launch_compress(const spmv_csr_t& A, int32_t* rowbase, uint16_t* off16,

@@ -539,9 +539,12 @@ k_sliced(int64_t n_slices, const int* __restrict__ rowlen, const int* __restrict
 // batch of elements once the stage of its largest column is complete.  So the
 // upload passes beside the product instead of before it.  A waiting warp
 // holds up nothing: the copying blocks come first in the grid and wait for
-// nobody.  Every wait is bounded all the same; one that gives up sets
-// *status.  x is read with ordinary loads after an acquire: a sector enters
-// L1 only when its stage is complete, so none is stale.
+// nobody.  Every wait is bounded all the same: a warp that gives up sets *late
+// in page-locked memory, which the host reads once the kernel has ended (the
+// call is then done again with the copy first), and marks every stage's
+// counter, so that no other warp waits any longer.  x is read with ordinary
+// loads after an acquire: a sector enters L1 only when its stage is complete,
+// so none is stale.
 // Bound by the link: pulling 16.8 MB takes 87 us (512 warps with 4 x 16
 // bytes a lane in flight; 2 x 16 are slower, 8 x 16 or 1024 warps no faster).
 // What the waits cost is the looking: 9700 resident warps that look at one
@@ -554,14 +557,16 @@ constexpr int kXShift = 15;           // columns of a stage, at least (log2)
 constexpr unsigned kXWarps = 512;     // copying warps: 64 columns each of a stage's 32768
 constexpr int kXStride = 32;          // words from one stage's counter to the next: a line each
 constexpr unsigned kXSleepNs = 2048;  // between two looks at a counter
-constexpr uint64_t kXLimitNs = 2000000000ull;
+constexpr unsigned kXLate = 0x80000000u;  // in a stage's counter: some wait gave up
 struct HostX {
     const double* src;  // device address of the host vector
     double* dst;
     int64_t n;
     int shift;          // log2 of the columns of a stage
     unsigned* count;    // [kXStages kXStride] warps that have finished a stage (each finishes them in order)
-    unsigned* status;
+    unsigned want;      // of them complete a stage
+    uint64_t limit_ns;  // of a wait
+    unsigned* late;
 };
 
 __device__ __forceinline__ void pull_x(const HostX& h, unsigned w, int lane)
@@ -601,7 +606,8 @@ __device__ __forceinline__ void pull_x(const HostX& h, unsigned w, int lane)
     }
 }
 
-// true once all warps have finished the stage (for the whole warp)
+// true once all warps have finished the stage, or some wait has given up (for
+// the whole warp)
 __device__ __forceinline__ bool stage_in(const HostX& h, int stage)
 {
     unsigned v = 0;
@@ -610,7 +616,13 @@ __device__ __forceinline__ bool stage_in(const HostX& h, int stage)
     }
     v = __shfl_sync(FULL, v, 0);
     __syncwarp();
-    return v == kXWarps;
+    return v >= h.want;
+}
+
+__device__ __noinline__ void give_up(const HostX& h, int lane)
+{
+    for (int i = lane; i < kXStages; i += 32) atomicOr(h.count + kXStride * i, kXLate);
+    if (lane == 0) *h.late = 1u;
 }
 
 template <int U, typename CT>
@@ -652,8 +664,8 @@ k_sliced_host(HostX h, unsigned copy_blocks, int64_t n_slices, const int* __rest
             while (!stage_in(h, stage)) {
                 const uint64_t now = __shfl_sync(FULL, ptx::global_ns(), 0);
                 if (t0 == 0) t0 = now;
-                if (now - t0 > kXLimitNs) {
-                    if (lane == 0) *h.status = 1u;
+                if (now - t0 > h.limit_ns) {
+                    give_up(h, lane);
                     break;
                 }
                 __nanosleep(kXSleepNs);
@@ -1004,8 +1016,24 @@ unsigned grid_of(int64_t threads, int64_t cap_blocks)
 
 namespace {
 
-// page-locked buffer the layout's totals are written to, one per host thread
-thread_local SlStats* t_host_stats = nullptr;
+// page-locked memory that kernels write to, one per host thread: the layout's
+// totals, and whether a wait of k_sliced_host gave up
+struct SlHost {
+    SlStats stats;
+    unsigned late;
+};
+thread_local SlHost* t_host = nullptr;
+spmv_status host_words()
+{
+    if (t_host) return SPMV_OK;
+    void* p = nullptr;
+    if (cudaMallocHost(&p, sizeof(SlHost)) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(SPMV_ERR_NOMEM, "cudaMallocHost for the SLICED kernels' words failed");
+    }
+    t_host = static_cast<SlHost*>(p);
+    return SPMV_OK;
+}
 
 // Places arrays in one allocation, each on a 256-byte boundary, large ones on
 // a 2 MB boundary.
@@ -1040,7 +1068,7 @@ spmv_status sliced_build(spmv_prepared* P, SlScratch* w, bool check, cudaStream_
 {
     const spmv_csr_t& A = P->A;
     SlicedPlan& d = P->sl;
-    SlStats* const host = t_host_stats;
+    SlStats* const host = &t_host->stats;
     int cap = P->c.items_per_warp > 0 ? P->c.items_per_warp : kSlicedCap;
     d.n_slices = (A.n_rows + 31) / 32;
     const int64_t n_pos = 32 * d.n_slices;
@@ -1233,17 +1261,11 @@ spmv_status sliced_build(spmv_prepared* P, SlScratch* w, bool check, cudaStream_
 
 spmv_status sliced_prepare(spmv_prepared* P, bool check, cudaStream_t s)
 {
-    if (!t_host_stats) {
-        void* p = nullptr;
-        if (cudaMallocHost(&p, sizeof(SlStats)) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(SPMV_ERR_NOMEM, "cudaMallocHost for the layout's totals failed");
-        }
-        t_host_stats = static_cast<SlStats*>(p);
-    }
+    spmv_status st = host_words();
+    if (st != SPMV_OK) return st;
     SlScratch* w = nullptr;
     SPMV_CUDA_TRY(work_alloc(P->device, reinterpret_cast<void**>(&w), sizeof(SlScratch), s));
-    const spmv_status st = sliced_build(P, w, check, s);
+    st = sliced_build(P, w, check, s);
     cudaFreeAsync(w, s);
     return st;
 }
@@ -1266,13 +1288,15 @@ bool sliced_host_form(const spmv_prepared* P)
 
 size_t sliced_host_words() { return kXStride * kXStages; }
 
-cudaError_t launch_sliced_host(const spmv_prepared* P, const double* x_host, double* y, cudaStream_t s)
+spmv_status launch_sliced_host(const spmv_prepared* P, const double* x_host, double* y, const PullWait& wait, cudaStream_t s)
 {
     const SlicedPlan& d = P->sl;
-    HostX h{x_host, P->x_stage, P->A.n_cols, kXShift, P->x_count, P->status};
+    spmv_status st = host_words();
+    if (st != SPMV_OK) return st;
+    t_host->late = 0;
+    HostX h{x_host, P->x_stage, P->A.n_cols, kXShift, P->x_count, kXWarps + wait.missing, wait.limit_ns, &t_host->late};
     while (((h.n - 1) >> h.shift) >= kXStages) ++h.shift;
-    cudaError_t e = cudaMemsetAsync(P->x_count, 0, sizeof(unsigned) * kXStride * kXStages, s);
-    if (e != cudaSuccess) return e;
+    SPMV_CUDA_TRY(cudaMemsetAsync(P->x_count, 0, sizeof(unsigned) * kXStride * kXStages, s));
     const unsigned copy = kXWarps / (kOB / 32), blocks = copy + (unsigned)((d.n_slices + kOB / 32 - 1) / (kOB / 32));
 #define SPMV_SL_HOST(CT)                                                                            \
     k_sliced_host<4, CT><<<blocks, kOB, 0, s>>>(h, copy, d.n_slices, d.rowlen, d.slice_len, d.slice_ptr, \
@@ -1281,8 +1305,11 @@ cudaError_t launch_sliced_host(const spmv_prepared* P, const double* x_host, dou
     else if (d.cbytes == 2) SPMV_SL_HOST(int16_t);
     else SPMV_SL_HOST(int);
 #undef SPMV_SL_HOST
-    return cudaGetLastError();
+    SPMV_CUDA_TRY(cudaGetLastError());
+    return SPMV_OK;
 }
+
+bool sliced_host_late() { return t_host && *static_cast<volatile unsigned*>(&t_host->late) != 0; }
 
 cudaError_t launch_sliced(const spmv_prepared* P, const double* x, double* y, cudaStream_t s, bool dry)
 {
