@@ -265,11 +265,15 @@ k_update_p(int64_t n, double* __restrict__ p, const double* __restrict__ r, cons
 // lane computes its row's q_i (dev::slice_value / slice_value_lp, the same
 // arithmetic as the SLICED kernels) and adds p_i q_i to its block's sum.
 // Resident blocks per SM of the fused kernel: FP64 values fit 4 (32
-// registers, two elements in flight per lane); the low-precision bodies need
-// 40 registers, so 3.
+// registers, four elements in flight per lane as in the SLICED product), the
+// low-precision bodies need 40 registers, so 3.  Two elements in flight leave
+// the FP64 kernel waiting on its gathers, at the mercy of the order in which
+// the compiler places them: an iteration of 128^3 rows takes 200 us (27-point)
+// and 78 (7-point), with the row looked up before the loop 182 and 75; four
+// take 153 and 72, three 151 and 76, four on 48 warps of 40 registers 172 and 73.
 template <typename VT>
 constexpr int dot_blocks() { return sizeof(VT) == 8 ? 4 : 3; }
-constexpr int kDotU = 2;
+constexpr int kDotU = 4;
 
 struct SlArgs {
     int64_t n_slices;
