@@ -384,18 +384,24 @@ cudaError_t launch_sliced_dot(const spmv_prepared* P, const double* p, double* q
 // us here against 75 / 65).  Registers instead of shared memory for the state
 // of three rows a lane are as fast; chunks of the matrix loaded ahead are not
 // faster (64^3 18.7 / 16.1).
-constexpr uint64_t kMeetLimitNs = 2000000000ull;
+// `missing` blocks more than there are are waited for (none but in the wait's
+// self-test), for at most limit_ns each time.
+struct MeetWait {
+    unsigned missing = 0;
+    uint64_t limit_ns = 2000000000ull;
+};
 
 struct Meeting {
     double* sums;       // [2][gridDim.x]
     unsigned* arrived;  // 0 at the start
+    MeetWait wait;
     unsigned turn;
 };
 
 // Arrives and waits (one thread); false when the wait gave up.
 __device__ __forceinline__ bool arrive_and_wait(Meeting& m)
 {
-    const unsigned target = m.turn * gridDim.x;
+    const unsigned target = m.turn * (gridDim.x + m.wait.missing);
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(m.arrived) : "memory");
     uint64_t t0 = 0;
     for (unsigned tries = 1;; ++tries) {
@@ -405,7 +411,7 @@ __device__ __forceinline__ bool arrive_and_wait(Meeting& m)
         if ((tries & 63) == 0) {
             const uint64_t now = ptx::global_ns();
             if (t0 == 0) t0 = now;
-            else if (now - t0 > kMeetLimitNs) return false;
+            else if (now - t0 > m.wait.limit_ns) return false;
         }
     }
 }
@@ -564,6 +570,7 @@ struct ResidentArgs {
     unsigned* arrived;
     int iters, refine;
     int per_warp;       // slices per warp
+    MeetWait wait;
 };
 
 constexpr int kResidentWarps = 24;  // most per block; one block per SM (80 registers)
@@ -585,7 +592,7 @@ k_cg_resident(const ResidentArgs a)
     double* sx = sq + span;
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * BT + threadIdx.x) >> 5, n_warps = (int64_t)gridDim.x * (BT / 32);
-    Meeting m{a.sums, a.arrived, 0};
+    Meeting m{a.sums, a.arrived, a.wait, 0};
     // row of the lane in the warp's slice j, -1 past the last
     auto row_of = [&](int j) -> int {
         const int64_t p = (warp + j * n_warps) * 32 + lane;
@@ -809,7 +816,7 @@ struct CgBufs {
 
 spmv_status enqueue_cg(const spmv_prepared* Pi, const spmv_prepared* Pe, const double* b,
                        double* x, int iters, int refine, double* resid, const CgBufs& w,
-                       unsigned grid, const Resident& res, cudaStream_t s)
+                       unsigned grid, const Resident& res, const MeetWait& wait, cudaStream_t s)
 {
     const int64_t n = Pi->A.n_rows;
     spmv_status st;
@@ -825,7 +832,7 @@ spmv_status enqueue_cg(const spmv_prepared* Pi, const spmv_prepared* Pe, const d
     if (res.kernel && iters > 0) {
         SPMV_CUDA_TRY(cudaMemsetAsync(w.arrived, 0, sizeof(unsigned), s));
         ResidentArgs a{sl_args(Pi), refine > 0 ? sl_args(Pe) : SlArgs{}, refine > 0 ? Pe->sl.cbytes : 4, n, b, x, w.r, w.p,
-                       p32, resid, w.st, w.sums, w.arrived, iters, refine, res.per_warp};
+                       p32, resid, w.st, w.sums, w.arrived, iters, refine, res.per_warp, wait};
         void* args[] = {&a};
         SPMV_CUDA_TRY(cudaLaunchCooperativeKernel(res.kernel, dim3(res.grid), dim3(res.threads), args, res.smem, s));
         return SPMV_OK;
@@ -856,11 +863,13 @@ spmv_status enqueue_cg(const spmv_prepared* Pi, const spmv_prepared* Pe, const d
 
 using namespace spmvlib;
 
-extern "C" spmv_status spmv_cg(const spmv_prepared_t* A_inner, const spmv_prepared_t* A_exact,
-                               const double* b, double* x, int32_t iters, int32_t refine_every,
-                               double* resid, int32_t use_graph, spmv_stream_t stream)
+namespace {
+
+// spmv_cg; one_launch: refuses what does not run as one launch
+spmv_status cg_run(const spmv_prepared_t* A_inner, const spmv_prepared_t* A_exact, const double* b, double* x,
+                   int32_t iters, int32_t refine_every, double* resid, int32_t use_graph, const MeetWait& wait,
+                   bool one_launch, spmv_stream_t stream)
 {
-    clear_error();
     if (!A_inner || !b || !x || iters < 0 || refine_every < 0)
         return fail(SPMV_ERR_INVALID_ARG, "spmv_cg: bad argument");
     const spmv_prepared* Pi = A_inner;
@@ -878,6 +887,8 @@ extern "C" spmv_status spmv_cg(const spmv_prepared_t* A_inner, const spmv_prepar
     const unsigned grid = (unsigned)g;
     Resident res;
     if (!resident_choice(Pi, Pe, refine_every, dev.sm_count, &res)) res = Resident{};
+    if (one_launch && (!res.kernel || iters == 0))
+        return fail(SPMV_ERR_UNSUPPORTED, "this solve does not run as one launch");
     // the work vectors in one allocation
     CgBufs w;
     const size_t n_part = std::max<size_t>(grid, fusable(Pi) ? sliced_dot_grid(Pi) : 0);
@@ -904,7 +915,7 @@ extern "C" spmv_status spmv_cg(const spmv_prepared_t* A_inner, const spmv_prepar
         SPMV_CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
         cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            st = enqueue_cg(Pi, Pe, b, x, iters, refine_every, resid, w, grid, res, cs);
+            st = enqueue_cg(Pi, Pe, b, x, iters, refine_every, resid, w, grid, res, wait, cs);
             e = cudaStreamEndCapture(cs, &graph);
         }
         cudaStreamDestroy(cs);
@@ -918,10 +929,31 @@ extern "C" spmv_status spmv_cg(const spmv_prepared_t* A_inner, const spmv_prepar
         if (graph) cudaGraphDestroy(graph);
         if (e != cudaSuccess) return cuda_fail(e, "spmv_cg graph");
     } else {
-        st = enqueue_cg(Pi, Pe, b, x, iters, refine_every, resid, w, grid, res, s);
+        st = enqueue_cg(Pi, Pe, b, x, iters, refine_every, resid, w, grid, res, wait, s);
         if (st != SPMV_OK) return st;
     }
     cudaFreeAsync(base, s);
     SPMV_CUDA_TRY(cudaGetLastError());
     return SPMV_OK;
+}
+
+}  // namespace
+
+extern "C" spmv_status spmv_cg(const spmv_prepared_t* A_inner, const spmv_prepared_t* A_exact,
+                               const double* b, double* x, int32_t iters, int32_t refine_every,
+                               double* resid, int32_t use_graph, spmv_stream_t stream)
+{
+    clear_error();
+    return cg_run(A_inner, A_exact, b, x, iters, refine_every, resid, use_graph, MeetWait{}, false, stream);
+}
+
+extern "C" spmv_status spmv_cg_wait_check(const spmv_prepared_t* A_inner, const spmv_prepared_t* A_exact,
+                                          const double* b, double* x, int32_t iters, int32_t refine_every,
+                                          double* resid, int64_t limit_ns, int32_t arrive, spmv_stream_t stream)
+{
+    clear_error();
+    if (limit_ns <= 0 || limit_ns > 2000000000ll)
+        return fail(SPMV_ERR_INVALID_ARG, "spmv_cg_wait_check: limit_ns must be in 1..2e9");
+    return cg_run(A_inner, A_exact, b, x, iters, refine_every, resid, 0, MeetWait{arrive ? 0u : 1u, (uint64_t)limit_ns},
+                  true, stream);
 }
