@@ -670,8 +670,9 @@ void spmv_batch_free(spmv_batch_t *B);
  * refining, an A_exact of that kind with FP64 values) of up to about 1.05 M
  * rows the whole loop is one cooperative kernel launch, whatever use_graph
  * says; its blocks wait for one another with a bound of two seconds, after
- * which x and the remaining entries of resid are NaN.  Otherwise use_graph !=
- * 0 captures the whole loop into a CUDA graph and launches it.  Allocates its
+ * which x and the remaining entries of resid are NaN.  Otherwise, and where the
+ * device refuses that launch (fewer SMs free to this process than it has),
+ * use_graph != 0 captures the whole loop into a CUDA graph and launches it.  Allocates its
  * work vectors (3n doubles) stream-ordered.
  * Asynchronous on `stream`; dot products are deterministic. */
 spmv_status spmv_cg(const spmv_prepared_t *A_inner, const spmv_prepared_t *A_exact,

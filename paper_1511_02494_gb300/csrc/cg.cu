@@ -814,29 +814,53 @@ struct CgBufs {
     unsigned* arrived = nullptr;
 };
 
-spmv_status enqueue_cg(const spmv_prepared* Pi, const spmv_prepared* Pe, const double* b,
-                       double* x, int iters, int refine, double* resid, const CgBufs& w,
-                       unsigned grid, const Resident& res, const MeetWait& wait, cudaStream_t s)
+// r0 = b - A x0 (exact), p0 = r0.  A SLICED inner matrix takes the fused q = A
+// p, p.q kernel; when it sums in FP32, p's FP32 copy is written by the p
+// updates.
+float* direction_copy(const spmv_prepared* Pi) { return fusable(Pi) && Pi->sl.acc32 ? Pi->sl.x32 : nullptr; }
+
+spmv_status enqueue_start(const spmv_prepared* Pi, const spmv_prepared* Pe, const double* b, double* x, double* resid,
+                          const CgBufs& w, unsigned grid, cudaStream_t s)
 {
     const int64_t n = Pi->A.n_rows;
     spmv_status st;
-    // a SLICED inner matrix takes the fused q = A p, p.q kernel; when it sums
-    // in FP32, p's FP32 copy is written by the p update
-    const bool fused = fusable(Pi);
-    float* p32 = fused && Pi->sl.acc32 ? Pi->sl.x32 : nullptr;
-    // r0 = b - A x0 (exact), p0 = r0
     if ((st = spmv(Pe, x, w.q, reinterpret_cast<spmv_stream_t>(s))) != SPMV_OK) return st;
-    const int n_pq = (int)(fused ? sliced_dot_grid(Pi) : grid), n_rr = (int)grid;
     k_update<true><<<grid, kCT, 0, s>>>(n, x, w.p, w.r, w.q, b, nullptr, 0, w.rr, w.st, 0);
-    k_update_p<kFirst><<<grid, kCT, 0, s>>>(n, w.p, w.r, w.rr, n_rr, w.st, resid, 0, p32);
-    if (res.kernel && iters > 0) {
-        SPMV_CUDA_TRY(cudaMemsetAsync(w.arrived, 0, sizeof(unsigned), s));
-        ResidentArgs a{sl_args(Pi), refine > 0 ? sl_args(Pe) : SlArgs{}, refine > 0 ? Pe->sl.cbytes : 4, n, b, x, w.r, w.p,
-                       p32, resid, w.st, w.sums, w.arrived, iters, refine, res.per_warp, wait};
-        void* args[] = {&a};
-        SPMV_CUDA_TRY(cudaLaunchCooperativeKernel(res.kernel, dim3(res.grid), dim3(res.threads), args, res.smem, s));
+    k_update_p<kFirst><<<grid, kCT, 0, s>>>(n, w.p, w.r, w.rr, (int)grid, w.st, resid, 0, direction_copy(Pi));
+    SPMV_CUDA_TRY(cudaGetLastError());
+    return SPMV_OK;
+}
+
+// The one launch after enqueue_start.  *refused: the device does not take it
+// (fewer SMs are free to this process than it has, or no cooperative launches):
+// nothing was launched.
+spmv_status enqueue_resident(const spmv_prepared* Pi, const spmv_prepared* Pe, const double* b, double* x, int iters,
+                             int refine, double* resid, const CgBufs& w, const Resident& res, const MeetWait& wait,
+                             bool* refused, cudaStream_t s)
+{
+    SPMV_CUDA_TRY(cudaMemsetAsync(w.arrived, 0, sizeof(unsigned), s));
+    ResidentArgs a{sl_args(Pi), refine > 0 ? sl_args(Pe) : SlArgs{}, refine > 0 ? Pe->sl.cbytes : 4, Pi->A.n_rows, b, x,
+                   w.r, w.p, direction_copy(Pi), resid, w.st, w.sums, w.arrived, iters, refine, res.per_warp, wait};
+    void* args[] = {&a};
+    const cudaError_t e = cudaLaunchCooperativeKernel(res.kernel, dim3(res.grid), dim3(res.threads), args, res.smem, s);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources || e == cudaErrorNotSupported) {
+        cudaGetLastError();
+        *refused = true;
         return SPMV_OK;
     }
+    if (e != cudaSuccess) return cuda_fail(e, "spmv_cg launch");
+    return SPMV_OK;
+}
+
+spmv_status enqueue_loop(const spmv_prepared* Pi, const spmv_prepared* Pe, const double* b, double* x, int iters,
+                         int refine, double* resid, const CgBufs& w, unsigned grid, cudaStream_t s)
+{
+    const int64_t n = Pi->A.n_rows;
+    spmv_status st;
+    if ((st = enqueue_start(Pi, Pe, b, x, resid, w, grid, s)) != SPMV_OK) return st;
+    const bool fused = fusable(Pi);
+    float* p32 = direction_copy(Pi);
+    const int n_pq = (int)(fused ? sliced_dot_grid(Pi) : grid), n_rr = (int)grid;
     for (int t = 1; t <= iters; ++t) {
         if (fused) {
             SPMV_CUDA_TRY(launch_sliced_dot(Pi, w.p, w.q, w.pq, s));
@@ -864,6 +888,48 @@ spmv_status enqueue_cg(const spmv_prepared* Pi, const spmv_prepared* Pe, const d
 using namespace spmvlib;
 
 namespace {
+
+// The three-kernel loop from a graph: captured on a private stream (the
+// caller's may be the legacy default stream, which cannot be captured), then
+// launched on the caller's.
+spmv_status launch_graph(const spmv_prepared* Pi, const spmv_prepared* Pe, const double* b, double* x, int iters,
+                         int refine, double* resid, const CgBufs& w, unsigned grid, cudaStream_t s)
+{
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    cudaStream_t cs = nullptr;
+    spmv_status st = SPMV_OK;
+    SPMV_CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
+    cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        st = enqueue_loop(Pi, Pe, b, x, iters, refine, resid, w, grid, cs);
+        e = cudaStreamEndCapture(cs, &graph);
+    }
+    cudaStreamDestroy(cs);
+    if (st == SPMV_OK && e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
+    if (st == SPMV_OK && e == cudaSuccess) e = cudaGraphLaunch(exec, s);
+    if (exec) cudaGraphExecDestroy(exec);
+    if (graph) cudaGraphDestroy(graph);
+    if (st == SPMV_OK && e != cudaSuccess) st = cuda_fail(e, "spmv_cg graph");
+    return st;
+}
+
+spmv_status enqueue_cg(const spmv_prepared* Pi, const spmv_prepared* Pe, const double* b, double* x, int iters,
+                       int refine, double* resid, bool use_graph, const CgBufs& w, unsigned grid, const Resident& res,
+                       const MeetWait& wait, bool one_launch, cudaStream_t s)
+{
+    spmv_status st;
+    SPMV_CUDA_TRY(cudaMemsetAsync(w.st, 0, sizeof(CgState), s));
+    if (res.kernel && iters > 0) {
+        bool refused = false;
+        if ((st = enqueue_start(Pi, Pe, b, x, resid, w, grid, s)) != SPMV_OK) return st;
+        st = enqueue_resident(Pi, Pe, b, x, iters, refine, resid, w, res, wait, &refused, s);
+        if (st != SPMV_OK || !refused) return st;
+        if (one_launch) return fail(SPMV_ERR_UNSUPPORTED, "this solve does not run as one launch");
+    }
+    return use_graph ? launch_graph(Pi, Pe, b, x, iters, refine, resid, w, grid, s)
+                     : enqueue_loop(Pi, Pe, b, x, iters, refine, resid, w, grid, s);
+}
 
 // spmv_cg; one_launch: refuses what does not run as one launch
 spmv_status cg_run(const spmv_prepared_t* A_inner, const spmv_prepared_t* A_exact, const double* b, double* x,
@@ -905,34 +971,9 @@ spmv_status cg_run(const spmv_prepared_t* A_inner, const spmv_prepared_t* A_exac
     w.st = reinterpret_cast<CgState*>(base + 3 * vec + parts);
     w.arrived = reinterpret_cast<unsigned*>(base + 3 * vec + parts + state);
     w.sums = reinterpret_cast<double*>(base + 3 * vec + parts + state + room(sizeof(unsigned)));
-    SPMV_CUDA_TRY(cudaMemsetAsync(w.st, 0, sizeof(CgState), s));
-    if (use_graph && !res.kernel) {
-        // capture on a private stream (the caller's may be the legacy default
-        // stream, which cannot be captured), then launch on the caller's
-        cudaGraph_t graph = nullptr;
-        cudaGraphExec_t exec = nullptr;
-        cudaStream_t cs = nullptr;
-        SPMV_CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-        cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-        if (e == cudaSuccess) {
-            st = enqueue_cg(Pi, Pe, b, x, iters, refine_every, resid, w, grid, res, wait, cs);
-            e = cudaStreamEndCapture(cs, &graph);
-        }
-        cudaStreamDestroy(cs);
-        if (st != SPMV_OK) {
-            if (graph) cudaGraphDestroy(graph);
-            return st;
-        }
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
-        if (e == cudaSuccess) e = cudaGraphLaunch(exec, s);
-        if (exec) cudaGraphExecDestroy(exec);
-        if (graph) cudaGraphDestroy(graph);
-        if (e != cudaSuccess) return cuda_fail(e, "spmv_cg graph");
-    } else {
-        st = enqueue_cg(Pi, Pe, b, x, iters, refine_every, resid, w, grid, res, wait, s);
-        if (st != SPMV_OK) return st;
-    }
-    cudaFreeAsync(base, s);
+    st = enqueue_cg(Pi, Pe, b, x, iters, refine_every, resid, use_graph != 0, w, grid, res, wait, one_launch, s);
+    cudaFreeAsync(base, s);  // after an error too
+    if (st != SPMV_OK) return st;
     SPMV_CUDA_TRY(cudaGetLastError());
     return SPMV_OK;
 }

@@ -83,3 +83,56 @@ def test_free_waits_for_the_device_that_owns_the_object(fake):
     d = C.c_int(-1)
     f.lib.cudaGetDevice(C.byref(d))
     assert d.value == 1 and f.lib.fake_live() == 0
+
+
+# ---- conjugate gradients ----------------------------------------------------------
+
+COOPERATIVE_TOO_LARGE = 720
+
+
+def _cg(f, h, n, iters=3, refine=0, graph=0):
+    v = np.ones((2, n))
+    return f.lib.spmv_cg(h, h, v[0].ctypes.data, v[1].ctypes.data, iters, refine, None, graph, None)
+
+
+def _kernels(log):
+    return [ln.split()[1] for ln in log if ln.startswith("kernel ")]
+
+
+@pytest.mark.parametrize("graph", [0, 1])
+@pytest.mark.parametrize("code", [COOPERATIVE_TOO_LARGE, 701, 801])
+def test_cg_runs_in_three_kernels_where_the_one_launch_is_refused(fake, code, graph):
+    f = fake()
+    st, h = f.prepare(f.matrix(1000))
+    assert st == OK
+    f.lib.fake_clear()
+    assert _cg(f, h, 1000, graph=graph) == OK
+    assert _kernels(f.log()).count("k_cg_resident") == 1 and "begin capture" not in f.log()
+    f.fail("cudaLaunchCooperativeKernel", code)
+    f.lib.fake_clear()
+    assert _cg(f, h, 1000, graph=graph) == OK
+    ran = _kernels(f.log())
+    assert "k_cg_resident" not in ran and ran.count("k_sliced_dot") == 3
+    assert ("graph launch" in f.log()) == (graph == 1)
+    f.lib.spmv_prepared_free(h)
+    assert f.lib.fake_live() == 0
+
+
+@pytest.mark.parametrize("fn,after,code,graph", [
+    ("cudaLaunchCooperativeKernel", 0, 700, 0),      # an error that is not a refusal
+    ("launch", 0, 98, 0), ("launch", 1, 98, 1),
+    ("cudaStreamCreateWithFlags", 0, 2, 1), ("cudaStreamBeginCapture", 0, 900, 1),
+    ("cudaGraphInstantiate", 0, 2, 1), ("cudaMemsetAsync", 0, 1, 0), ("cudaMemsetAsync", 1, 1, 0)])
+def test_cg_frees_its_vectors_after_an_error(fake, fn, after, code, graph):
+    f = fake()
+    st, h = f.prepare(f.matrix(1000))
+    assert st == OK
+    assert _cg(f, h, 1000) == OK                       # what a first call allocates for good
+    if graph:
+        f.fail("cudaLaunchCooperativeKernel", COOPERATIVE_TOO_LARGE)
+    before = f.lib.fake_live()
+    f.fail(fn, code, after)
+    assert _cg(f, h, 1000, graph=graph) == CUDA
+    assert f.lib.fake_live() == before
+    f.lib.spmv_prepared_free(h)
+    assert f.lib.fake_live() == 0
