@@ -668,12 +668,15 @@ void spmv_batch_free(spmv_batch_t *B);
  * Runs `iters` iterations without a convergence test (no host sync inside the
  * loop).  With a SLICED A_inner without long rows or coded columns (and, when
  * refining, an A_exact of that kind with FP64 values) of up to about 1.05 M
- * rows the whole loop is one cooperative kernel launch, whatever use_graph
- * says; its blocks wait for one another with a bound of two seconds, after
- * which x and the remaining entries of resid are NaN.  Otherwise, and where the
- * device refuses that launch (fewer SMs free to this process than it has),
- * use_graph != 0 captures the whole loop into a CUDA graph and launches it.  Allocates its
- * work vectors (3n doubles) stream-ordered.
+ * rows, whose stored arrays take at most nine tenths of the L2 (seven tenths
+ * with FP32 or BF16 values), the whole loop is one cooperative kernel launch,
+ * whatever use_graph says; its blocks wait for one another with a bound of two
+ * seconds, after which x and the remaining entries of resid are NaN.  Above
+ * some 40,000 rows that launch takes every SM, so that such solves on several
+ * streams run one after another.  Otherwise, and where the device refuses the
+ * launch (fewer SMs free to this process than it has), use_graph != 0 captures
+ * the whole loop into a CUDA graph and launches it.  Allocates its work vectors
+ * (3n doubles) stream-ordered.
  * Asynchronous on `stream`; dot products are deterministic. */
 spmv_status spmv_cg(const spmv_prepared_t *A_inner, const spmv_prepared_t *A_exact,
                     const double *b, double *x, int32_t iters, int32_t refine_every,

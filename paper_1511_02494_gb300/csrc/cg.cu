@@ -354,14 +354,13 @@ cudaError_t launch_sliced_dot(const spmv_prepared* P, const double* p, double* q
 
 // ---- the whole loop in one launch --------------------------------------------
 // For small and middle-sized matrices the loop is bound not by memory but by
-// launches: three kernels an iteration, each a few microseconds of latency
-// and each with a last block that sums the others' partials (14.4 us an
-// iteration at 36,000 rows).  Here one cooperative launch, one block per SM,
-// runs every iteration.  A lane owns the same rows for the whole solve and
-// keeps their x, r, p and q in shared memory, so per iteration only p (or its
-// FP32 copy) goes through memory, and the blocks meet three times: for p.q,
-// for r.r and when p is written.  The slices go round the warps of the grid;
-// with up to three per warp their heads stay in registers (RT).
+// launches and latency: three kernels an iteration, each a few microseconds
+// of it (15 us an iteration at 36,000 rows).  Here one cooperative launch, one
+// block per SM, runs every iteration.  A lane owns the same rows for the whole
+// solve and keeps their x, r, p and q in shared memory, so per iteration only p
+// (or its FP32 copy) goes through memory, and the blocks meet three times: for
+// p.q, for r.r and when p is written.  The slices go round the warps of the
+// grid; with up to three per warp their heads stay in registers (RT).
 //
 // A meeting: the block's first warp adds the block's values, stores the sum,
 // arrives at one counter and waits until every block has; then it adds all
@@ -375,15 +374,24 @@ cudaError_t launch_sliced_dot(const spmv_prepared* P, const double* p, double* q
 // (all blocks resident), and each wait is bounded all the same: a block that
 // gives up sets x and the remaining residuals to NaN and returns.
 //
-// Measured per iteration, against three launches from a graph, 7-point
-// Laplacians with FP64 / BF16 values: 33^3 rows 8.8 / 8.9 us against 14.4 /
-// 14.6, 64^3 17.7 / 15.3 against 22.7 / 21.4, 100^3 35.3 / 29.9 against 45.4 /
-// 37.0; 27-point 64^3 33.0 / 22.0 against 36.2 / 26.6.  Beyond the shared
-// memory of the chip (1.05 M rows) the state would go through memory again,
-// and the three kernels with their 64 warps per SM are faster (128^3: 82 / 71
-// us here against 75 / 65).  Registers instead of shared memory for the state
-// of three rows a lane are as fast; chunks of the matrix loaded ahead are not
-// faster (64^3 18.7 / 16.1).
+// Measured per iteration, against three launches from a graph, FP64 / BF16
+// values: 7-point Laplacians of 33^3 rows 8.6 / 8.8 us against 14.7 / 14.5, 48^3
+// 12.0 / 11.0 against 17.0 / 15.6, 64^3 17.5 / 14.9 against 22.1 / 17.8, 90^3
+// 28.5 / 23.7 against 36.6 / 27.0, 101^3 36.0 / 28.0 against 44.3 / 33.0;
+// 27-point 48^3 17.6 / 14.0 against 25.6 / 20.8, 64^3 34.3 / 22.6 against 36.0 /
+// 25.7 (where it ends: resident_choice).  Beyond the shared memory of the chip
+// (1.05 M rows) the state would go through memory again, and the three kernels
+// with their 64 warps per SM are faster (128^3: 82 / 71 us here against 72 /
+// 60).  Registers instead of shared memory for the state of three rows a lane
+// are as fast; chunks of the matrix loaded ahead are not faster (64^3 18.7 /
+// 16.1).
+//
+// A solve above 40,000 rows or so takes every SM, so that several on as many
+// streams run one after another, where the three kernels of several overlap.
+// Two such solves are no slower for it, many of middle size are: 16 of 200
+// iterations on 8 streams take 12.5 ms at 33^3 rows (three kernels 20.4), 37.2 at
+// 48^3 (22.5), 55 at 64^3 (38.5), 91 at 90^3 (98.7).
+//
 // `missing` blocks more than there are are waited for (none but in the wait's
 // self-test), for at most limit_ns each time.
 struct MeetWait {
@@ -786,11 +794,38 @@ bool resident_fits(int64_t n_slices, int sm_count, Resident* out)
 
 bool fp64_sliced(const spmv_prepared* P) { return fusable(P) && P->sl.value_type == SPMV_VAL_F64; }
 
-// whether the whole loop runs in one launch, and with which kernel
-bool resident_choice(const spmv_prepared* Pi, const spmv_prepared* Pe, int refine, int sm_count, Resident* out)
+// What a product of P reads every time: elements (padding included), the
+// positions' headers and the gathered vector.
+int64_t product_bytes(const spmv_prepared* P)
+{
+    const SlicedPlan& d = P->sl;
+    const bool f64 = d.value_type == SPMV_VAL_F64;
+    const int vb = f64 ? 8 : d.value_type == SPMV_VAL_F32 ? 4 : 2, cb = f64 ? d.cbytes : d.off16 ? 2 : 4;
+    return (vb + cb) * d.tot + (d.off16 ? 268 : 140) * d.n_slices + (d.acc32 ? 4 : 8) * P->A.n_cols;
+}
+
+// Whether the whole loop runs in one launch, and with which kernel: a product
+// whose operands stay in the L2 from one iteration to the next waits for
+// latency, which the one launch has less of; a larger one streams from memory,
+// for which 24 warps per SM keep less in flight than the product kernel's 64
+// (or 48).  The line lies at nine tenths of the L2 for FP64 values and at seven
+// tenths for FP32 and BF16 ones, whose product takes less time for the same
+// bytes.  An iteration here / in three kernels, us, by product_bytes (an L2 of
+// 135.5 MB):
+//   FP64  7-point 101^3   99 MB 36 / 46  band 524288 x 17 113 MB  44 / 47
+//         27-point 72^3  126 MB 47 / 45  band 262144 x 41 132 MB  50 / 46
+//         27-point 90^3  245 MB 74 / 66  band 1.04 M x 41 525 MB 130 / 115
+//   BF16  27-point 80^3   64 MB 31 / 39  27-point 90^3     91 MB  44 / 48
+//         band 1.04 M x 17 96 MB 51 / 48 band 524288 x 41  99 MB  51 / 47
+//         27-point 100^3 124 MB 75 / 60  band 1.04 M x 41 196 MB  98 / 74
+//   FP32  27-point 80^3   92 MB 39 / 45  band 524288 x 25  95 MB  33 / 43
+//         band 786432 x 17 104 MB 46 / 46 band 393216 x 41 109 MB 50 / 45
+bool resident_choice(const spmv_prepared* Pi, const spmv_prepared* Pe, int refine, const DeviceInfo& dev, Resident* out)
 {
     if (!fusable(Pi) || (refine > 0 && !fp64_sliced(Pe))) return false;
     const SlicedPlan& d = Pi->sl;
+    const int sm_count = dev.sm_count;
+    if (10 * product_bytes(Pi) > (d.value_type == SPMV_VAL_F64 ? 9 : 7) * (int64_t)dev.l2_bytes) return false;
     if (d.value_type == SPMV_VAL_F64) {
         if (d.cbytes == 1) return resident_fits<double, false, false, int8_t>(d.n_slices, sm_count, out);
         if (d.cbytes == 2) return resident_fits<double, false, false, int16_t>(d.n_slices, sm_count, out);
@@ -952,7 +987,7 @@ spmv_status cg_run(const spmv_prepared_t* A_inner, const spmv_prepared_t* A_exac
     if (g > (int64_t)dev.sm_count * 2) g = (int64_t)dev.sm_count * 2;
     const unsigned grid = (unsigned)g;
     Resident res;
-    if (!resident_choice(Pi, Pe, refine_every, dev.sm_count, &res)) res = Resident{};
+    if (!resident_choice(Pi, Pe, refine_every, dev, &res)) res = Resident{};
     if (one_launch && (!res.kernel || iters == 0))
         return fail(SPMV_ERR_UNSUPPORTED, "this solve does not run as one launch");
     // the work vectors in one allocation

@@ -105,3 +105,39 @@ def test_solves_that_do_not_run_as_one_launch(form):
     with pytest.raises(sp.SpmvError, match="does not run as one launch"):
         sp.spmv_cg_wait_check(P, b, x, iters, LIMIT, False, refine, E)
     assert not x.any()
+
+
+def _band(n, width):
+    """Rows of `width` columns around the diagonal, as many as lie inside."""
+    c = torch.arange(n, device="cuda")[:, None] + torch.arange(-(width // 2), width - width // 2, device="cuda")
+    keep = (c >= 0) & (c < n)
+    rp = torch.cat([torch.zeros(1, dtype=torch.int64, device="cuda"), keep.sum(1).cumsum(0)]).to(torch.int32)
+    ci = c[keep].to(torch.int32)
+    v = torch.where(ci == torch.repeat_interleave(torch.arange(n, device="cuda"), keep.sum(1)), 2.0 * width, -1.0)
+    return sp.DeviceCSR(n, n, rp, ci, v.to(torch.float64))
+
+
+@pytest.mark.parametrize("kw,bytes_a_slot,head,vector,tenths", [
+    ({}, 12, 140, 8, 9), (dict(index_bytes=2), 10, 140, 8, 9), (dict(value_type=sp.VAL_F32), 6, 268, 4, 7),
+    (dict(value_type=sp.VAL_BF16), 4, 268, 4, 7), (dict(value_type=sp.VAL_BF16, accumulate=sp.ACC_F64), 4, 268, 8, 7)])
+def test_one_launch_while_the_product_fits_the_l2(kw, bytes_a_slot, head, vector, tenths):
+    """Rows of 40 (whole groups of four): the row counts, in slices, just
+    inside and just past the limit; both solve the system."""
+    l2 = torch.cuda.get_device_properties(0).L2_cache_size
+    slices = tenths * l2 // 10 // (32 * 40 * bytes_a_slot + head + 32 * vector)
+    for n, one in ((32 * (slices - 1), True), (32 * (slices + 2), False)):
+        A = _band(n, 40)
+        P, E = sp.spmv_prepare(A, sp.make_choice("sliced", block_nnz=1, **kw)), sp.spmv_prepare(A, sp.make_choice("sliced"))
+        b, x, r = _vectors(n, 6)
+        if one:
+            sp.spmv_cg_wait_check(P, b, x, 6, LONG, True, 3, E, r)
+        else:
+            with pytest.raises(sp.SpmvError, match="does not run as one launch"):
+                sp.spmv_cg_wait_check(P, b, x, 6, LONG, True, 3, E, r)
+        x.zero_()
+        sp.spmv_cg(P, b, x, 6, 3, A_exact=E, resid=r)
+        y = torch.empty_like(b)
+        sp.spmv(E, x, y)
+        left = float(torch.linalg.vector_norm(b - y))
+        # the last iteration refined: the residual is the FP64 one of x
+        assert abs(float(r[-1]) - left) <= 1e-9 * float(r[0]) and left < 0.5 * float(r[0])
