@@ -797,10 +797,7 @@ spmv_status spmv_prepare(const spmv_csr_t* A, const spmv_choice_t* c, int32_t tr
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     // SLICED reads the verdict of the validation at the first wait of its own
     const bool check_later = !trusted && c->variant == SPMV_V7_SLICED && A->n_rows > 0;
-    if (!trusted) {
-        st = check_later ? feature_pass_enqueue(A, 128, false, s) : run_feature_pass(A, 128, nullptr, s);
-        if (st != SPMV_OK) return st;
-    }
+    if (!trusted && !check_later && (st = run_feature_pass(A, 128, nullptr, s)) != SPMV_OK) return st;
     DeviceInfo dev;
     if ((st = current_device(&dev)) != SPMV_OK) return st;
     spmv_prepared_t* P = new (std::nothrow) spmv_prepared_t();
@@ -813,7 +810,10 @@ spmv_status spmv_prepare(const spmv_csr_t* A, const spmv_choice_t* c, int32_t tr
         delete P;
         return st;
     }
-    st = prepare_impl(P, check_later, s);
+    // from here on an error waits for the stream before it returns: the caller
+    // may free the matrix then
+    if (check_later) st = feature_pass_enqueue(A, 128, false, s);
+    if (st == SPMV_OK) st = prepare_impl(P, check_later, s);
     if (st == SPMV_OK && (c->variant != SPMV_V7_SLICED || A->n_rows == 0)) {
         cudaError_t e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) st = cuda_fail(e, "spmv_prepare");

@@ -24,7 +24,7 @@ struct Range {
     size_t bytes;
 };
 struct Fault {
-    int after, code;  // the call after `after` more returns code
+    int after, code;  // the call after `after` more returns code; every call when after < 0
 };
 std::recursive_mutex mu;
 std::string lines;
@@ -56,9 +56,11 @@ cudaError_t result(const char* fn)
     std::lock_guard<std::recursive_mutex> lk(mu);
     auto f = faults.find(fn);
     if (f == faults.end()) return cudaSuccess;
-    if (f->second.after-- > 0) return cudaSuccess;
     const int code = f->second.code;
-    faults.erase(f);
+    if (f->second.after >= 0) {
+        if (f->second.after-- > 0) return cudaSuccess;
+        faults.erase(f);
+    }
     log("%s fails", fn);
     return last = (cudaError_t)code;
 }
@@ -169,8 +171,9 @@ cudaError_t cudaMalloc(void** p, size_t bytes)
 cudaError_t cudaFree(void* p) { log("device %d cudaFree", device); give(p); return cudaSuccess; }
 cudaError_t cudaMallocHost(void** p, size_t bytes)
 {
-    *p = calloc(bytes, 1);
-    return cudaSuccess;
+    const cudaError_t e = result("cudaMallocHost");
+    if (e == cudaSuccess) *p = calloc(bytes, 1);
+    return e;
 }
 cudaError_t cudaMallocAsync(void** p, size_t bytes, cudaStream_t)
 {

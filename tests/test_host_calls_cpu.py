@@ -85,6 +85,20 @@ def test_free_waits_for_the_device_that_owns_the_object(fake):
     assert d.value == 1 and f.lib.fake_live() == 0
 
 
+@pytest.mark.parametrize("fn,after", [("cudaMemPoolCreate", 0), ("cudaMallocFromPoolAsync", 0),
+                                      ("cudaMallocFromPoolAsync", -1), ("cudaMallocHost", 1)])
+def test_a_prepare_that_fails_leaves_no_validation_running(fake, fn, after):
+    """The caller may free the matrix once spmv_prepare has returned."""
+    f = fake()
+    A = f.matrix(1000)
+    f.fail(fn, CUDA_ERROR_MEMORY, after)
+    st, h = f.prepare(A, trusted=0)
+    assert (st == OK) == (fn == "cudaMallocFromPoolAsync" and after == 0) and bool(h) == (st == OK)   # tried once more
+    log = f.log()
+    runs = [i for i, ln in enumerate(log) if ln.startswith("kernel ")]
+    assert not runs or "stream 0 synchronize" in log[runs[-1]:], log
+
+
 # ---- conjugate gradients ----------------------------------------------------------
 
 COOPERATIVE_TOO_LARGE = 720
