@@ -68,6 +68,24 @@ struct DevicePool {
 std::mutex g_pool_mu;
 DevicePool g_pool[kMaxDevices];
 
+// Memory of cudaMalloc is open to every peer that enabled access; a pool's is
+// open to the devices it names.
+void pool_open_to_peers(cudaMemPool_t pool, int d)
+{
+    int n = 1;
+    if (cudaGetDeviceCount(&n) != cudaSuccess) n = 1;
+    for (int peer = 0; peer < n; ++peer) {
+        int can = 0;
+        if (peer == d || cudaDeviceCanAccessPeer(&can, peer, d) != cudaSuccess || !can) continue;
+        cudaMemAccessDesc a = {};
+        a.location.type = cudaMemLocationTypeDevice;
+        a.location.id = peer;
+        a.flags = cudaMemAccessFlagsProtReadWrite;
+        cudaMemPoolSetAccess(pool, &a, 1);  // a device that cannot after all stays without
+    }
+    cudaGetLastError();
+}
+
 // g_pool_mu held; d is the current device (its stream is made here)
 cudaError_t pool_open(int d)
 {
@@ -89,6 +107,7 @@ cudaError_t pool_open(int d)
         if (pool) cudaMemPoolDestroy(pool);
         return e;
     }
+    pool_open_to_peers(pool, d);
     g.pool = pool;
     g.stream = stream;
     return cudaSuccess;

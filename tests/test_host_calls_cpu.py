@@ -99,6 +99,27 @@ def test_a_prepare_that_fails_leaves_no_validation_running(fake, fn, after):
     assert not runs or "stream 0 synchronize" in log[runs[-1]:], log
 
 
+def test_peers_reach_prepared_arrays(fake):
+    """As they reach memory of cudaMalloc: every device that can, and no other."""
+    f = fake(devices=4)
+    for a, b in ((1, 0), (3, 0), (0, 2)):               # 1 and 3 reach 0; 0 reaches 2
+        f.lib.fake_peer(a, b)
+    st, h = f.prepare(f.matrix(1000))
+    assert st == OK
+    opened = [ln for ln in f.log() if ln.startswith("pool of device 0 open")]
+    assert opened == ["pool of device 0 open to device 1", "pool of device 0 open to device 3"]
+    f.lib.spmv_prepared_free(h)
+
+
+def test_a_pool_that_cannot_be_opened_to_a_peer(fake):
+    f = fake(devices=2)
+    f.lib.fake_peer(1, 0)
+    f.fail("cudaMemPoolSetAccess", 1, after=-1)
+    st, h = f.prepare(f.matrix(1000))
+    assert st == OK
+    f.lib.spmv_prepared_free(h)
+
+
 # ---- conjugate gradients ----------------------------------------------------------
 
 COOPERATIVE_TOO_LARGE = 720
