@@ -1,5 +1,6 @@
 // C ABI entry points: status and errors, validation, features, selection,
 // prepare / run / free.  See include/spmv.h for the contract of each call.
+#include <cuda.h>
 #include <math.h>
 #include <string.h>
 
@@ -561,29 +562,55 @@ spmv_status run_impl(const spmv_prepared_t* P, const double* x, double* y, cudaS
     return SPMV_OK;
 }
 
-// The device's address of n doubles of page-locked host memory, mapped from
-// the first to the last; null for other memory.
+// The device's address of n doubles of page-locked host memory, every one of
+// them mapped; null for other memory.  (First and last element alone do not
+// tell: there may be pages between two registrations that the device cannot
+// reach.)  Where a registration ends is the driver's to say; a vector that runs
+// on into the next one is followed.  A query takes half a microsecond.
 double* mapped(double* host, int64_t n)
 {
-    cudaPointerAttributes a, b;
-    if (cudaPointerGetAttributes(&a, host) != cudaSuccess || cudaPointerGetAttributes(&b, host + n - 1) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
+    using Query = CUresult (*)(void*, CUpointer_attribute, CUdeviceptr);
+    static const Query query = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<Query>(f);
+    }();
+    if (!query) return nullptr;
+    const size_t size = 8 * (size_t)n;
+    char* dev = nullptr;
+    for (size_t at = 0; at < size;) {
+        cudaPointerAttributes a;
+        if (cudaPointerGetAttributes(&a, reinterpret_cast<char*>(host) + at) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        char* const here = static_cast<char*>(a.devicePointer);
+        if (at == 0) dev = here;
+        if (a.type != cudaMemoryTypeHost || !here || here != dev + at) return nullptr;
+        CUdeviceptr start = 0;
+        size_t bytes = 0;
+        const CUdeviceptr p = reinterpret_cast<CUdeviceptr>(here);
+        if (query(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, p) != CUDA_SUCCESS ||
+            query(&bytes, CU_POINTER_ATTRIBUTE_RANGE_SIZE, p) != CUDA_SUCCESS || p - start >= bytes)
+            return nullptr;
+        at += bytes - (p - start);
     }
-    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer ||
-        static_cast<double*>(b.devicePointer) != static_cast<double*>(a.devicePointer) + n - 1)
-        return nullptr;
-    return static_cast<double*>(a.devicePointer);
+    return reinterpret_cast<double*>(dev);
 }
 
 // Where the kernels of P can write y into the caller's host memory
 // themselves, so that its download passes behind the product instead of after
 // it (27-point stencil 128^3, 16.8 MB of y: 217 us for the call against 315):
 // every element is written once and whole stretches of at least 128 bytes by
-// a warp at a time -- rows in order, at most two lanes a row -- and the memory
-// is page-locked and mapped from the first element to the last.  Rows sorted
-// by length would scatter 8-byte writes over the link, and the STREAM and
-// MERGE fix-ups read y back: those keep the staging vector.
+// a warp at a time -- rows in order, at most two lanes a row -- and all of the
+// memory is page-locked and mapped.  Rows sorted by length would scatter
+// 8-byte writes over the link, and the STREAM and MERGE fix-ups read y back:
+// those keep the staging vector.
 double* host_target(const spmv_prepared* P, double* y_host)
 {
     const spmv_choice_t& c = P->c;

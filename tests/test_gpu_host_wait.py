@@ -118,3 +118,26 @@ def test_limits_out_of_range(limit):
     x, y = _host(HALF_M)
     with pytest.raises(sp.SpmvError, match="limit_ns"):
         sp.spmv_host_wait_check(P, x, y, limit, arrive=True)
+
+
+@pytest.mark.parametrize("pieces", [1, 2])
+def test_registered_vectors(pieces):
+    """Memory of the caller's own that it registered, as a whole or in two parts
+    end to end, is used in place."""
+    P = _prepare(_band(HALF_M))
+    raw = torch.zeros(8 * HALF_M + 4096, dtype=torch.uint8)
+    at = -raw.data_ptr() % 4096
+    x = raw[at:at + 8 * HALF_M].view(torch.float64)
+    x.copy_(synth.uniform_vector(HALF_M, 5))
+    y = torch.empty(HALF_M, dtype=torch.float64).pin_memory()
+    want = _product(P, x)
+    rt, size = torch.cuda.cudart(), 8 * HALF_M // pieces
+    starts = [x.data_ptr() + i * size for i in range(pieces)]
+    for p in starts:
+        assert int(rt.cudaHostRegister(p, size, 0)) == 0
+    try:
+        assert not sp.spmv_host_wait_check(P, x, y, 2_000_000_000, arrive=True)
+        assert torch.equal(y, want)
+    finally:
+        for p in starts:
+            rt.cudaHostUnregister(p)

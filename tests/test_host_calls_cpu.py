@@ -120,6 +120,46 @@ def test_a_pool_that_cannot_be_opened_to_a_peer(fake):
     f.lib.spmv_prepared_free(h)
 
 
+# ---- page-locked vectors -------------------------------------------------------------
+
+N = 1 << 19                       # columns from which the kernel pulls x
+PAGE = 4096
+X_PULLED, X_COPIED, Y_COPIED = "kernel k_sliced_host on stream 0", f"copy up {8 * N}", f"copy down {8 * N}"
+
+
+def _paged(n):
+    """n doubles from a page boundary on, and what keeps them."""
+    raw = np.zeros(8 * n + PAGE, dtype=np.uint8)
+    at = -raw.ctypes.data % PAGE
+    return raw[at:at + 8 * n].view(np.float64)
+
+
+@pytest.mark.parametrize("vector", ["x", "y"])
+@pytest.mark.parametrize("locked,direct", [
+    ([(0, 8 * N)], True),                                              # all of it
+    ([(0, PAGE), (8 * N - PAGE, PAGE)], False),                        # a hole between two registrations
+    ([(0, 8 * N - PAGE), (8 * N - PAGE, PAGE)], True),                 # two, end to end
+    ([(0, PAGE), (PAGE, PAGE), (2 * PAGE, 8 * N)], True),              # three, and past the end
+    ([(0, 8 * N - PAGE)], False), ([(PAGE, 8 * N - PAGE)], False), ([], False)])
+def test_host_vectors_are_used_where_registrations_hold_all_of_them(fake, vector, locked, direct):
+    f = fake()
+    st, h = f.prepare(f.matrix(N), block_nnz=1, threads_per_row=1)
+    assert st == OK
+    x, y = _paged(N), _paged(N)
+    for v, ranges in ((x, locked if vector == "x" else [(0, 8 * N)]), (y, locked if vector == "y" else [(0, 8 * N)])):
+        for at, n in ranges:
+            f.lib.fake_lock(v.ctypes.data + at, n)
+    f.lib.fake_clear()
+    assert f.lib.spmv_host(h, x.ctypes.data, y.ctypes.data, None) == OK
+    log = f.log()
+    assert ((X_PULLED in log), (X_COPIED in log)) == ((True, False) if direct or vector == "y" else (False, True))
+    assert (Y_COPIED in log) == (vector == "y" and not direct)
+    f.lib.fake_clear()
+    assert f.lib.spmv_host_async(h, x.ctypes.data, y.ctypes.data, None) == OK
+    assert X_COPIED in f.log() and Y_COPIED in f.log() and X_PULLED not in f.log()
+    f.lib.spmv_prepared_free(h)
+
+
 # ---- conjugate gradients ----------------------------------------------------------
 
 COOPERATIVE_TOO_LARGE = 720
