@@ -178,10 +178,20 @@ void pool_release(int device)
     if (--g_pool[device].users == 0) cudaMemPoolTrimTo(g_pool[device].pool, 0);
 }
 
+void pool_give_back()
+{
+    int d = -1;
+    if (cudaGetDevice(&d) != cudaSuccess || d < 0 || d >= kMaxDevices) return;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (!g_pool[d].pool) return;
+    cudaStreamSynchronize(g_pool[d].stream);
+    cudaMemPoolTrimTo(g_pool[d].pool, 0);
+}
+
 cudaError_t work_alloc(int device, void** p, size_t bytes, cudaStream_t s)
 {
     // large scratch does not stay mapped: the device's default pool
-    if (bytes > kPoolKeep / 4) return cudaMallocAsync(p, bytes, s);
+    if (bytes > kPoolKeep / 4) return stream_alloc(p, bytes, s);
     cudaMemPool_t pool;
     cudaStream_t st;
     cudaError_t e = pool_get(device, &pool, &st);

@@ -209,7 +209,7 @@ spmv_status build_items(spmv_batch* B, cudaStream_t s)
     B->d_items = nullptr;
     B->n_items = (int64_t)items.size();
     if (items.empty()) return SPMV_OK;
-    SPMV_CUDA_TRY(cudaMalloc(reinterpret_cast<void**>(&B->d_items), sizeof(BatchItem) * items.size()));
+    SPMV_CUDA_TRY(device_alloc(reinterpret_cast<void**>(&B->d_items), sizeof(BatchItem) * items.size()));
     SPMV_CUDA_TRY(cudaMemcpyAsync(B->d_items, items.data(), sizeof(BatchItem) * items.size(),
                                   cudaMemcpyHostToDevice, s));
     SPMV_CUDA_TRY(cudaStreamSynchronize(s));
@@ -221,10 +221,10 @@ spmv_status finish_create(spmv_batch* B, int32_t count, cudaStream_t s, spmv_bat
 {
     B->xs.assign(count, nullptr);
     B->ys.assign(count, nullptr);
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&B->d_counter), 8);
+    cudaError_t e = device_alloc(reinterpret_cast<void**>(&B->d_counter), 8);
     if (e == cudaSuccess) e = cudaMemsetAsync(B->d_counter, 0, 8, s);
     if (e == cudaSuccess && count > 0)
-        e = cudaMalloc(reinterpret_cast<void**>(&B->d_mats), sizeof(BatchMat) * count);
+        e = device_alloc(reinterpret_cast<void**>(&B->d_mats), sizeof(BatchMat) * count);
     if (e != cudaSuccess) { spmv_batch_free(B); return cuda_fail(e, "spmv_batch_create"); }
     // which segments belong to rows of several
     B->seg_row.resize(count);
@@ -493,7 +493,7 @@ spmv_status spmv_batch_autotune(spmv_batch_t* B, int32_t reps, spmv_stream_t str
             if (d_tmp) cudaFreeAsync(d_tmp, s);
             d_tmp = nullptr;
             cap = items.size();
-            e = cudaMallocAsync(reinterpret_cast<void**>(&d_tmp), sizeof(BatchItem) * cap, s);
+            e = stream_alloc(reinterpret_cast<void**>(&d_tmp), sizeof(BatchItem) * cap, s);
         }
         if (e == cudaSuccess && !items.empty())
             e = cudaMemcpyAsync(d_tmp, items.data(), sizeof(BatchItem) * items.size(),

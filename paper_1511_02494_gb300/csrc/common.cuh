@@ -55,6 +55,27 @@ spmv_status pool_acquire(int device);
 void pool_release(int device);
 // scratch of one call, ordered on its stream; freed with cudaFreeAsync
 cudaError_t work_alloc(int device, void** p, size_t bytes, cudaStream_t s);
+// An allocation from elsewhere: where there is no memory for it, what the
+// current device's pool keeps idle goes back to the system and it is tried once
+// more, so that the pool costs no call its memory.
+void pool_give_back();
+template <typename F>
+cudaError_t alloc_or_give_back(F alloc)
+{
+    cudaError_t e = alloc();
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    pool_give_back();
+    return alloc();
+}
+inline cudaError_t device_alloc(void** p, size_t bytes)
+{
+    return alloc_or_give_back([&] { return cudaMalloc(p, bytes); });
+}
+inline cudaError_t stream_alloc(void** p, size_t bytes, cudaStream_t s)
+{
+    return alloc_or_give_back([&] { return cudaMallocAsync(p, bytes, s); });
+}
 
 // ---- matrix checks on the host side of the ABI ----------------------------------
 spmv_status check_csr_args(const spmv_csr_t* A);

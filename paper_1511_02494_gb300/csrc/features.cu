@@ -633,7 +633,7 @@ spmv_status feature_pass_enqueue(const spmv_csr_t* A, int32_t line_bytes, bool f
             t_scratch = nullptr;
             t_scratch_bytes = 0;
             t_scratch_clean = false;
-            e = cudaMalloc(&t_scratch, at);
+            e = device_alloc(&t_scratch, at);
             if (e == cudaSuccess) { t_scratch_bytes = at; t_scratch_device = dev.device; }
         }
         if (e == cudaSuccess && !t_scratch_clean) e = cudaMemsetAsync(t_scratch, 0, t_scratch_bytes, s);

@@ -677,8 +677,7 @@ spmv_status loss_grad_impl(const float* params, int32_t h1, int32_t h2, int32_t 
     const int64_t P = n_params(h1, h2, k);
     const int64_t stride = (P + 31) / 32 * 32;  // partials start on 128-byte lines
     float* part = nullptr;
-    SPMV_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&part),
-                                  sizeof(float) * ((size_t)parts * stride + parts), s));
+    SPMV_CUDA_TRY(stream_alloc(reinterpret_cast<void**>(&part), sizeof(float) * ((size_t)parts * stride + parts), s));
     // shared memory for the widest shape is allowed once per device
     static LaunchCache cache;
     int per_sm = 0;

@@ -174,7 +174,7 @@ extern "C" spmv_status spmv_gather_probe(const spmv_csr_t* A, const double* x, u
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const int grid = dev.sm_count * 8;
     unsigned long long* part = nullptr;
-    SPMV_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&part), sizeof(unsigned long long) * grid, s));
+    SPMV_CUDA_TRY(stream_alloc(reinterpret_cast<void**>(&part), sizeof(unsigned long long) * grid, s));
     k_gather_probe<4><<<grid, kGT, 0, s>>>(A->nnz, A->colind, x, part);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) {
@@ -209,11 +209,11 @@ struct Probes {
         const int64_t N = A->n_rows, NNZ = A->nnz;
         T = auto_threads_per_row((double)NNZ / (double)N / 4.0);
         b_bounds.s = b_zero.s = b_rp64.s = b_ci64.s = b_st.s = s;
-        SPMV_CUDA_TRY(cudaMallocAsync(&b_bounds.p, sizeof(int64_t) * (W + 1), s));
-        SPMV_CUDA_TRY(cudaMallocAsync(&b_zero.p, sizeof(int) * NNZ, s));
-        SPMV_CUDA_TRY(cudaMallocAsync(&b_rp64.p, sizeof(int64_t) * (N + 1), s));
-        SPMV_CUDA_TRY(cudaMallocAsync(&b_ci64.p, sizeof(int64_t) * NNZ, s));
-        SPMV_CUDA_TRY(cudaMallocAsync(&b_st.p, sizeof(unsigned long long) * 2 * W, s));
+        SPMV_CUDA_TRY(stream_alloc(&b_bounds.p, sizeof(int64_t) * (W + 1), s));
+        SPMV_CUDA_TRY(stream_alloc(&b_zero.p, sizeof(int) * NNZ, s));
+        SPMV_CUDA_TRY(stream_alloc(&b_rp64.p, sizeof(int64_t) * (N + 1), s));
+        SPMV_CUDA_TRY(stream_alloc(&b_ci64.p, sizeof(int64_t) * NNZ, s));
+        SPMV_CUDA_TRY(stream_alloc(&b_st.p, sizeof(unsigned long long) * 2 * W, s));
         bounds = static_cast<int64_t*>(b_bounds.p);
         zero_ci = static_cast<int*>(b_zero.p);
         rp64 = static_cast<int64_t*>(b_rp64.p);
@@ -288,7 +288,7 @@ extern "C" spmv_status spmv_profile(const spmv_csr_t* A, const double* x, int32_
     if ((st = pr.setup(A, W, s)) != SPMV_OK) return st;
     DevBuf b_y;
     b_y.s = s;
-    SPMV_CUDA_TRY(cudaMallocAsync(&b_y.p, sizeof(double) * A->n_rows, s));
+    SPMV_CUDA_TRY(stream_alloc(&b_y.p, sizeof(double) * A->n_rows, s));
     double* y = static_cast<double*>(b_y.p);
 
     cudaEvent_t e0, e1;

@@ -120,6 +120,70 @@ def test_a_pool_that_cannot_be_opened_to_a_peer(fake):
     f.lib.spmv_prepared_free(h)
 
 
+def _features(f, A):
+    return f.lib.spmv_features(C.byref(A), 128, C.byref(_abi.Features()), None)
+
+
+def _validate(f, A):
+    return f.lib.spmv_validate(C.byref(A), None)
+
+
+def _batch(f, A):
+    B = C.c_void_p()
+    st = f.lib.spmv_batch_create(C.byref(A), 1, None, None, C.byref(B), None)
+    f.lib.spmv_batch_free(B)
+    return st
+
+
+def _train(f, A):
+    m = np.ones(16 * 8 + 8 + 8 * 8 + 8 + 2 * 8 + 2, dtype=np.float32)
+    g, loss, z, y = np.empty_like(m), np.zeros(1, np.float32), np.zeros((4, 16), np.float32), np.zeros(4, np.int32)
+    return f.lib.spmv_mlp_loss_grad(m.ctypes.data, 8, 8, 2, z.ctypes.data, y.ctypes.data, 4, g.ctypes.data,
+                                    loss.ctypes.data, None)
+
+
+def _probe(f, A):
+    x, s = np.ones(A.n_cols), np.zeros(1, np.uint64)
+    return f.lib.spmv_gather_probe(C.byref(A), x.ctypes.data, s.ctypes.data, None)
+
+
+def _profile_outputs(f, A):
+    x, y = np.ones(A.n_cols), np.zeros(A.n_rows)
+    return f.lib.spmv_profile_outputs(C.byref(A), x.ctypes.data, 4, None, y.ctypes.data, None, None, None, None)
+
+
+@pytest.mark.parametrize("call,fn,after", [
+    (_features, "cudaMalloc", 0), (_validate, "cudaMalloc", 0), (_batch, "cudaMalloc", 0), (_batch, "cudaMalloc", 1),
+    (_batch, "cudaMalloc", 2), (_train, "cudaMallocAsync", 0), (_probe, "cudaMallocAsync", 0),
+    (_profile_outputs, "cudaMallocAsync", 0), (_profile_outputs, "cudaMallocAsync", 4)])
+def test_the_pools_idle_memory_is_given_back_before_a_call_fails(fake, call, fn, after):
+    f = fake()
+    A = f.matrix(1000)
+    st, kept = f.prepare(A)
+    st2, h = f.prepare(A)
+    assert st == st2 == OK
+    f.lib.spmv_prepared_free(h)                          # its arrays stay in the pool, which `kept` holds open
+    f.lib.fake_clear()
+    f.fail(fn, CUDA_ERROR_MEMORY, after)
+    assert call(f, A) == OK
+    assert "trim to 0" in f.log()
+    f.fail(fn, CUDA_ERROR_MEMORY, -1)
+    assert call(f, A) in (OK, NOMEM, CUDA)               # OK where an earlier call's scratch serves
+    f.lib.fake_reset(1)
+    f.lib.spmv_prepared_free(kept)
+
+
+def test_the_pools_idle_memory_is_given_back_for_large_work_vectors(fake):
+    f = fake()
+    n = 12_000_000                                       # three vectors: more than the pool keeps for scratch
+    st, h = f.prepare(f.matrix(n))
+    assert st == OK
+    f.lib.fake_clear()
+    f.fail("cudaMallocAsync", CUDA_ERROR_MEMORY)
+    assert _cg(f, h, n, iters=1) == OK and "trim to 0" in f.log()
+    f.lib.spmv_prepared_free(h)
+
+
 # ---- page-locked vectors -------------------------------------------------------------
 
 N = 1 << 19                       # columns from which the kernel pulls x
