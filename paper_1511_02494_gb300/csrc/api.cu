@@ -65,9 +65,19 @@ struct DevicePool {
     cudaMemPool_t pool = nullptr;
     cudaStream_t stream = nullptr;
     int users = 0;
+    uint64_t live = 0;  // bytes of the objects' arrays
 };
 std::mutex g_pool_mu;
 DevicePool g_pool[kMaxDevices];
+
+// g_pool_mu held.  What a wait may leave mapped: the objects' arrays and
+// kPoolKeep, so that scratch of many calls in flight at once does not stay;
+// nothing without objects.
+void pool_bound(DevicePool& g)
+{
+    uint64_t keep = g.users > 0 ? g.live + kPoolKeep : 0;
+    cudaMemPoolSetAttribute(g.pool, cudaMemPoolAttrReleaseThreshold, &keep);
+}
 
 // Memory of cudaMalloc is open to every peer that enabled access; a pool's is
 // open to the devices it names.
@@ -99,10 +109,6 @@ cudaError_t pool_open(int d)
     cudaMemPool_t pool = nullptr;
     cudaStream_t stream = nullptr;
     cudaError_t e = cudaMemPoolCreate(&pool, &props);
-    // nothing is given back behind our back at a synchronisation: pool_free
-    // and pool_release keep the bound
-    uint64_t never = UINT64_MAX;
-    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &never);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         if (pool) cudaMemPoolDestroy(pool);
@@ -149,15 +155,26 @@ cudaError_t pool_alloc(int device, void** p, size_t bytes)
         cudaMemPoolTrimTo(pool, 0);
         e = cudaMallocFromPoolAsync(p, bytes, pool, st);
     }
-    return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+    if (e != cudaSuccess) return e;
+    {
+        std::lock_guard<std::mutex> lk(g_pool_mu);
+        g_pool[device].live += bytes;
+        pool_bound(g_pool[device]);
+    }
+    return cudaStreamSynchronize(st);
 }
 
-void pool_free(int device, void* const* p, size_t count)
+void pool_free(int device, void* const* p, size_t count, size_t bytes)
 {
     if (count == 0) return;
     cudaMemPool_t pool;
     cudaStream_t st;
     if (pool_get(device, &pool, &st) != cudaSuccess) return;
+    {
+        std::lock_guard<std::mutex> lk(g_pool_mu);
+        g_pool[device].live -= bytes;
+        pool_bound(g_pool[device]);
+    }
     for (size_t i = 0; i < count; ++i) cudaFreeAsync(p[i], st);
     cudaStreamSynchronize(st);
     pool_trim(pool, kPoolKeep);
@@ -169,13 +186,16 @@ spmv_status pool_acquire(int device)
     std::lock_guard<std::mutex> lk(g_pool_mu);
     SPMV_CUDA_TRY(pool_open(device));
     ++g_pool[device].users;
+    pool_bound(g_pool[device]);
     return SPMV_OK;
 }
 
 void pool_release(int device)
 {
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    if (--g_pool[device].users == 0) cudaMemPoolTrimTo(g_pool[device].pool, 0);
+    if (--g_pool[device].users > 0) return;
+    pool_bound(g_pool[device]);
+    cudaMemPoolTrimTo(g_pool[device].pool, 0);
 }
 
 void pool_give_back()
@@ -302,7 +322,7 @@ spmv_status dev_alloc(spmv_prepared_t* P, T** p, int64_t count)
 // in P->owned when it was made), whatever the variant.
 void release(spmv_prepared_t* P)
 {
-    pool_free(P->device, P->owned.data(), P->owned.size());
+    pool_free(P->device, P->owned.data(), P->owned.size(), (size_t)P->owned_bytes);
     P->owned.clear();
     pool_release(P->device);
     if (P->persist_held) {

@@ -40,16 +40,16 @@ spmv_status current_device(DeviceInfo* out);
 
 // ---- device memory ------------------------------------------------------------
 // The library's memory pool of a device.  Prepared objects live in it, and
-// while any does, up to kPoolKeep bytes that freed objects left stay mapped
-// for the next one (mapping and unmapping memory took 0.6 of the 1.5 ms that
-// a 100^3 27-point stencil spent from features to first product); when the
-// device's last object is freed, all of it goes back to the system.  Safe
-// from several threads.
+// while any does, up to kPoolKeep bytes that freed objects and finished calls
+// left stay mapped for the next ones (mapping and unmapping memory took 0.6 of
+// the 1.5 ms that a 100^3 27-point stencil spent from features to first
+// product); when the device's last object is freed, all of it goes back to the
+// system.  Safe from several threads.
 constexpr size_t kPoolKeep = (size_t)1 << 30;
 // usable on every stream once the call returns, like cudaMalloc
 cudaError_t pool_alloc(int device, void** p, size_t bytes);
-// with no work on p in flight
-void pool_free(int device, void* const* p, size_t count);
+// with no work on p in flight; `bytes` of all of them together
+void pool_free(int device, void* const* p, size_t count, size_t bytes);
 // counts prepared objects (the last one to go empties the pool)
 spmv_status pool_acquire(int device);
 void pool_release(int device);

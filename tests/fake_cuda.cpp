@@ -15,6 +15,7 @@
 #include <mutex>
 #include <string>
 #include <utility>
+#include <vector>
 
 #undef cudaGetDriverEntryPointByVersion
 
@@ -36,7 +37,9 @@ std::map<std::string, int> peers;            // "a b": a can reach b
 int n_devices = 1;
 thread_local int device = 0;
 thread_local cudaError_t last = cudaSuccess;
-size_t used = 0, reserved = 0;
+size_t used = 0, reserved = 0, threshold = 0;
+bool later = false;                          // frees on a stream take effect when something waits
+std::vector<void*> freed;
 int streams = 0;
 
 void log(const char* fmt, ...)
@@ -87,6 +90,16 @@ void give(void* p)
     free(p);
 }
 
+// a wait: what was freed on a stream is free, and the pool keeps its threshold
+void waited()
+{
+    std::lock_guard<std::recursive_mutex> lk(mu);
+    for (void* p : freed) give(p);
+    freed.clear();
+    const size_t keep = threshold > used ? threshold : used;
+    if (reserved > keep) reserved = keep;
+}
+
 std::map<char*, Range>::iterator range_of(const void* p)
 {
     auto it = locked.upper_bound((char*)p);
@@ -132,6 +145,7 @@ void fake_clear() { lines.clear(); }
 void fake_fail(const char* fn, int after, int code) { faults[fn] = {after, code}; }
 void fake_lock(void* p, size_t bytes) { locked[(char*)p] = {bytes}; }
 void fake_peer(int a, int b) { peers[std::to_string(a) + " " + std::to_string(b)] = 1; }
+void fake_free_later(int on) { later = on; }
 long long fake_live() { return (long long)live.size(); }
 long long fake_reserved() { return (long long)reserved; }
 
@@ -157,7 +171,12 @@ cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int)
 cudaError_t cudaDeviceGetLimit(size_t* v, cudaLimit) { *v = 0; return cudaSuccess; }
 cudaError_t cudaDeviceSetLimit(cudaLimit, size_t) { return cudaSuccess; }
 cudaError_t cudaCtxResetPersistingL2Cache() { return cudaSuccess; }
-cudaError_t cudaDeviceSynchronize() { log("device %d synchronize", device); return result("cudaDeviceSynchronize"); }
+cudaError_t cudaDeviceSynchronize()
+{
+    log("device %d synchronize", device);
+    waited();
+    return result("cudaDeviceSynchronize");
+}
 cudaError_t cudaGetLastError() { cudaError_t e = last; last = cudaSuccess; return e; }
 const char* cudaGetErrorName(cudaError_t) { return "error"; }
 const char* cudaGetErrorString(cudaError_t) { return "an error of the fake runtime"; }
@@ -185,7 +204,13 @@ cudaError_t cudaMallocFromPoolAsync(void** p, size_t bytes, cudaMemPool_t, cudaS
     const cudaError_t e = result("cudaMallocFromPoolAsync");
     return e == cudaSuccess ? take(p, bytes, 1) : e;
 }
-cudaError_t cudaFreeAsync(void* p, cudaStream_t s) { log("free %p on stream %zx", p, (size_t)s); give(p); return cudaSuccess; }
+cudaError_t cudaFreeAsync(void* p, cudaStream_t s) 
+{
+    log("free %p on stream %zx", p, (size_t)s);
+    if (later) freed.push_back(p);
+    else give(p);
+    return cudaSuccess;
+}
 cudaError_t cudaMemPoolCreate(cudaMemPool_t* p, const cudaMemPoolProps* props)
 {
     *p = (cudaMemPool_t)(size_t)(0x100 + props->location.id);
@@ -199,7 +224,11 @@ cudaError_t cudaMemPoolSetAccess(cudaMemPool_t p, const cudaMemAccessDesc* d, si
         log("pool of device %d open to device %d", (int)(size_t)p - 0x100, d[i].flags == cudaMemAccessFlagsProtReadWrite ? d[i].location.id : -1);
     return result("cudaMemPoolSetAccess");
 }
-cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void*) { return cudaSuccess; }
+cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr a, void* v)
+{
+    if (a == cudaMemPoolAttrReleaseThreshold) threshold = *(uint64_t*)v;
+    return cudaSuccess;
+}
 cudaError_t cudaMemPoolGetAttribute(cudaMemPool_t, cudaMemPoolAttr a, void* v)
 {
     *(uint64_t*)v = a == cudaMemPoolAttrUsedMemCurrent ? used : reserved;
@@ -245,7 +274,12 @@ cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned)
     return result("cudaStreamCreateWithFlags");
 }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t s) { log("stream %zx synchronize", (size_t)s); return result("cudaStreamSynchronize"); }
+cudaError_t cudaStreamSynchronize(cudaStream_t s)
+{
+    log("stream %zx synchronize", (size_t)s);
+    waited();
+    return result("cudaStreamSynchronize");
+}
 cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { log("begin capture"); return result("cudaStreamBeginCapture"); }
 cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { *g = (cudaGraph_t)1; return cudaSuccess; }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t* x, cudaGraph_t, unsigned long long) { *x = (cudaGraphExec_t)1; return result("cudaGraphInstantiate"); }
