@@ -619,10 +619,13 @@ __device__ __forceinline__ bool stage_in(const HostX& h, int stage)
     return v >= h.want;
 }
 
-__device__ __noinline__ void give_up(const HostX& h, int lane)
+// (as a call, with the parameters' addresses taken, the kernel takes 168 us in
+// place of 158 for the 27-point stencil 128^3)
+__device__ __forceinline__ void give_up(unsigned* count, unsigned* late, int lane)
 {
-    for (int i = lane; i < kXStages; i += 32) atomicOr(h.count + kXStride * i, kXLate);
-    if (lane == 0) *h.late = 1u;
+#pragma unroll 1
+    for (int i = lane; i < kXStages; i += 32) atomicOr(count + kXStride * i, kXLate);
+    if (lane == 0) *late = 1u;
 }
 
 template <int U, typename CT>
@@ -665,7 +668,7 @@ k_sliced_host(HostX h, unsigned copy_blocks, int64_t n_slices, const int* __rest
                 const uint64_t now = __shfl_sync(FULL, ptx::global_ns(), 0);
                 if (t0 == 0) t0 = now;
                 if (now - t0 > h.limit_ns) {
-                    give_up(h, lane);
+                    give_up(h.count, h.late, lane);
                     break;
                 }
                 __nanosleep(kXSleepNs);
