@@ -418,31 +418,43 @@ k_feature_pass(int64_t n_rows, int64_t n_cols, int64_t nnz, const int* __restric
             else row_ok = true;
         }
         // long rows: a list entry each and one per piece (pieces start on the
-        // scan's boundaries); overlapping rows (a rowptr that is not
-        // monotone) can list more than the buffers hold, and the error flag
-        // is set for them
-        for (unsigned todo = __ballot_sync(FULL_MASK, is_long); todo; todo &= todo - 1) {
-            const int src = __ffs(todo) - 1;
-            const int lb = __shfl_sync(FULL_MASK, b, src), le = __shfl_sync(FULL_MASK, e, src);
-            const int64_t l0 = batch_start(t, lb);
-            const unsigned np = (unsigned)((le - l0 + kPiece - 1) / kPiece);
+        // scan's boundaries), with one pair of atomics for the tile's rows
+        // (with a pair for each, one after another, 200 rows of 1100 take 48
+        // us in place of 33, 20,000 rows of 1030 94 in place of 68);
+        // overlapping rows (a rowptr that is not monotone) can list more than
+        // the buffers hold, and the error flag is set for them
+        if (const unsigned longs = __ballot_sync(FULL_MASK, is_long)) {
             unsigned q = 0, p0 = 0;
-            if (lane == src) {
-                q = atomicAdd(&w.ctl->n_long, 1u);
-                if (q < w.max_long) {
-                    p0 = atomicAdd(&w.ctl->n_pieces, np);
-                    w.row[q] = make_int2(0, 0);
-                    w.done[q] = 0;
-                }
+            if (lane == 0) q = atomicAdd(&w.ctl->n_long, (unsigned)__popc(longs));
+            q = __shfl_sync(FULL_MASK, q, 0) + __popc(longs & ((1u << lane) - 1u));
+            const int l0 = (int)batch_start(t, b);
+            unsigned np = 0;
+            if (is_long && q < w.max_long) {
+                np = (unsigned)((e - (int64_t)l0 + kPiece - 1) / kPiece);
+                w.row[q] = make_int2(0, 0);
+                w.done[q] = 0;
+            } else if (is_long) {
+                err |= 4;
             }
-            q = __shfl_sync(FULL_MASK, q, src);
-            p0 = __shfl_sync(FULL_MASK, p0, src);
-            if (q >= w.max_long) { err |= 4; continue; }
+            unsigned upto = np;  // pieces of the tile's rows up to this one
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned v = __shfl_up_sync(FULL_MASK, upto, o);
+                if (lane >= o) upto += v;
+            }
+            if (lane == 31) p0 = atomicAdd(&w.ctl->n_pieces, upto);
+            p0 = __shfl_sync(FULL_MASK, p0, 31) + upto - np;
             // every entry below n_pieces that the buffer holds is written
             const unsigned room = p0 < w.max_pieces ? w.max_pieces - p0 : 0u;
             if (np > room) err |= 4;
-            for (unsigned p = lane; p < min(np, room); p += 32)
-                w.piece[p0 + p] = make_int4((int)q, (int)(l0 + p * kPiece), lb, le);
+            const unsigned mine = min(np, room);
+            for (unsigned todo = longs; todo; todo &= todo - 1) {
+                const int src = __ffs(todo) - 1;
+                const int rq = __shfl_sync(FULL_MASK, (int)q, src), rl = __shfl_sync(FULL_MASK, l0, src),
+                          rb = __shfl_sync(FULL_MASK, b, src), re = __shfl_sync(FULL_MASK, e, src);
+                const unsigned rp0 = __shfl_sync(FULL_MASK, p0, src), n = __shfl_sync(FULL_MASK, mine, src);
+                for (unsigned p = lane; p < n; p += 32)
+                    w.piece[rp0 + p] = make_int4(rq, rl + (int)(p * kPiece), rb, re);
+            }
         }
         if (!row_ok) b = e = 0;
         unsigned ng = 0, ms = 0;
