@@ -131,11 +131,14 @@ __global__ void k_mlp_forward(const float* __restrict__ params, const float* __r
 // Hence slices of 8 samples, so that 1600 samples put a CTA on every SM (200
 // CTAs; 32 samples a CTA left two thirds of the SMs idle), a thread per
 // output and sample pair (each weight read feeds two FMAs; rows padded by
-// four floats, so the 16-byte reads are free of bank conflicts), and at most
-// two resident CTAs per SM looping over the slices, which bounds the
-// partials to 304 whatever n is.  1600 samples of the 16-64-64-8 network:
-// 12.2 us, against 99.8 us with 50 CTAs that re-read the weights from global
-// memory for every product.
+// four floats, so the 16-byte reads are free of bank conflicts), and two to
+// four resident CTAs per SM, as many as fit, looping over the slices, which
+// bounds the partials to 608 whatever n is.  1600 samples of the 16-64-64-8
+// network: 12.2 us, against 99.8 us with 50 CTAs that re-read the weights from
+// global memory for every product.  With two CTAs per SM whatever the network,
+// the barriers of small ones leave the SM idle: 200,000 samples of 16-7-5-3 take
+// 520 us a call in place of 292, of 16-64-64-8 758 in place of 643 (eight: 295,
+// 635, and more time in the reduction at 10,000 samples).
 constexpr int kSlice = 8;
 constexpr int kMT = 256;
 static_assert(kMT / 32 == kSlice, "a warp per sample in the softmax");
@@ -169,6 +172,14 @@ __host__ __device__ __forceinline__ TrainLayout train_layout(int h1, int h2, int
     L.d3 = L.d2 + kSlice * L.as2;
     L.total = L.d3 + kSlice * L.ds3 + kSlice;  // + the slice's losses
     return L;
+}
+
+// CTAs per SM: those that fit its 228 KB of shared memory (1 KB each is the
+// system's), at least two (the widest network's) and at most four
+inline int train_ctas(size_t smem)
+{
+    const int fit = (int)((228 << 10) / (smem + (1 << 10)));
+    return std::max(2, std::min(4, fit));
 }
 
 __device__ __forceinline__ void cp_async4(float* dst, const float* src)
@@ -673,7 +684,8 @@ spmv_status loss_grad_impl(const float* params, int32_t h1, int32_t h2, int32_t 
     DeviceInfo dev;
     spmv_status st = current_device(&dev);
     if (st != SPMV_OK) return st;
-    const int parts = std::min((n + kSlice - 1) / kSlice, 2 * dev.sm_count);
+    const size_t smem = sizeof(float) * train_layout(h1, h2, k).total;
+    const int parts = std::min((n + kSlice - 1) / kSlice, train_ctas(smem) * dev.sm_count);
     const int64_t P = n_params(h1, h2, k);
     const int64_t stride = (P + 31) / 32 * 32;  // partials start on 128-byte lines
     float* part = nullptr;
@@ -684,7 +696,6 @@ spmv_status loss_grad_impl(const float* params, int32_t h1, int32_t h2, int32_t 
     const TrainLayout widest = train_layout(kTrainMaxH, kTrainMaxH, kMaxK);
     cudaError_t e = cached_occupancy(cache, k_mlp_loss_grad, kMT, sizeof(float) * widest.total, &per_sm);
     if (e == cudaSuccess) {
-        const size_t smem = sizeof(float) * train_layout(h1, h2, k).total;
         k_mlp_loss_grad<<<parts, kMT, smem, s>>>(params, h1, h2, k, z, labels, q, n, stride, part,
                                                  part + (size_t)parts * stride);
         e = cudaGetLastError();
