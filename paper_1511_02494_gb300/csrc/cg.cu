@@ -42,7 +42,7 @@ __device__ __forceinline__ int64_t grid_step() { return (int64_t)gridDim.x * kCT
 // rs[t & 1] is r.r after iteration t, so that the kernel that stores one does
 // not overwrite the one its other blocks still read.
 struct CgState {
-    double rs[2], alpha;
+    double rs[2];
 };
 
 // A dot product is left as one sum per block, and the blocks of the kernel
@@ -105,17 +105,13 @@ __device__ __forceinline__ double take_sum(const double* __restrict__ part, int 
     return warp_total((a[0] + a[1]) + (a[2] + a[3]));
 }
 
-// alpha = rs / p.q, to every thread of the block; block 0 keeps it for the
-// kernels after this one
-__device__ __forceinline__ double take_alpha(const double* __restrict__ part, int n, CgState* st, int t)
+// alpha = rs / p.q, to every thread of the block
+__device__ __forceinline__ double take_alpha(const double* __restrict__ part, int n, const CgState* st, int t)
 {
     __shared__ double s_alpha;
     if (threadIdx.x < 32) {
         const double pq = take_sum(part, n);
-        if (threadIdx.x == 0) {
-            s_alpha = st->rs[(t - 1) & 1] / pq;
-            if (blockIdx.x == 0) st->alpha = s_alpha;
-        }
+        if (threadIdx.x == 0) s_alpha = st->rs[(t - 1) & 1] / pq;
     }
     __syncthreads();
     return s_alpha;
@@ -210,7 +206,8 @@ k_axpy_x(int64_t n, double* __restrict__ x, const double* __restrict__ p, const 
 // FP32 (the same rounding its own conversion of x would apply).
 // 128^3 rows with BF16 values: 58.2 us an iteration, against 65.9 with a last
 // block after each dot product and the conversions on the FP64 pipe (FP64
-// values: 76.8 and 75.6).  Launched as programmatic dependents of one another
+// values: 76.8 and 75.6; 72 with four elements in flight in the product, see
+// kDotU).  Launched as programmatic dependents of one another
 // the three kernels are slower (61.4): blocks that start early take room from
 // the ones still running.
 enum Step { kFirst, kNext, kRestart };

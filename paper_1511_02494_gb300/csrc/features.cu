@@ -77,10 +77,11 @@ __device__ __forceinline__ u64 warp_sum_u64(u64 v) {
 // division and without 64-bit conversions (which run on the FP64 pipe): an
 // FP32 estimate of the quotient (a / b < 1, so it fits 32 bits), then the
 // integer remainder a 2^32 - q b, converted to FP32 from two 32-bit halves,
-// gives a correction, and the remainder is brought into [0, b).  The
-// reciprocal and the three products are each off by at most 2 ulp, so the
-// first estimate is within 2^10 of the quotient, |remainder| < 2^42 and the
-// second within one, which the last line settles.
+// gives a correction, and the remainder is brought into [0, b).  The two
+// conversions and the product are off by half an ulp each, the reciprocal by
+// at most two ulps: 7 x 2^-24 of a quotient below 2^32 in all, so the first
+// estimate is within 1793 < 2^11 of it, |remainder| < 2^42 and the second
+// within one, which the last line settles.
 // Arguments outside that range come only from rows the pass flags as invalid
 // (columns not strictly increasing or out of range), whose results are
 // discarded: they give 0.

@@ -1065,8 +1065,9 @@ struct Arena {
 };
 
 // check: the matrix's validation pass is on the stream; its verdict is read
-// at the first wait (what runs before that reads row pointers only, each as
-// a number)
+// at the first wait (what runs before that reads row pointers, each as a
+// number, and in k_sl_layout columns of elements that it has found to lie in
+// [0, nnz), also as numbers)
 spmv_status sliced_build(spmv_prepared* P, SlScratch* w, bool check, cudaStream_t s)
 {
     const spmv_csr_t& A = P->A;
