@@ -411,10 +411,13 @@ k_mlp_loss_grad(const float* __restrict__ params, int h1, int h2, int k, const f
 }
 
 // Sum of the CTAs' partials: a block takes 32 entries, warp w their partials
-// w, w + 8, ... in order, and the eight sums are added in warp order.  Block
-// 0 also sums the losses.  5768 entries of 200 partials: 3.7 us on 181
-// blocks (a thread per entry, 23 blocks, took 5.2 us for 50 partials).
+// w, w + 8, ... in order, a new chain after every 304 partials (38 of the
+// warp's; chains of 76 over 608 partials have 10 % more rounding error), and
+// the eight sums are added in warp order.  Block 0 also sums the losses.  5768
+// entries of 200 partials: 3.7 us on 181 blocks (a thread per entry, 23 blocks,
+// took 5.2 us for 50 partials).
 constexpr int kRT = 256;
+constexpr int kChain = 304;
 __global__ void __launch_bounds__(kRT)
 k_mlp_reduce(const float* __restrict__ part, const float* __restrict__ part_loss, int n_parts, int64_t part_stride,
              int64_t P, int n, float* __restrict__ grad, float* __restrict__ loss)
@@ -424,8 +427,12 @@ k_mlp_reduce(const float* __restrict__ part, const float* __restrict__ part_loss
     const int64_t e = (int64_t)blockIdx.x * 32 + lane;
     float acc = 0.f;
     if (e < P) {
+        for (int c0 = 0; c0 < n_parts; c0 += kChain) {
+            float a = 0.f;
 #pragma unroll 8
-        for (int c = warp; c < n_parts; c += kRT / 32) acc += __ldcg(part + (int64_t)c * part_stride + e);
+            for (int c = c0 + warp; c < min(n_parts, c0 + kChain); c += kRT / 32) a += __ldcg(part + (int64_t)c * part_stride + e);
+            acc = c0 == 0 ? a : acc + a;
+        }
     }
     sums[warp][lane] = acc;
     __syncthreads();
