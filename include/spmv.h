@@ -668,7 +668,7 @@ void spmv_batch_free(spmv_batch_t *B);
  * Runs `iters` iterations without a convergence test (no host sync inside the
  * loop).  With a SLICED A_inner without long rows or coded columns (and, when
  * refining, an A_exact of that kind with FP64 values) of up to about 1.05 M
- * rows, whose stored arrays take at most nine tenths of the L2 (seven tenths
+ * rows, whose stored arrays take at most 1.7 times the L2 (seven tenths of it
  * with FP32 or BF16 values), the whole loop is one cooperative kernel launch,
  * whatever use_graph says; its blocks wait for one another with a bound of two
  * seconds, after which x and the remaining entries of resid are NaN.  Above

@@ -805,24 +805,27 @@ int64_t product_bytes(const spmv_prepared* P)
 // whose operands stay in the L2 from one iteration to the next waits for
 // latency, which the one launch has less of; a larger one streams from memory,
 // for which 24 warps per SM keep less in flight than the product kernel's 64
-// (or 48).  The line lies at nine tenths of the L2 for FP64 values and at seven
-// tenths for FP32 and BF16 ones, whose product takes less time for the same
-// bytes.  An iteration here / in three kernels, us, by product_bytes (an L2 of
-// 135.5 MB):
-//   FP64  7-point 101^3   99 MB 36 / 46  band 524288 x 17 113 MB  44 / 47
-//         27-point 72^3  126 MB 47 / 45  band 262144 x 41 132 MB  50 / 46
-//         27-point 90^3  245 MB 74 / 66  band 1.04 M x 41 525 MB 130 / 115
-//   BF16  27-point 80^3   64 MB 31 / 39  27-point 90^3     91 MB  44 / 48
-//         band 1.04 M x 17 96 MB 51 / 48 band 524288 x 41  99 MB  51 / 47
-//         27-point 100^3 124 MB 75 / 60  band 1.04 M x 41 196 MB  98 / 74
-//   FP32  27-point 80^3   92 MB 39 / 45  band 524288 x 25  95 MB  33 / 43
-//         band 786432 x 17 104 MB 46 / 46 band 393216 x 41 109 MB 50 / 45
+// (or 48).  FP32 and BF16 products take little more than their bytes' time:
+// the line lies at seven tenths of the L2.  With FP64 values the DFMAs take
+// their time either way, and both loops are equal within 6 % up to 1.7 times
+// the L2, where the line lies.  An iteration here / in three kernels, us, by
+// product_bytes (an L2 of 135.5 MB):
+//   FP64  7-point 101^3     99 MB 36 / 46  27-point 72^3    126 MB  47 / 45
+//         27-point 80^3    172 MB 57 / 56  band 524288 x 25 164 MB  55 / 57
+//         band 1.04 M x 17 225 MB 73 / 68  27-point 90^3    245 MB  74 / 66
+//         band 524288 x 41 264 MB 76 / 76  band 1.04 M x 41 525 MB 130 / 115
+//     16-bit columns: 524288 x 41 221 MB 72 / 77, 27-point 100^3 277 MB 92 / 84
+//   BF16  27-point 80^3     64 MB 31 / 39  27-point 90^3     91 MB  44 / 48
+//         band 1.04 M x 17  96 MB 51 / 48  band 524288 x 41  99 MB  51 / 47
+//         27-point 100^3   124 MB 75 / 60  band 1.04 M x 41 196 MB  98 / 74
+//   FP32  27-point 80^3     92 MB 39 / 45  band 524288 x 25  95 MB  33 / 43
+//         band 786432 x 17 104 MB 46 / 46  band 393216 x 41 109 MB  50 / 45
 bool resident_choice(const spmv_prepared* Pi, const spmv_prepared* Pe, int refine, const DeviceInfo& dev, Resident* out)
 {
     if (!fusable(Pi) || (refine > 0 && !fp64_sliced(Pe))) return false;
     const SlicedPlan& d = Pi->sl;
     const int sm_count = dev.sm_count;
-    if (10 * product_bytes(Pi) > (d.value_type == SPMV_VAL_F64 ? 9 : 7) * (int64_t)dev.l2_bytes) return false;
+    if (10 * product_bytes(Pi) > (d.value_type == SPMV_VAL_F64 ? 17 : 7) * (int64_t)dev.l2_bytes) return false;
     if (d.value_type == SPMV_VAL_F64) {
         if (d.cbytes == 1) return resident_fits<double, false, false, int8_t>(d.n_slices, sm_count, out);
         if (d.cbytes == 2) return resident_fits<double, false, false, int16_t>(d.n_slices, sm_count, out);

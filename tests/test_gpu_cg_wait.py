@@ -118,9 +118,9 @@ def _band(n, width):
 
 
 @pytest.mark.parametrize("kw,bytes_a_slot,head,vector,tenths", [
-    ({}, 12, 140, 8, 9), (dict(index_bytes=2), 10, 140, 8, 9), (dict(value_type=sp.VAL_F32), 6, 268, 4, 7),
+    ({}, 12, 140, 8, 17), (dict(index_bytes=2), 10, 140, 8, 17), (dict(value_type=sp.VAL_F32), 6, 268, 4, 7),
     (dict(value_type=sp.VAL_BF16), 4, 268, 4, 7), (dict(value_type=sp.VAL_BF16, accumulate=sp.ACC_F64), 4, 268, 8, 7)])
-def test_one_launch_while_the_product_fits_the_l2(kw, bytes_a_slot, head, vector, tenths):
+def test_one_launch_by_the_products_bytes_and_the_l2(kw, bytes_a_slot, head, vector, tenths):
     """Rows of 40 (whole groups of four): the row counts, in slices, just
     inside and just past the limit; both solve the system."""
     l2 = torch.cuda.get_device_properties(0).L2_cache_size
