@@ -186,8 +186,8 @@ def test_the_pools_idle_memory_is_given_back_for_large_work_vectors(fake):
 
 def test_scratch_of_many_calls_at_once_does_not_stay(fake):
     """40 solves in flight, 48 MB of work vectors each: once they have been
-    waited for, the pool keeps 1 GB beyond the objects; with the last object
-    nothing, also not what was in flight then."""
+    waited for, the pool keeps 1 GB and a step of 256 MB beyond the objects;
+    with the last object nothing, also not what was in flight then."""
     f = fake()
     n = 2_000_000
     st, h = f.prepare(f.matrix(n))
@@ -198,7 +198,7 @@ def test_scratch_of_many_calls_at_once_does_not_stay(fake):
         assert _cg(f, h, n, iters=1) == OK
     assert f.lib.fake_reserved() > objects + 40 * 24 * n - 1
     f.lib.cudaDeviceSynchronize()
-    assert objects < f.lib.fake_reserved() <= objects + (1 << 30) + (1 << 20)
+    assert objects < f.lib.fake_reserved() <= objects + (1 << 30) + (1 << 28) + (1 << 20)
     assert _cg(f, h, n, iters=1) == OK
     f.lib.spmv_prepared_free(h)
     f.lib.cudaDeviceSynchronize()
