@@ -438,12 +438,15 @@ k_feature_pass(int64_t n_rows, int64_t n_cols, int64_t nnz, const int* __restric
                 err |= 4;
             }
             unsigned upto = np;  // pieces of the tile's rows up to this one
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned v = __shfl_up_sync(FULL_MASK, upto, o);
-                if (lane >= o) upto += v;
+            if (longs & (longs - 1)) {
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned v = __shfl_up_sync(FULL_MASK, upto, o);
+                    if (lane >= o) upto += v;
+                }
             }
-            if (lane == 31) p0 = atomicAdd(&w.ctl->n_pieces, upto);
-            p0 = __shfl_sync(FULL_MASK, p0, 31) + upto - np;
+            const int last_long = 31 - __clz((int)longs);
+            if (lane == last_long) p0 = atomicAdd(&w.ctl->n_pieces, upto);
+            p0 = __shfl_sync(FULL_MASK, p0, last_long) + upto - np;
             // every entry below n_pieces that the buffer holds is written
             const unsigned room = p0 < w.max_pieces ? w.max_pieces - p0 : 0u;
             if (np > room) err |= 4;
