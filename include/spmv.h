@@ -682,15 +682,14 @@ spmv_status spmv_cg(const spmv_prepared_t *A_inner, const spmv_prepared_t *A_exa
                     const double *b, double *x, int32_t iters, int32_t refine_every,
                     double *resid, int32_t use_graph, spmv_stream_t stream);
 
-/* Self-test of the one-launch loop's waits: spmv_cg with a limit of limit_ns
- * (1..2e9) nanoseconds, whose blocks also wait for one that does not exist when
- * arrive == 0, so that the first wait runs out: x and resid[1..iters] are then
- * NaN.  SPMV_ERR_UNSUPPORTED, with nothing done, for a solve that does not run
- * as one launch.  Asynchronous on `stream`. */
+/* Self-test of the one-launch loop's waits: spmv_cg, whose blocks are one
+ * arrival short when arrive == 0, so that the first wait runs out after its two
+ * seconds: x and resid[1..iters] are then NaN.  SPMV_ERR_UNSUPPORTED, with
+ * nothing done, for a solve that does not run as one launch.  Asynchronous on
+ * `stream`. */
 spmv_status spmv_cg_wait_check(const spmv_prepared_t *A_inner, const spmv_prepared_t *A_exact,
                                const double *b, double *x, int32_t iters, int32_t refine_every,
-                               double *resid, int64_t limit_ns, int32_t arrive,
-                               spmv_stream_t stream);
+                               double *resid, int32_t arrive, spmv_stream_t stream);
 
 /* ---- no-allocation entry point ---------------------------------------------- */
 /* The paper has no counterpart of this call; it exists for callers that must

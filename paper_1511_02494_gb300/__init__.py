@@ -294,13 +294,13 @@ def spmv_cg(A_inner: Prepared, b, x, iters: int, refine_every: int = 0,
                          _stream(stream)))
 
 
-def spmv_cg_wait_check(A_inner: Prepared, b, x, iters: int, limit_ns: int, arrive: bool, refine_every: int = 0,
+def spmv_cg_wait_check(A_inner: Prepared, b, x, iters: int, arrive: bool, refine_every: int = 0,
                        A_exact: Prepared | None = None, resid=None, stream=None) -> None:
     """Self-test of the one-launch CG loop's waits: as spmv_cg; without
     arrive the first wait runs out and x and resid[1:] become NaN.  Raises
     SpmvError (UNSUPPORTED) for a solve that does not run as one launch."""
     _check(lib().spmv_cg_wait_check(A_inner.handle, A_exact.handle if A_exact else None, _ptr(b), _ptr(x),
-                                    int(iters), int(refine_every), _ptr(resid), int(limit_ns), 1 if arrive else 0,
+                                    int(iters), int(refine_every), _ptr(resid), 1 if arrive else 0,
                                     _stream(stream)))
 
 

@@ -114,7 +114,7 @@ def declare(lib):
         "spmv_prepared_status": (I32, [P, P]),
         "spmv_stream_noalloc": (I32, [C.POINTER(CSR), P, P, P]),
         "spmv_cg": (I32, [P, P, P, P, I32, I32, P, I32, P]),
-        "spmv_cg_wait_check": (I32, [P, P, P, P, I32, I32, P, I64, I32, P]),
+        "spmv_cg_wait_check": (I32, [P, P, P, P, I32, I32, P, I32, P]),
         "spmv_batch_create": (I32, [C.POINTER(CSR), I32, P, P, C.POINTER(P), P]),
         "spmv_batch_create_prepared": (I32, [P, I32, P, P]),
         "spmv_batch_create_sliced": (I32, [P, I32, P, P]),

@@ -389,24 +389,22 @@ cudaError_t launch_sliced_dot(const spmv_prepared* P, const double* p, double* q
 // iterations on 8 streams take 12.5 ms at 33^3 rows (three kernels 20.4), 37.2 at
 // 48^3 (22.5), 55 at 64^3 (38.5), 91 at 90^3 (98.7).
 //
-// `missing` blocks more than there are are waited for (none but in the wait's
-// self-test), for at most limit_ns each time.
-struct MeetWait {
-    unsigned missing = 0;
-    uint64_t limit_ns = 2000000000ull;
-};
+// The bound is a constant: as an argument of the launch (or a word that the
+// waiting thread reads) it made some forms 1.4 % slower by other instruction
+// orders.  A wait runs out all the same when the counter starts one short, as
+// spmv_cg_wait_check has it.
+constexpr uint64_t kMeetLimitNs = 2000000000ull;
 
 struct Meeting {
     double* sums;       // [2][gridDim.x]
     unsigned* arrived;  // 0 at the start
-    MeetWait wait;
     unsigned turn;
 };
 
 // Arrives and waits (one thread); false when the wait gave up.
 __device__ __forceinline__ bool arrive_and_wait(Meeting& m)
 {
-    const unsigned target = m.turn * (gridDim.x + m.wait.missing);
+    const unsigned target = m.turn * gridDim.x;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(m.arrived) : "memory");
     uint64_t t0 = 0;
     for (unsigned tries = 1;; ++tries) {
@@ -416,7 +414,7 @@ __device__ __forceinline__ bool arrive_and_wait(Meeting& m)
         if ((tries & 63) == 0) {
             const uint64_t now = ptx::global_ns();
             if (t0 == 0) t0 = now;
-            else if (now - t0 > m.wait.limit_ns) return false;
+            else if (now - t0 > kMeetLimitNs) return false;
         }
     }
 }
@@ -575,7 +573,6 @@ struct ResidentArgs {
     unsigned* arrived;
     int iters, refine;
     int per_warp;       // slices per warp
-    MeetWait wait;
 };
 
 constexpr int kResidentWarps = 24;  // most per block; one block per SM (80 registers)
@@ -597,7 +594,7 @@ k_cg_resident(const ResidentArgs a)
     double* sx = sq + span;
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * BT + threadIdx.x) >> 5, n_warps = (int64_t)gridDim.x * (BT / 32);
-    Meeting m{a.sums, a.arrived, a.wait, 0};
+    Meeting m{a.sums, a.arrived, 0};
     // row of the lane in the warp's slice j, -1 past the last
     auto row_of = [&](int j) -> int {
         const int64_t p = (warp + j * n_warps) * 32 + lane;
@@ -866,16 +863,17 @@ spmv_status enqueue_start(const spmv_prepared* Pi, const spmv_prepared* Pe, cons
     return SPMV_OK;
 }
 
-// The one launch after enqueue_start.  *refused: the device does not take it
+// The one launch after enqueue_start.  short_of: arrivals that the meetings are
+// short of (none but in the waits' self-test).  *refused: the device does not take it
 // (fewer SMs are free to this process than it has, or no cooperative launches):
 // nothing was launched.
 spmv_status enqueue_resident(const spmv_prepared* Pi, const spmv_prepared* Pe, const double* b, double* x, int iters,
-                             int refine, double* resid, const CgBufs& w, const Resident& res, const MeetWait& wait,
+                             int refine, double* resid, const CgBufs& w, const Resident& res, int short_of,
                              bool* refused, cudaStream_t s)
 {
-    SPMV_CUDA_TRY(cudaMemsetAsync(w.arrived, 0, sizeof(unsigned), s));
+    SPMV_CUDA_TRY(cudaMemsetAsync(w.arrived, short_of ? 0xff : 0, sizeof(unsigned), s));  // 0 or -1
     ResidentArgs a{sl_args(Pi), refine > 0 ? sl_args(Pe) : SlArgs{}, refine > 0 ? Pe->sl.cbytes : 4, Pi->A.n_rows, b, x,
-                   w.r, w.p, direction_copy(Pi), resid, w.st, w.sums, w.arrived, iters, refine, res.per_warp, wait};
+                   w.r, w.p, direction_copy(Pi), resid, w.st, w.sums, w.arrived, iters, refine, res.per_warp};
     void* args[] = {&a};
     const cudaError_t e = cudaLaunchCooperativeKernel(res.kernel, dim3(res.grid), dim3(res.threads), args, res.smem, s);
     if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources || e == cudaErrorNotSupported) {
@@ -951,14 +949,14 @@ spmv_status launch_graph(const spmv_prepared* Pi, const spmv_prepared* Pe, const
 
 spmv_status enqueue_cg(const spmv_prepared* Pi, const spmv_prepared* Pe, const double* b, double* x, int iters,
                        int refine, double* resid, bool use_graph, const CgBufs& w, unsigned grid, const Resident& res,
-                       const MeetWait& wait, bool one_launch, cudaStream_t s)
+                       int short_of, bool one_launch, cudaStream_t s)
 {
     spmv_status st;
     SPMV_CUDA_TRY(cudaMemsetAsync(w.st, 0, sizeof(CgState), s));
     if (res.kernel && iters > 0) {
         bool refused = false;
         if ((st = enqueue_start(Pi, Pe, b, x, resid, w, grid, s)) != SPMV_OK) return st;
-        st = enqueue_resident(Pi, Pe, b, x, iters, refine, resid, w, res, wait, &refused, s);
+        st = enqueue_resident(Pi, Pe, b, x, iters, refine, resid, w, res, short_of, &refused, s);
         if (st != SPMV_OK || !refused) return st;
         if (one_launch) return fail(SPMV_ERR_UNSUPPORTED, "this solve does not run as one launch");
     }
@@ -968,8 +966,8 @@ spmv_status enqueue_cg(const spmv_prepared* Pi, const spmv_prepared* Pe, const d
 
 // spmv_cg; one_launch: refuses what does not run as one launch
 spmv_status cg_run(const spmv_prepared_t* A_inner, const spmv_prepared_t* A_exact, const double* b, double* x,
-                   int32_t iters, int32_t refine_every, double* resid, int32_t use_graph, const MeetWait& wait,
-                   bool one_launch, spmv_stream_t stream)
+                   int32_t iters, int32_t refine_every, double* resid, int32_t use_graph, int short_of, bool one_launch,
+                   spmv_stream_t stream)
 {
     if (!A_inner || !b || !x || iters < 0 || refine_every < 0)
         return fail(SPMV_ERR_INVALID_ARG, "spmv_cg: bad argument");
@@ -1006,7 +1004,7 @@ spmv_status cg_run(const spmv_prepared_t* A_inner, const spmv_prepared_t* A_exac
     w.st = reinterpret_cast<CgState*>(base + 3 * vec + parts);
     w.arrived = reinterpret_cast<unsigned*>(base + 3 * vec + parts + state);
     w.sums = reinterpret_cast<double*>(base + 3 * vec + parts + state + room(sizeof(unsigned)));
-    st = enqueue_cg(Pi, Pe, b, x, iters, refine_every, resid, use_graph != 0, w, grid, res, wait, one_launch, s);
+    st = enqueue_cg(Pi, Pe, b, x, iters, refine_every, resid, use_graph != 0, w, grid, res, short_of, one_launch, s);
     cudaFreeAsync(base, s);  // after an error too
     if (st != SPMV_OK) return st;
     SPMV_CUDA_TRY(cudaGetLastError());
@@ -1020,16 +1018,13 @@ extern "C" spmv_status spmv_cg(const spmv_prepared_t* A_inner, const spmv_prepar
                                double* resid, int32_t use_graph, spmv_stream_t stream)
 {
     clear_error();
-    return cg_run(A_inner, A_exact, b, x, iters, refine_every, resid, use_graph, MeetWait{}, false, stream);
+    return cg_run(A_inner, A_exact, b, x, iters, refine_every, resid, use_graph, 0, false, stream);
 }
 
 extern "C" spmv_status spmv_cg_wait_check(const spmv_prepared_t* A_inner, const spmv_prepared_t* A_exact,
                                           const double* b, double* x, int32_t iters, int32_t refine_every,
-                                          double* resid, int64_t limit_ns, int32_t arrive, spmv_stream_t stream)
+                                          double* resid, int32_t arrive, spmv_stream_t stream)
 {
     clear_error();
-    if (limit_ns <= 0 || limit_ns > 2000000000ll)
-        return fail(SPMV_ERR_INVALID_ARG, "spmv_cg_wait_check: limit_ns must be in 1..2e9");
-    return cg_run(A_inner, A_exact, b, x, iters, refine_every, resid, 0, MeetWait{arrive ? 0u : 1u, (uint64_t)limit_ns},
-                  true, stream);
+    return cg_run(A_inner, A_exact, b, x, iters, refine_every, resid, 0, arrive ? 0 : 1, true, stream);
 }

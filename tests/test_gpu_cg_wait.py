@@ -1,6 +1,6 @@
-"""The one-launch CG loop's waits run out (a block that does not exist, a limit
-of a millisecond): x and the residuals after the first are NaN, and the next
-solve on the same objects is right.  Which solves run as one launch.  And the
+"""The one-launch CG loop's waits run out (one arrival short, two seconds): x and
+the residuals after the first are NaN, and the next solve on the same objects is
+right.  Which solves run as one launch.  And the
 smallest system, one row, solved exactly by its first iteration."""
 import numpy as np
 import pytest
@@ -11,7 +11,6 @@ import paper_1511_02494_gb300 as sp
 import synth
 
 pytestmark = pytest.mark.gpu
-LIMIT, LONG = 1_000_000, 2_000_000_000
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -30,16 +29,15 @@ def _vectors(n, iters):
     return synth.uniform_vector(n, 3, device="cuda"), x, torch.full((iters + 1,), -1.0, dtype=torch.float64, device="cuda")
 
 
-@pytest.mark.parametrize("refine", [0, 3])
-@pytest.mark.parametrize("kw", [{}, dict(index_bytes=2), dict(value_type=sp.VAL_F32), dict(value_type=sp.VAL_BF16),
-                                dict(value_type=sp.VAL_BF16, accumulate=sp.ACC_F64)])
-@pytest.mark.parametrize("side", [5, 33, 64])
+@pytest.mark.parametrize("side,kw,refine", [
+    (5, {}, 0), (33, {}, 3), (64, {}, 0), (33, dict(index_bytes=2), 0), (33, dict(value_type=sp.VAL_F32), 0),
+    (64, dict(value_type=sp.VAL_BF16), 3), (5, dict(value_type=sp.VAL_BF16, accumulate=sp.ACC_F64), 3)])
 def test_a_wait_that_gives_up(side, kw, refine):
     A = synth.laplacian_3d_7pt(side)
     P, E = _prepare(A, **kw), _prepare(A)
     iters = 8
     b, x, r = _vectors(A.n_rows, iters)
-    sp.spmv_cg_wait_check(P, b, x, iters, LIMIT, False, refine, E, r)
+    sp.spmv_cg_wait_check(P, b, x, iters, False, refine, E, r)
     assert torch.isnan(x).all() and torch.isnan(r[1:]).all()
     start = float(r[0])
     assert abs(start - float(torch.linalg.vector_norm(b))) <= 1e-12 * start
@@ -47,20 +45,12 @@ def test_a_wait_that_gives_up(side, kw, refine):
     for check in (True, False):
         b, x, r = _vectors(A.n_rows, iters)
         if check:
-            sp.spmv_cg_wait_check(P, b, x, iters, LONG, True, refine, E, r)
+            sp.spmv_cg_wait_check(P, b, x, iters, True, refine, E, r)
         else:
             sp.spmv_cg(P, b, x, iters, refine, A_exact=E, resid=r)
         solved.append((x.cpu(), r.cpu()))
         assert float(r[0]) == start and float(r[-1]) < 0.9 * start
     assert torch.equal(solved[0][0], solved[1][0]) and torch.equal(solved[0][1], solved[1][1])
-
-
-@pytest.mark.parametrize("limit", [0, -1, 2_000_000_001])
-def test_limits_out_of_range(limit):
-    P = _prepare(synth.laplacian_3d_7pt(5))
-    b, x, _ = _vectors(125, 1)
-    with pytest.raises(sp.SpmvError, match="limit_ns"):
-        sp.spmv_cg_wait_check(P, b, x, 1, limit, True)
 
 
 def test_one_row_is_solved_by_the_first_iteration():
@@ -71,7 +61,7 @@ def test_one_row_is_solved_by_the_first_iteration():
     for iters in (1, 3):
         x = torch.zeros(1, dtype=torch.float64, device="cuda")
         r = torch.full((iters + 1,), -1.0, dtype=torch.float64, device="cuda")
-        sp.spmv_cg_wait_check(P, b.cuda(), x, iters, LONG, True, resid=r)
+        sp.spmv_cg_wait_check(P, b.cuda(), x, iters, True, resid=r)
         xo, ro = oracle.cg(A, b, np.zeros(1), iters)
         assert np.array_equal(r.cpu().numpy(), ro, equal_nan=True)
         assert np.array_equal(x.cpu().numpy(), xo, equal_nan=True)
@@ -103,7 +93,7 @@ def test_solves_that_do_not_run_as_one_launch(form):
     P, E, iters, refine = OTHER_FORMS[form]()
     b, x, _ = _vectors(P.A.n_rows, iters)
     with pytest.raises(sp.SpmvError, match="does not run as one launch"):
-        sp.spmv_cg_wait_check(P, b, x, iters, LIMIT, False, refine, E)
+        sp.spmv_cg_wait_check(P, b, x, iters, False, refine, E)
     assert not x.any()
 
 
@@ -130,10 +120,10 @@ def test_one_launch_by_the_products_bytes_and_the_l2(kw, bytes_a_slot, head, vec
         P, E = sp.spmv_prepare(A, sp.make_choice("sliced", block_nnz=1, **kw)), sp.spmv_prepare(A, sp.make_choice("sliced"))
         b, x, r = _vectors(n, 6)
         if one:
-            sp.spmv_cg_wait_check(P, b, x, 6, LONG, True, 3, E, r)
+            sp.spmv_cg_wait_check(P, b, x, 6, True, 3, E, r)
         else:
             with pytest.raises(sp.SpmvError, match="does not run as one launch"):
-                sp.spmv_cg_wait_check(P, b, x, 6, LONG, True, 3, E, r)
+                sp.spmv_cg_wait_check(P, b, x, 6, True, 3, E, r)
         x.zero_()
         sp.spmv_cg(P, b, x, 6, 3, A_exact=E, resid=r)
         y = torch.empty_like(b)
